@@ -163,7 +163,9 @@ void ori_default_plan_opts(ori_plan_opts* o);
  *   n        cells per axis, 2 <= n <= 1024.  The padded FFT length per axis
  *            is L = the smallest power of two >= 2n (the paper pads to 2b-2
  *            by mirroring, Section 3; any L >= 2n-1 gives the same crop), at
- *            most 2048.  L <= 1024 runs the register-tile and persistent
+ *            most 2048.  Without opts->min_L the transforms run at M = the
+ *            smallest of L, 144, 200, 288, 400, 576 and 800 that is >= 2n and
+ *            in (L/2, L]: the same operator with less padding.  L <= 1024 runs the register-tile and persistent
  *            pipelined FFT passes; at L = 2048 the FP32 passes stay pipelined
  *            (the TILES schedules of the Y and Z passes select shared-memory
  *            radix-8 kernels) and the FP64 and paired-FP32 passes run
@@ -191,16 +193,17 @@ ori_status ori_plan(int64_t n, double k, const ori_domain* dom,
  * on h, N or the origin.
  *
  * ori_plan_spectrum_bytes - *bytes = size of the saved form: a 576-byte header
- *   (format tag, n, L, wave numbers, c_S, side) and n_k (L/2+1)^3 complex128
- *   spectrum entries.
+ *   (format tag, n, M, wave numbers, c_S, side) and n_k (M/2+1)^3 complex128
+ *   spectrum entries, M the plan's transform length (ori_plan).
  * ori_plan_save_spectrum - write the saved form into host_buf (bytes >= the
  *   size above; pageable or pinned host memory).  A lean plan writes its
  *   paired-FP32 spectrum widened to complex128 (about 48 significant bits).
  *   Synchronises `stream`.
  * ori_plan_from_spectrum - as ori_plan, but the spectra come from a saved form
- *   instead of being computed: n, L (with opts->min_L), c_S (opts->c_S) and
- *   side (dom->side) must equal the saved ones, and the wave numbers are the
- *   saved ones (k, opts->n_k and opts->ks are ignored).  A mismatch, or a
+ *   instead of being computed: n, c_S (opts->c_S) and side (dom->side) must
+ *   equal the saved ones, the saved length must be this plan's M or its L
+ *   (with opts->min_L; the plan then transforms at the saved length), and the
+ *   wave numbers are the saved ones (k, opts->n_k and opts->ks are ignored).  A mismatch, or a
  *   buffer that is too short or not a saved spectrum, returns
  *   ORI_ERR_INVALID_ARG.  Synchronises `stream`.
  */
@@ -219,7 +222,7 @@ ori_status ori_plan_set_medium(ori_plan_t plan, const double* h_dev,
 /* Free the plan and its device memory (synchronises the device first). */
 ori_status ori_plan_destroy(ori_plan_t plan);
 
-/* Grid size, padded length, and bytes of device memory the plan holds. */
+/* Grid size, padded length L (ori_plan), and bytes of device memory the plan holds. */
 ori_status ori_plan_info(ori_plan_t plan, int64_t* n, int64_t* L, size_t* bytes);
 
 /*
@@ -373,7 +376,10 @@ typedef struct {
                            of 16 columns with the transform split L = L1 * L2,
                            L1 = 2^ceil(log2(L) / 2); 1: tiles of 8 columns;
                            2: 16 columns, split (2 L1) * (L2 / 2).  Other lengths
-                           have variant 0 only                                     */
+                           have variant 0 only.  A plan whose transform length M
+                           is not a power of two runs one persistent kernel per
+                           pass whatever these fields say (zconv_variant 1: its
+                           rows by cp.async instead of TMA)                        */
   int zconv_variant;
   int yinv_variant;
 } ori_schedule;

@@ -243,9 +243,113 @@ __device__ __forceinline__ void dft_radix2(cpx<T> (&a)[R]) {
   for (int i = 0; i < R; ++i) a[i] = t[i];
 }
 
+// ---------------------------------------------------------------------------
+// Sizes with a factor 3 or 5 (R = P Q, P a power of two, Q = 3 or 5): the
+// in-register transforms of the padded lengths between powers of two.
+// ---------------------------------------------------------------------------
+constexpr bool is_pow2(int v) { return (v & (v - 1)) == 0; }
+constexpr int pow2_part(int v) { return (v & 1) ? 1 : 2 * pow2_part(v / 2); }
+
+// cos/sin of 2 pi j / R as a compile-time constant of type T (paired FP32
+// specialises it in dfloat.cuh).
+template <int R, class T>
+struct TwR {
+  static constexpr T c(int j) { return T(turn_cos_sin(8LL * j, 8LL * R).c); }
+  static constexpr T s(int j) { return T(turn_cos_sin(8LL * j, 8LL * R).s); }
+};
+
+// a + s t and m + SIGN i n (a quarter turn folded into the sums).
+template <class T>
+__device__ __forceinline__ cpx<T> axpy_r(T s, cpx<T> t, cpx<T> a) { return {a.x + s * t.x, a.y + s * t.y}; }
+template <int SIGN, class T>
+__device__ __forceinline__ cpx<T> add_i(cpx<T> m, cpx<T> n) {
+  return SIGN > 0 ? cpx<T>{m.x - n.y, m.y + n.x} : cpx<T>{m.x + n.y, m.y - n.x};
+}
+
+template <int SIGN, class T>
+__device__ __forceinline__ void dft3(cpx<T>& a, cpx<T>& b, cpx<T>& c) {
+  constexpr T half = TwR<3, T>::c(1), sn = TwR<3, T>::s(1);   // cos = -1/2
+  const cpx<T> t = b + c, d = b - c;
+  const cpx<T> m = axpy_r(half, t, a), n = {sn * d.x, sn * d.y};
+  a = a + t;
+  b = add_i<SIGN>(m, n);
+  c = add_i<-SIGN>(m, n);
+}
+
+template <int SIGN, class T>
+__device__ __forceinline__ void dft5(cpx<T>& a, cpx<T>& b, cpx<T>& c, cpx<T>& d, cpx<T>& e) {
+  constexpr T c1 = TwR<5, T>::c(1), c2 = TwR<5, T>::c(2), s1 = TwR<5, T>::s(1), s2 = TwR<5, T>::s(2);
+  const cpx<T> t1 = b + e, t2 = c + d, t3 = b - e, t4 = c - d;
+  const cpx<T> m1 = axpy_r(c2, t2, axpy_r(c1, t1, a)), m2 = axpy_r(c1, t2, axpy_r(c2, t1, a));
+  const cpx<T> n1 = axpy_r(s2, t4, cpx<T>{s1 * t3.x, s1 * t3.y});
+  const cpx<T> n2 = axpy_r(-s1, t4, cpx<T>{s2 * t3.x, s2 * t3.y});
+  a = a + (t1 + t2);
+  b = add_i<SIGN>(m1, n1);
+  e = add_i<-SIGN>(m1, n1);
+  c = add_i<SIGN>(m2, n2);
+  d = add_i<-SIGN>(m2, n2);
+}
+
+template <int R, int SIGN, bool HALF, class T>
+__device__ __forceinline__ void dft(cpx<T> (&a)[R]);
+
+// z * exp(SIGN 2 pi i j / R), j and R compile-time constants.
+template <int R, int SIGN, class T>
+__device__ __forceinline__ cpx<T> twR_mul(cpx<T> z, int j) {
+  if (j == 0) return z;
+  const T c = TwR<R, T>::c(j), s = TwR<R, T>::s(j);
+  return cmul(z, cpx<T>{c, SIGN > 0 ? s : -s});
+}
+
+// Prime-factor form (Good 1958): with n = Q n1 + P n2 (mod R) and k read mod P
+// and mod Q, w_R^(nk) = w_P^(n1 k) w_Q^(n2 k): P-point and Q-point transforms
+// with no twiddles between them.
+template <int R, int SIGN, class T>
+__device__ __forceinline__ void dft_pfa(cpx<T> (&a)[R]) {
+  constexpr int P = pow2_part(R), Q = R / P;
+  static_assert(Q == 3 || Q == 5, "one odd factor, 3 or 5");
+  cpx<T> t[Q][P];
+#pragma unroll
+  for (int n2 = 0; n2 < Q; ++n2) {
+#pragma unroll
+    for (int n1 = 0; n1 < P; ++n1) t[n2][n1] = a[(Q * n1 + P * n2) % R];
+    if constexpr (P > 1) dft<P, SIGN, false>(t[n2]);
+  }
+#pragma unroll
+  for (int k = 0; k < P; ++k) {
+    if constexpr (Q == 3) dft3<SIGN>(t[0][k], t[1][k], t[2][k]);
+    else dft5<SIGN>(t[0][k], t[1][k], t[2][k], t[3][k], t[4][k]);
+  }
+#pragma unroll
+  for (int k = 0; k < R; ++k) a[k] = t[k % Q][k % P];
+}
+
+// HALF for a composite R: the even outputs are the R/2-point transform of the
+// nonzero half, the odd ones that of the half times w^j.
+template <int R, int SIGN, class T>
+__device__ __forceinline__ void dft_half_in(cpx<T> (&a)[R]) {
+  constexpr int M = R / 2;
+  cpx<T> e[M], o[M];
+#pragma unroll
+  for (int j = 0; j < M; ++j) {
+    e[j] = a[j];
+    o[j] = twR_mul<R, SIGN>(a[j], j);
+  }
+  dft_pfa<M, SIGN>(e);
+  dft_pfa<M, SIGN>(o);
+#pragma unroll
+  for (int k = 0; k < M; ++k) {
+    a[2 * k] = e[k];
+    a[2 * k + 1] = o[k];
+  }
+}
+
 template <int R, int SIGN, bool HALF, class T>
 __device__ __forceinline__ void dft(cpx<T> (&a)[R]) {
-  if constexpr (R > 1 && R <= 8) {
+  if constexpr (!is_pow2(R)) {
+    if constexpr (HALF) dft_half_in<R, SIGN>(a);
+    else dft_pfa<R, SIGN>(a);
+  } else if constexpr (R > 1 && R <= 8) {
     dft_radix2<R, SIGN, HALF>(a);
   } else if constexpr (R > 1) {
     bool first = true;
@@ -300,13 +404,55 @@ __device__ __forceinline__ void dft(cpx<T> (&a)[R]) {
   }
 }
 
+// The same transform when only the outputs k < R/2 are used (the rows an
+// inverse pass keeps).  A composite R combines two R/2-point transforms for
+// those outputs alone; a power of two leaves the pruning to the compiler.
+template <int R, int SIGN, class T>
+__device__ __forceinline__ void dft_low(cpx<T> (&a)[R]) {
+  if constexpr (is_pow2(R)) {
+    dft<R, SIGN, false>(a);
+  } else {
+    constexpr int M = R / 2;
+    cpx<T> e[M], o[M];
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+      e[j] = a[2 * j];
+      o[j] = a[2 * j + 1];
+    }
+    dft_pfa<M, SIGN>(e);
+    dft_pfa<M, SIGN>(o);
+#pragma unroll
+    for (int j = 0; j < M; ++j) a[j] = e[j] + twR_mul<R, SIGN>(o[j], j);
+  }
+}
+
+// Transform lengths with a factor 9 or 25, for grids whose power of two would
+// be mostly padding (transform_length).  Every one is 8 r2 r3 (the stages of
+// the shared-memory transforms, MixRad) and L1 L2 with L1 a multiple of an
+// even L2 (the two register stages, Split).
+constexpr bool is_mixed_len(int L) { return !is_pow2(L); }
+template <int L> struct MixRad;
+template <> struct MixRad<144> { static constexpr int r2 = 6, r3 = 3, L1 = 12; };
+template <> struct MixRad<200> { static constexpr int r2 = 5, r3 = 5, L1 = 20; };
+template <> struct MixRad<288> { static constexpr int r2 = 6, r3 = 6, L1 = 24; };
+template <> struct MixRad<400> { static constexpr int r2 = 10, r3 = 5, L1 = 20; };
+template <> struct MixRad<576> { static constexpr int r2 = 6, r3 = 12, L1 = 24; };
+template <> struct MixRad<800> { static constexpr int r2 = 10, r3 = 10, L1 = 40; };
+
 // Split of the padded length L = L1 * L2 into two in-register stages.
 constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v >> 1); }
-template <int L>
+template <int L, bool MIXED = is_mixed_len(L)>
 struct Split {
   static constexpr int lg = ilog2(L);
   static constexpr int L1 = 1 << ((lg + 1) / 2);
   static constexpr int L2 = L / L1;
+};
+
+template <int L>
+struct Split<L, true> {
+  static constexpr int L1 = MixRad<L>::L1;
+  static constexpr int L2 = L / L1;
+  static_assert(L1 % L2 == 0 && L2 % 2 == 0 && L % 8 == 0, "mixed transform length");
 };
 
 }  // namespace ori

@@ -9,6 +9,8 @@
 //   forward: decimation in frequency, natural order in, digit-reversed out
 //   inverse: decimation in time, digit-reversed in, natural order out
 //
+// The mixed lengths (MixRad) run three stages of radices 8, r2 and r3.
+//
 // so a forward transform, a pointwise product (indexed through the digit
 // reversal) and an inverse need no reordering pass.  The X inverse pass,
 // whose input comes in natural order from global memory, runs the DIF
@@ -33,6 +35,11 @@ struct DRad {
 // significant digit of the frequency).
 template <int L>
 __device__ __forceinline__ int digit_rev(int p) {
+  if constexpr (is_mixed_len(L)) {   // p = (t1 r2 + t2) r3 + t3 holds k = t1 + 8 (t2 + r2 t3)
+    constexpr int r2 = MixRad<L>::r2, r3 = MixRad<L>::r3;
+    const int q = p / r3;
+    return q / r2 + 8 * (q % r2 + r2 * (p - q * r3));
+  } else {
   using DR = DRad<L>;
   int k = 0, w = 1;
   // digits of p, least significant first, belong to the stages last-to-first
@@ -50,11 +57,17 @@ __device__ __forceinline__ int digit_rev(int p) {
     w *= R;
   }
   return k;
+  }
 }
 
 // Position that holds frequency k after the forward stages (inverse of digit_rev).
 template <int L>
 __device__ __forceinline__ int inv_digit_rev(int k) {
+  if constexpr (is_mixed_len(L)) {
+    constexpr int r2 = MixRad<L>::r2, r3 = MixRad<L>::r3;
+    const int q = k / 8, t3 = q / r2;
+    return ((k & 7) * r2 + (q - t3 * r2)) * r3 + t3;
+  } else {
   using DR = DRad<L>;
   // k = d_1 + 8 d_2 + ... (first stage's digit least significant), last digit radix RL
   int q = k;
@@ -67,6 +80,7 @@ __device__ __forceinline__ int inv_digit_rev(int k) {
 #pragma unroll
   for (int i = DR::NST8 - 1; i >= 0; --i) { p += dig[i] * w; w *= 8; }
   return p;
+  }
 }
 
 // Shared-memory index of point j of column c: rows of C columns, the column
@@ -90,7 +104,7 @@ __device__ __forceinline__ void dif_stage(cpx<T>* X, int M, const cpx<T>* tw, in
     for (int t = 0; t < R; ++t) v[t] = ld_stage(X + sidx<C>(base + t * s, c));
     dft<R, SIGN, false>(v);
 #pragma unroll
-    for (int t = 1; t < R; ++t) v[t] = twL_mul<SIGN>(v[t], tw, (j * t * step) & (L - 1));
+    for (int t = 1; t < R; ++t) v[t] = twL_mul<SIGN>(v[t], tw, j * t * step);   // j t < M
 #pragma unroll
     for (int t = 0; t < R; ++t) st_stage(X + sidx<C>(base + t * s, c), settle(v[t]));
   }
@@ -110,7 +124,7 @@ __device__ __forceinline__ void dit_stage(cpx<T>* X, int M, const cpx<T>* tw, in
 #pragma unroll
     for (int t = 0; t < R; ++t) v[t] = ld_stage(X + sidx<C>(base + t * s, c));
 #pragma unroll
-    for (int t = 1; t < R; ++t) v[t] = twL_mul<SIGN>(v[t], tw, (j * t * step) & (L - 1));
+    for (int t = 1; t < R; ++t) v[t] = twL_mul<SIGN>(v[t], tw, j * t * step);   // j t < M
     dft<R, SIGN, false>(v);
 #pragma unroll
     for (int t = 0; t < R; ++t) st_stage(X + sidx<C>(base + t * s, c), settle(v[t]));
@@ -121,6 +135,12 @@ __device__ __forceinline__ void dit_stage(cpx<T>* X, int M, const cpx<T>* tw, in
 // block sizes L/8, L/64, ...  SIGN -1: forward transform; +1: inverse.
 template <int L, int C, int SIGN = -1, class T>
 __device__ __forceinline__ void dif_rest(cpx<T>* X, const cpx<T>* tw, int tid, int nt) {
+  if constexpr (is_mixed_len(L)) {
+    dif_stage<MixRad<L>::r2, SIGN, L, C>(X, L / 8, tw, tid, nt);
+    __syncthreads();
+    dif_stage<MixRad<L>::r3, SIGN, L, C>(X, MixRad<L>::r3, tw, tid, nt);
+    __syncthreads();
+  } else {
   using DR = DRad<L>;
   int M = L / 8;
 #pragma unroll 1
@@ -133,12 +153,19 @@ __device__ __forceinline__ void dif_rest(cpx<T>* X, const cpx<T>* tw, int tid, i
     dif_stage<DR::RL, SIGN, L, C>(X, M, tw, tid, nt);
     __syncthreads();
   }
+  }
 }
 
 // Inverse DIT stages except the last (block size L), which the callers fuse
 // with their stores: block sizes RL (if any), then 8 RL, 64 RL, ... up to L/8.
 template <int L, int C, class T>
 __device__ __forceinline__ void dit_head(cpx<T>* X, const cpx<T>* tw, int tid, int nt) {
+  if constexpr (is_mixed_len(L)) {
+    dit_stage<MixRad<L>::r3, +1, L, C>(X, MixRad<L>::r3, tw, tid, nt);
+    __syncthreads();
+    dit_stage<MixRad<L>::r2, +1, L, C>(X, L / 8, tw, tid, nt);
+    __syncthreads();
+  } else {
   using DR = DRad<L>;
   int M = 1;
   if constexpr (DR::RL > 1) {
@@ -151,6 +178,7 @@ __device__ __forceinline__ void dit_head(cpx<T>* X, const cpx<T>* tw, int tid, i
     M *= 8;
     dit_stage<8, +1, L, C>(X, M, tw, tid, nt);
     __syncthreads();
+  }
   }
 }
 

@@ -66,7 +66,8 @@ void set_last_error(const std::string& msg) { g_last_error = msg; }
 // ---------------------------------------------------------------------------
 struct ori_plan_s {
   int device = 0;
-  int n = 0, L = 0, H = 0;
+  int n = 0, L = 0;                // L: padded length (ori_plan_info)
+  int M = 0, H = 0;                // transform length of the passes (transform_length, M <= L), H = M/2 + 1
   long long n3 = 0;
   double d = 0, c_S = 0, side = 0, origin[3] = {0, 0, 0};
   std::vector<double> ks;          // wave numbers; one spectrum each
@@ -270,8 +271,8 @@ static void drop_graphs(ori_plan_s* p) {
   p->graph_f_len = p->graph_d_len = 0;
 }
 
-static size_t t1_elems(const ori_plan_s* p) { return size_t(p->n) * p->n * p->L; }
-static size_t t2_elems(const ori_plan_s* p) { return size_t(p->n) * p->L * p->L; }
+static size_t t1_elems(const ori_plan_s* p) { return size_t(p->n) * p->n * p->M; }
+static size_t t2_elems(const ori_plan_s* p) { return size_t(p->n) * p->M * p->M; }
 
 // Release the batch-sized buffers.
 static void free_capacity(ori_plan_s* p) {
@@ -366,10 +367,10 @@ static void plan_free(ori_plan_s* p) {
 }
 
 // Host twiddle table tab[m] = (cos, sin)(2 pi m / L), from the compile-time
-// evaluable series in common.cuh on a fine circle (2^20 points).
+// evaluable series in common.cuh on a fine circle (2^20 points; 8 L at the mixed lengths).
 template <class T>
 static void host_twiddles(int L, cpx<T>* out) {
-  const long long M = 1LL << 20;
+  const long long M = is_mixed_len(L) ? 8LL * L : 1LL << 20;
   for (int m = 0; m < L; ++m) {
     CosSin v = turn_cos_sin((long long)m * (M / L), M);
     out[m] = cpx<T>{T(v.c), T(v.s)};
@@ -419,9 +420,11 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 }
 
 // Whether the FP32 Z pass stages its tiles by bulk copies: the pipelined
-// kernel with 16-column tiles (ZPipe::TMA), given a valid tensor map.
+// kernel with 16-column tiles (ZPipe::TMA), or k_zconv_mix unless launch
+// variant 1 asks for cp.async staging, given a valid tensor map.
 static bool z_bulk_staged(const ori_plan_s* p) {
-  const int L = p->L;
+  const int L = p->M;
+  if (is_mixed_len(L)) return p->zmap_ok && p->var_z != 1;
   if (!p->zmap_ok || L < 64 || L > 1024 || p->sched_z == SCHED_TILES) return false;
   return !(has_pipe_variants(L) && p->var_z == 1);
 }
@@ -438,7 +441,7 @@ static void z_tensor_map(ori_plan_s* p, SArgs& z, int nrhs) {
     p->zmap_ok = 0;
     p->zmap_ptr = p->T2f;
     p->zmap_R = R;
-    const int L = p->L;
+    const int L = p->M;
     const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (enc != nullptr && L >= 64 && L <= 1024 && (reinterpret_cast<uintptr_t>(p->T2f) & 15u) == 0) {
       const cuuint64_t es = sizeof(cpx<float>);
@@ -446,39 +449,41 @@ static void z_tensor_map(ori_plan_s* p, SArgs& z, int nrhs) {
       const cuuint64_t strides[3] = {cuuint64_t(L) * es, cuuint64_t(L) * L * es, cuuint64_t(t2_elems(p)) * es};
       const int zbox = std::min(L / 2, 256);
       const cuuint32_t box[4] = {cuuint32_t(kZGroup), 1, cuuint32_t(zbox), 1};
+      const cuuint32_t mbox[4] = {cuuint32_t(zgroup(L)), 1, cuuint32_t(even_box(L / 2)), 1};   // mixed lengths
       const cuuint32_t estr[4] = {1, 1, 1, 1};
-      if (enc(&p->zmap, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, p->T2f, dims, strides, box, estr,
+      if (enc(&p->zmap, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, p->T2f, dims, strides,
+              is_mixed_len(L) ? mbox : box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS) {
         p->zmap_ok = 1;
-        p->zbox = zbox;
+        p->zbox = is_mixed_len(L) ? even_box(L / 2) : zbox;
       }
     }
   }
   z.zrows = p->zmap;
-  z.zrows_ok = p->zmap_ok;
+  z.zrows_ok = p->zmap_ok && !(is_mixed_len(p->M) && p->var_z == 1);
   z.zbox = p->zbox;
   z.err = p->d_fault;
 }
 
 // Tensor maps of the rows the pipelined FP32 Y passes stage per tile (16
 // FP32 columns = 128 bytes a row): the Y-forward input T1f, dims (kx, y, z,
-// right-hand side) and box (16, ybox_f, 1, 1), ybox_f = min(L/2, 256) (a
-// power of two dividing L/2: the zero-filled rows past n stay within the L/2
-// staged rows); the Y-inverse input T2f, dims (kx, ky, z, right-hand side)
-// and box (16, ybox_i, 1, 1), ybox_i = min(L, 256).
+// right-hand side) and box (16, ybox_f, 1, 1), ybox_f = even_box(L/2) (it
+// divides L/2: the zero-filled rows past n stay within the L/2 staged rows);
+// the Y-inverse input T2f, dims (kx, ky, z, right-hand side) and box
+// (16, ybox_i, 1, 1), ybox_i = even_box(L).
 static void y_tensor_maps(ori_plan_s* p, SArgs& y, SArgs& yi, int nrhs) {
   const int R = std::max(1, nrhs);
   if (p->ymap_ptr != p->T1f || p->ymap_R != R) {
     p->ymap_ok = 0;
     p->ymap_ptr = p->T1f;
     p->ymap_R = R;
-    const int L = p->L, n = p->n;
+    const int L = p->M, n = p->n;
     const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (enc != nullptr && L >= 64 && L <= 1024 && ((reinterpret_cast<uintptr_t>(p->T1f) |
                                                     reinterpret_cast<uintptr_t>(p->T2f)) & 15u) == 0) {
       const cuuint64_t es = sizeof(cpx<float>);
-      const int bf = std::min(L / 2, 256), bi = std::min(L, 256);
+      const int bf = even_box(L / 2), bi = even_box(L);
       const cuuint32_t estr[4] = {1, 1, 1, 1};
       const cuuint64_t dims_f[4] = {cuuint64_t(L), cuuint64_t(n), cuuint64_t(n), cuuint64_t(R)};
       const cuuint64_t str_f[3] = {cuuint64_t(L) * es, cuuint64_t(n) * L * es, cuuint64_t(t1_elems(p)) * es};
@@ -518,7 +523,7 @@ static ori_status run_conv(ori_plan_s* p, XArgs pro, XArgs epi, int fin, cudaStr
   cpx<T>* T2 = reinterpret_cast<cpx<T>*>(f32 ? (void*)p->T2f : (void*)p->T2d);
   const void* tw = K == 0 ? (const void*)p->tw32 : (K == ORI_PASS_FP64 ? (const void*)p->tw64 : (const void*)p->twdf);
   const void* gh = K == 0 ? (const void*)p->ghat32 : (K == ORI_PASS_FP64 ? (const void*)p->ghat64 : (const void*)p->ghatdf);
-  const int n = p->n, L = p->L;
+  const int n = p->n, L = p->M;
   const long long H3 = (long long)p->H * p->H * p->H;
   const long long bsT1 = (long long)t1_elems(p) * sizeof(cpx<T>);
   const long long bsT2 = (long long)t2_elems(p) * sizeof(cpx<T>);
@@ -552,7 +557,7 @@ static ori_status run_conv(ori_plan_s* p, XArgs pro, XArgs epi, int fin, cudaStr
   z.done = mask.flags; z.done_stride = mask.stride; z.sm_count = p->sm_count;
   z.nrhs = nrhs; z.bs_in = bsT2; z.bs_out = bsT2;
   z.bs_ghat = H3 * (long long)sizeof(cpx<T>);
-  z.bs_ghatZ = (long long)p->H * p->H * p->L * (long long)sizeof(cpx<float>);
+  z.bs_ghatZ = (long long)p->H * p->H * p->M * (long long)sizeof(cpx<float>);
   z.rhs_per_ghat = rhs_per_k;
   z.sched = p->sched_z; z.cta_cap = p->cta_cap; z.variant = p->var_z;
   if (f32) z_tensor_map(p, z, nrhs);
@@ -682,7 +687,7 @@ static ori_status set_medium(ori_plan_s* p, const double* h_dev, const double* N
 // copy.  Transient memory: the H^3 octant and a batch of L^2 planes.
 static ori_status build_spectrum(ori_plan_s* p) {
   NvtxRange nvtx("ori plan spectrum");
-  const int L = p->L, n = p->n, H = p->H;
+  const int L = p->M, n = p->n, H = p->H;
   const long long L3 = (long long)L * L * L;
   const long long H3 = (long long)H * H * H;
   const long long HZ = (long long)H * H * L;
@@ -744,7 +749,7 @@ static ori_status build_spectrum(ori_plan_s* p) {
                                                    p->ghatdf + ik * H3, H, H, scale);
     if (!check(cudaGetLastError(), "plan extract")) break;
     if (p->ghatZ32) {
-      k_build_ghatZ<<<p->vec_grid, 256, 0, p->ps>>>(p->ghat32 + ik * H3, p->ghatZ32 + ik * HZ, L, H);
+      k_build_ghatZ<<<p->vec_grid, 256, 0, p->ps>>>(p->ghat32 + ik * H3, p->ghatZ32 + ik * HZ, L, H, zgroup(L));
       if (!check(cudaGetLastError(), "plan Z spectrum")) break;
     }
     check(cudaStreamSynchronize(p->ps), "plan spectrum");
@@ -762,7 +767,7 @@ struct SpecHeader {
   int32_t version;      // 1
   int32_t n, L, n_k;
   double c_S, side;
-  uint64_t entries;     // n_k (L/2+1)^3
+  uint64_t entries;     // n_k (L/2+1)^3, L the transform length of the saving plan
   double ks[64];
 };
 static constexpr size_t kSpecPayload = 576;
@@ -777,7 +782,7 @@ static size_t spectrum_bytes(const ori_plan_s* p) {
 static ori_status load_spectrum(ori_plan_s* p, const unsigned char* buf) {
   NvtxRange nvtx("ori plan spectrum (saved)");
   const long long H3 = (long long)p->H * p->H * p->H;
-  const long long HZ = (long long)p->H * p->H * p->L;
+  const long long HZ = (long long)p->H * p->H * p->M;
   const cpx<double>* src = reinterpret_cast<const cpx<double>*>(buf + kSpecPayload);
   // a lean plan has no FP64 spectrum: the entries go through a bounded staging buffer
   const long long chunk = p->ghat64 ? H3 : std::min<long long>(H3, 1LL << 26);
@@ -804,7 +809,7 @@ static ori_status load_spectrum(ori_plan_s* p, const unsigned char* buf) {
       if (e != cudaSuccess) st = fail(ORI_ERR_CUDA, std::string("spectrum load: ") + cudaGetErrorString(e));
     }
     if (st == ORI_OK && p->ghatZ32) {
-      k_build_ghatZ<<<p->vec_grid, 256, 0, p->ps>>>(p->ghat32 + ik * H3, p->ghatZ32 + ik * HZ, p->L, p->H);
+      k_build_ghatZ<<<p->vec_grid, 256, 0, p->ps>>>(p->ghat32 + ik * H3, p->ghatZ32 + ik * HZ, p->M, p->H, zgroup(p->M));
       cudaError_t e = cudaGetLastError();
       if (e == cudaSuccess) e = cudaStreamSynchronize(p->ps);
       if (e != cudaSuccess) st = fail(ORI_ERR_CUDA, std::string("spectrum load: ") + cudaGetErrorString(e));
@@ -881,6 +886,7 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
   if (o.min_L != 0 && (o.min_L < 4 || o.min_L > 2048 || (o.min_L & (o.min_L - 1)) != 0))
     return fail(ORI_ERR_INVALID_ARG, "min_L must be 0 or a power of two in [4, 2048]");
   std::vector<double> ks;
+  int spec_M = 0;   // transform length of the saved spectrum
   if (spec) {
     SpecHeader hd;
     if (spec_bytes < kSpecPayload) return fail(ORI_ERR_INVALID_ARG, "saved spectrum: buffer shorter than its header");
@@ -889,12 +895,16 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
       return fail(ORI_ERR_INVALID_ARG, "saved spectrum: not a saved spectrum of this format");
     int Lw = 4;
     while (Lw < 2 * n) Lw *= 2;
+    // saved at this plan's transform length, or at the power of two: the
+    // plan then runs at that length
+    const int Mw = o.min_L ? std::max(Lw, o.min_L) : transform_length(int(n), Lw);
     Lw = std::max(Lw, o.min_L);
-    const long long H = Lw / 2 + 1;
-    if (hd.n != n || hd.L != Lw)
+    if (hd.n != n || (hd.L != Lw && hd.L != Mw))
       return fail(ORI_ERR_INVALID_ARG, "saved spectrum: n or padded length L differs from this plan's");
     if (hd.c_S != o.c_S || hd.side != dom->side)
       return fail(ORI_ERR_INVALID_ARG, "saved spectrum: c_S or the cube side differs from this plan's");
+    const long long H = hd.L / 2 + 1;
+    spec_M = hd.L;
     if (hd.n_k < 1 || hd.n_k > 64 || hd.entries != uint64_t(hd.n_k) * uint64_t(H * H * H) ||
         spec_bytes < kSpecPayload + hd.entries * sizeof(cpx<double>))
       return fail(ORI_ERR_INVALID_ARG, "saved spectrum: truncated or inconsistent");
@@ -918,8 +928,9 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
     p->n = int(n);
     p->L = 4;
     while (p->L < 2 * p->n) p->L *= 2;
+    p->M = spec_M ? spec_M : (o.min_L ? std::max(p->L, o.min_L) : transform_length(p->n, p->L));
     p->L = std::max(p->L, o.min_L);
-    p->H = p->L / 2 + 1;
+    p->H = p->M / 2 + 1;
     p->n3 = (long long)n * n * n;
     p->ks = ks;
     p->side = dom->side;
@@ -945,9 +956,9 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
         (st = alloc_n(p, &p->S64, n3)) || (st = alloc_n(p, &p->S32, n3)) || (st = alloc_n(p, &p->Sdf, n3)) ||
         (st = alloc_n(p, &p->ghat32, nk * H3)) ||
         (st = alloc_n(p, &p->ghatdf, nk * H3)) ||
-        (st = alloc_n(p, &p->ghatZ32, nk * size_t(p->H) * p->H * p->L)) ||
-        (st = alloc_n(p, &p->tw64, size_t(p->L))) || (st = alloc_n(p, &p->tw32, size_t(p->L))) ||
-        (st = alloc_n(p, &p->twdf, size_t(p->L))) || (st = alloc_n(p, &p->d_count, 1)) ||
+        (st = alloc_n(p, &p->ghatZ32, nk * size_t(p->H) * p->H * p->M)) ||
+        (st = alloc_n(p, &p->tw64, size_t(p->M))) || (st = alloc_n(p, &p->tw32, size_t(p->M))) ||
+        (st = alloc_n(p, &p->twdf, size_t(p->M))) || (st = alloc_n(p, &p->d_count, 1)) ||
         (st = alloc_n(p, &p->d_fault, 1)))
       break;
     if (cudaMemset(p->d_fault, 0, sizeof(int)) != cudaSuccess || cudaMallocHost(&p->h_fault, sizeof(int)) != cudaSuccess ||
@@ -960,19 +971,19 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
     *p->h_fault = 0;
     *p->h_count = 0;
     unsigned bx32 = 0, bx64 = 0, bxdf = 0;
-    if ((st = setup_kernels<float>(p->L, &bx32, p->n, p->sm_count)) ||
-        (st = setup_kernels<double>(p->L, &bx64, p->n, p->sm_count)) ||
-        (st = setup_kernels<dfl>(p->L, &bxdf, p->n, p->sm_count)))
+    if ((st = setup_kernels<float>(p->M, &bx32, p->n, p->sm_count)) ||
+        (st = setup_kernels<double>(p->M, &bx64, p->n, p->sm_count)) ||
+        (st = setup_kernels<dfl>(p->M, &bxdf, p->n, p->sm_count)))
       break;
     p->xinv_blocks = std::max({bx32, bx64, bxdf});
     if ((st = enter(p, user))) break;
     {
-      cpx<double>* twd = new cpx<double>[p->L];
-      cpx<float>* twf = new cpx<float>[p->L];
-      cpx<dfl>* twdf = new cpx<dfl>[p->L];
-      host_twiddles<double>(p->L, twd);
-      host_twiddles<float>(p->L, twf);
-      for (int m = 0; m < p->L; ++m) {   // the stage layout of paired FP32: (re.hi, im.hi, re.lo, im.lo)
+      cpx<double>* twd = new cpx<double>[p->M];
+      cpx<float>* twf = new cpx<float>[p->M];
+      cpx<dfl>* twdf = new cpx<dfl>[p->M];
+      host_twiddles<double>(p->M, twd);
+      host_twiddles<float>(p->M, twf);
+      for (int m = 0; m < p->M; ++m) {   // the stage layout of paired FP32: (re.hi, im.hi, re.lo, im.lo)
         const dfl re = df_from_double_host(twd[m].x), im = df_from_double_host(twd[m].y);
         float* f = reinterpret_cast<float*>(twdf + m);
         f[0] = re.hi;
@@ -980,9 +991,9 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
         f[2] = re.lo;
         f[3] = im.lo;
       }
-      cudaError_t e1 = cudaMemcpy(p->tw64, twd, sizeof(cpx<double>) * p->L, cudaMemcpyHostToDevice);
-      cudaError_t e2 = cudaMemcpy(p->tw32, twf, sizeof(cpx<float>) * p->L, cudaMemcpyHostToDevice);
-      cudaError_t e3 = cudaMemcpy(p->twdf, twdf, sizeof(cpx<dfl>) * p->L, cudaMemcpyHostToDevice);
+      cudaError_t e1 = cudaMemcpy(p->tw64, twd, sizeof(cpx<double>) * p->M, cudaMemcpyHostToDevice);
+      cudaError_t e2 = cudaMemcpy(p->tw32, twf, sizeof(cpx<float>) * p->M, cudaMemcpyHostToDevice);
+      cudaError_t e3 = cudaMemcpy(p->twdf, twdf, sizeof(cpx<dfl>) * p->M, cudaMemcpyHostToDevice);
       delete[] twd;
       delete[] twf;
       delete[] twdf;
@@ -1034,7 +1045,7 @@ ori_status ori_plan_save_spectrum(ori_plan_t p, void* host_buf, size_t bytes, vo
   std::memcpy(hd.tag, kSpecTag, sizeof(kSpecTag));
   hd.version = 1;
   hd.n = p->n;
-  hd.L = p->L;
+  hd.L = p->M;
   hd.n_k = int32_t(p->ks.size());
   hd.c_S = p->c_S;
   hd.side = p->side;
@@ -1884,7 +1895,7 @@ static ori_status autotune(ori_plan_s* p, int nrhs, int reps, ori_schedule* best
   // FFT pass schedules (only the FP32 passes at L >= 64 have alternatives):
   // one field at a time, keeping the best value of each before the next
   ORI_TRY(time_fp32_operator(p, nrhs, reps, &best_t));
-  if (p->L >= 64 && p->L <= 1024) {   // longer transforms have one schedule
+  if (p->M >= 64 && p->M <= 1024 && !is_mixed_len(p->M)) {   // longer and mixed transforms have one schedule
     const int nv = pipe_variants(p->L);
     // fields: 0-2 kernel choice of Y fwd, Z, Y inv; 3-5 their launch variants
     // (persistent kernels only); 6 the persistent CTA cap

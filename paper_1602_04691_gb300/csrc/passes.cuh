@@ -29,6 +29,7 @@
 #include <cuda.h>   // CUtensorMap (the type only; maps are encoded through the runtime's driver entry point)
 
 #include <algorithm>
+#include <initializer_list>
 
 namespace ori {
 
@@ -140,6 +141,26 @@ enum { SCHED_PERSISTENT = 0, SCHED_TILES = 1 };
 
 // Columns per group of the Z-tile-ordered FP32 spectrum [my][kx / kZGroup][mz][kZGroup].
 constexpr int kZGroup = 16;
+// ... at transform length L: the mixed lengths (MixRad) group by the 8 columns of their Z tiles.
+constexpr int zgroup(int L) { return is_mixed_len(L) ? 8 : kZGroup; }
+
+// Transform length of a grid: the smallest instantiated length >= 2n.  Any
+// length >= 2n - 1 gives the same operator, and the work of a pass grows with
+// its square, so the lengths between the powers of two pay for themselves
+// even though a power of two is 10-20% faster per point: n = 260 runs at 576
+// instead of 1024.  Below 144 the passes are launch-bound and the power of two stays.
+constexpr int transform_length(int n, int pow2) {
+  for (int m : {144, 200, 288, 400, 576, 800})
+    if (m >= 2 * n && m > pow2 / 2 && m < pow2) return m;
+  return pow2;
+}
+
+// Rows of one TMA box when boxes of equal size cover exactly `rows` staged rows (at most 256 each).
+constexpr int even_box(int rows) {
+  int q = (rows + 255) / 256;
+  while (rows % q != 0) ++q;
+  return rows / q;
+}
 
 // Move a pointer by `bytes` (null stays null).
 __device__ __forceinline__ const void* bmove(const void* p, long long bytes) {

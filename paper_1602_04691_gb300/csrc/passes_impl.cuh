@@ -77,7 +77,7 @@ __device__ __forceinline__ cpx<T> tw_mul_val(cpx<T> z, cpx<T> w) {
 }
 
 // Two-dimensional twiddle table of a two-stage length-L transform:
-// tab2[k1 * L2 + j] = tab[(j * k1) mod L] for k1 < L1, j < L2 (L entries), so
+// tab2[k1 * L2 + j] = tab[j * k1] for k1 < L1, j < L2 (j k1 < L; L entries), so
 // that a thread with fixed j (or fixed k1) finds its twiddles at constant
 // offsets from one base pointer.
 template <int L, int L2X = Split<L>::L2, class T>
@@ -85,7 +85,7 @@ __device__ __forceinline__ void fill_tw2(cpx<T>* tab2, const cpx<T>* tab, int ti
   constexpr int L2 = L2X;
   for (int i = tid; i < L; i += nt) {
     const int k1 = i / L2, j = i - k1 * L2;
-    tab2[i] = tab[(j * k1) & (L - 1)];
+    tab2[i] = tab[j * k1];
   }
 }
 
@@ -97,8 +97,14 @@ constexpr int lines_contig_f32() {
 }
 
 // Lines per tile of the persistent FP32 X passes: 128 threads of L2 each.
+// Mixed lengths: the fewest lines that make whole warps and at least 96 threads.
 template <int L>
 constexpr int xpipe_cols() {
+  if (is_mixed_len(L)) {
+    int m = 1;
+    while ((m * Split<L>::L2) % 32 != 0 || m * Split<L>::L2 < 96) ++m;
+    return m;
+  }
   constexpr int c = lines_contig_f32<L>() / 2;
   return c < 1 ? 1 : c;
 }
@@ -192,7 +198,7 @@ __global__ void __launch_bounds__(Tile<L, C, T>::NT, Tile<L, C, T>::MINB) k_xfwd
   }
   dft<L1, -1, HALF>(r);
 #pragma unroll
-  for (int k1 = 1; k1 < L1; ++k1) r[k1] = twL_mul<-1>(r[k1], tw, (j2 * k1) & (L - 1));
+  for (int k1 = 1; k1 < L1; ++k1) r[k1] = twL_mul<-1>(r[k1], tw, j2 * k1);
 #pragma unroll
   for (int k1 = 0; k1 < L1; ++k1) sm[c * PC + k1 * PK + j2] = settle(r[k1]);
   __syncthreads();
@@ -426,7 +432,7 @@ __global__ void __launch_bounds__(Tile<L, C, T>::NT, Tile<L, C, T>::MINB) k_xinv
       b[k2] = l2 < a.nlines ? in[l2 * a.line_len_in + k1 + L1 * k2] : czero<T>();
     dft<L2, +1, false>(b);
 #pragma unroll
-    for (int ja = 1; ja < L2; ++ja) b[ja] = twL_mul<+1>(b[ja], tw, (ja * k1) & (L - 1));
+    for (int ja = 1; ja < L2; ++ja) b[ja] = twL_mul<+1>(b[ja], tw, ja * k1);
 #pragma unroll
     for (int ja = 0; ja < L2; ++ja) sm[c2 * PCI + ja * PKI + k1] = settle(b[ja]);
   }
@@ -640,7 +646,7 @@ __global__ void __launch_bounds__(XInvPipe<L, C>::NT, L > 1024 ? 1 : 3) k_xinv_p
       for (int k2 = 0; k2 < L2; ++k2) b[it][k2] = okl ? B[c2 * L + k1 + L1 * k2] : czero<T>();
       dft<L2, +1, false>(b[it]);
 #pragma unroll
-      for (int j = 1; j < L2; ++j) b[it][j] = twL_mul<+1>(b[it][j], tw, (j * k1) & (L - 1));
+      for (int j = 1; j < L2; ++j) b[it][j] = twL_mul<+1>(b[it][j], tw, j * k1);
     }
     __syncthreads();   // raw tile consumed: the exchange reuses the buffer
 #pragma unroll
@@ -663,7 +669,7 @@ __global__ void __launch_bounds__(XInvPipe<L, C>::NT, L > 1024 ? 1 : 3) k_xinv_p
     } else {
       cp_async_commit();
     }
-    dft<L1, +1, false>(r);
+    dft_low<L1, +1>(r);
     if (bulk) {
       if (!bulk_wait(&bars[1], ph_e, pend_e)) { failed = true; break; }
     } else {
@@ -761,7 +767,7 @@ __global__ void __launch_bounds__(Tile<L, C, T>::NT) k_strided(SArgs a0) {
     }
     dft<L1, -1, HALF>(r);
 #pragma unroll
-    for (int k1 = 1; k1 < L1; ++k1) r[k1] = twL_mul<-1>(r[k1], tw, (j2 * k1) & (L - 1));
+    for (int k1 = 1; k1 < L1; ++k1) r[k1] = twL_mul<-1>(r[k1], tw, j2 * k1);
 #pragma unroll
     for (int k1 = 0; k1 < L1; ++k1) sm[c * PC + k1 * PK + j2] = settle(r[k1]);
     __syncthreads();
@@ -821,7 +827,7 @@ __global__ void __launch_bounds__(Tile<L, C, T>::NT) k_strided(SArgs a0) {
     map_s<LAYOUT_STRIDED, C, L1>(tid + it * NT, c2, k1);
     dft<L2, +1, false>(b[it]);
 #pragma unroll
-    for (int ja = 1; ja < L2; ++ja) b[it][ja] = twL_mul<+1>(b[it][ja], tw, (ja * k1) & (L - 1));
+    for (int ja = 1; ja < L2; ++ja) b[it][ja] = twL_mul<+1>(b[it][ja], tw, ja * k1);
 #pragma unroll
     for (int ja = 0; ja < L2; ++ja) sm[c2 * PCI + ja * PKI + k1] = settle(b[it][ja]);
   }
@@ -885,7 +891,7 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_st
       }
       dft<8, -1, HALF>(v);
 #pragma unroll
-      for (int t = 1; t < 8; ++t) v[t] = twL_mul<-1>(v[t], TW, (j * t) & (L - 1));
+      for (int t = 1; t < 8; ++t) v[t] = twL_mul<-1>(v[t], TW, j * t);
 #pragma unroll
       for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
     }
@@ -912,7 +918,7 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_st
       }
       dft<8, +1, false>(v);
 #pragma unroll
-      for (int t = 1; t < 8; ++t) v[t] = twL_mul<+1>(v[t], TW, (j * t) & (L - 1));
+      for (int t = 1; t < 8; ++t) v[t] = twL_mul<+1>(v[t], TW, j * t);
 #pragma unroll
       for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
     }
@@ -951,7 +957,7 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_xf
     }
     dft<8, -1, HALF>(v);
 #pragma unroll
-    for (int t = 1; t < 8; ++t) v[t] = twL_mul<-1>(v[t], TW, (j * t) & (L - 1));
+    for (int t = 1; t < 8; ++t) v[t] = twL_mul<-1>(v[t], TW, j * t);
 #pragma unroll
     for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
   }
@@ -996,7 +1002,7 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_xi
     for (int t = 0; t < 8; ++t) v[t] = line < a.nlines ? in[line * a.line_len_in + j + t * S8] : czero<T>();
     dft<8, +1, false>(v);
 #pragma unroll
-    for (int t = 1; t < 8; ++t) v[t] = twL_mul<+1>(v[t], TW, (j * t) & (L - 1));
+    for (int t = 1; t < 8; ++t) v[t] = twL_mul<+1>(v[t], TW, j * t);
 #pragma unroll
     for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
   }
@@ -1428,7 +1434,7 @@ k_zconv_pipe(const __grid_constant__ SArgs a) {
       for (int k1 = 1; k1 < L1; ++k1) r[k1] = tw_mul_val<-1>(r[k1], t2[k1 * L2]);
     } else {
 #pragma unroll
-      for (int k1 = 1; k1 < L1; ++k1) r[k1] = twL_mul<-1>(r[k1], tw, (jl * k1) & (L - 1));
+      for (int k1 = 1; k1 < L1; ++k1) r[k1] = twL_mul<-1>(r[k1], tw, jl * k1);
     }
 #pragma unroll
     for (int k1 = 0; k1 < L1; ++k1) E[c * PC + k1 * PK + jl] = r[k1];
@@ -1473,7 +1479,7 @@ k_zconv_pipe(const __grid_constant__ SArgs a) {
         for (int ja = 1; ja < L2; ++ja) b[it][ja] = tw_mul_val<+1>(b[it][ja], t2[ja]);
       } else {
 #pragma unroll
-        for (int ja = 1; ja < L2; ++ja) b[it][ja] = twL_mul<+1>(b[it][ja], tw, (ja * k1) & (L - 1));
+        for (int ja = 1; ja < L2; ++ja) b[it][ja] = twL_mul<+1>(b[it][ja], tw, ja * k1);
       }
     }
     __syncthreads();   // forward exchange and the spectrum slice fully read
@@ -1499,6 +1505,196 @@ k_zconv_pipe(const __grid_constant__ SArgs a) {
     tile = next;
   }
   cp_async_wait_all();
+}
+
+// ---------------------------------------------------------------------------
+// FP32 Z convolution at the mixed lengths: k_zconv_pipe's stages on 8-column
+// tiles, several small CTAs per SM (their arithmetic and shared-memory phases
+// overlap; one 16-column CTA per SM would take turns).  The column pitch of
+// the exchange is 2 modulo 4, so that the 8 columns x 2 rows of a half warp
+// fall into 16 different 8-byte banks, and the twiddle table is padded to
+// L2 + 1 entries a row for the same reason (square splits read it by its
+// symmetry instead).  The spectrum is grouped by 8 columns (zgroup), so a
+// tile's slice is one contiguous run.  n = 260, 576 points: 0.56 ms, where
+// the 1024-point pass on the same grid takes 3.06 ms.
+// ---------------------------------------------------------------------------
+template <int L>
+struct ZMix {
+  static constexpr int C = 8;
+  static constexpr int L1 = Split<L>::L1, L2 = Split<L>::L2;
+  static constexpr int NT = C * L2, NI = L1 / L2;
+  static constexpr int PK = L2 + 1, PKI = L1 + 1;
+  static constexpr int pitch(int v) { return v + (6 - v % 4) % 4; }   // next v = 2 (mod 4)
+  static constexpr int PC = pitch(L1 * PK), PCI = pitch(L2 * PKI);
+  static constexpr int PT = L1 == L2 ? L2 : L2 + 1;
+  static constexpr int r16(int v) { return (v + 15) / 16 * 16; }      // regions start on 128 bytes
+  static constexpr int E_ELEMS = r16(C * (PC > PCI ? PC : PCI));
+  static constexpr int S_ELEMS = r16((L / 2 + 1) * C);
+  static constexpr int TW_ELEMS = r16(L1 * PT);
+  static constexpr size_t SMEM_BYTES = size_t(E_ELEMS + S_ELEMS + TW_ELEMS) * sizeof(cpx<float>) + 128 + 16;
+  // CTAs per SM the register budget is set for: as many as shared memory holds,
+  static constexpr int fit = int(227 * 1024 / (SMEM_BYTES + 1024));
+  // at 96 registers a thread or more
+  static constexpr int warps = (NT + 31) / 32;
+  static constexpr int MINB = fit * warps > 21 ? 21 / warps : fit;
+};
+
+template <int L>
+__global__ void __launch_bounds__(ZMix<L>::NT, ZMix<L>::MINB) k_zconv_mix(const __grid_constant__ SArgs a) {
+  using T = float;
+  using Z = ZMix<L>;
+  constexpr int C = Z::C, L1 = Z::L1, L2 = Z::L2, NT = Z::NT, NI = Z::NI;
+  constexpr int PK = Z::PK, PC = Z::PC, PKI = Z::PKI, PCI = Z::PCI, PT = Z::PT;
+  constexpr int kSlice = (L / 2 + 1) * C;
+  extern __shared__ __align__(128) unsigned char smraw[];
+  unsigned char* base = smraw + ((128u - (smem_addr(smraw) & 127u)) & 127u);
+  cpx<T>* E = reinterpret_cast<cpx<T>*>(base);
+  cpx<T>* S = E + Z::E_ELEMS;
+  cpx<T>* TW = S + Z::S_ELEMS;
+  unsigned long long* bar = reinterpret_cast<unsigned long long*>(TW + Z::TW_ELEMS);
+  const int tid = threadIdx.x;
+  const int c = tid % C, jl = tid / C;
+  const cpx<T>* twg = reinterpret_cast<const cpx<T>*>(a.twL);
+  for (int i = tid; i < L; i += NT) {
+    const int k1 = i / L2, j = i - k1 * L2;
+    TW[k1 * PT + j] = twg[j * k1];
+  }
+  constexpr int col_blocks = L / C;
+  constexpr int per_rhs = L * col_blocks;
+  const int ntiles = per_rhs * (a.nrhs > 1 ? a.nrhs : 1);
+  const int step = gridDim.x;
+  const bool tma = a.zrows_ok != 0;   // uniform over the grid
+  unsigned phase = 0;
+  if (tma && tid == 0) {
+    mbar_init(bar, 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  // Wait for the staged copy, bounded as in k_zconv_pipe; false: leave.
+  auto staged = [&]() -> bool {
+    if (tma) {
+      const bool ok = mbar_wait(bar, phase);
+      if (__syncthreads_or(!ok)) {
+        if (tid == 0 && a.err != nullptr) atomicExch(a.err, 1);
+        if (!ok) mbar_wait(bar, phase);
+        return false;
+      }
+      phase ^= 1u;
+      return true;
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    return true;
+  };
+  auto stage_rows = [&](int t) {
+    if (!tma) {
+      zpipe_prefetch_rows<T, L, C, NT>(a, t, per_rhs, S);
+    } else if (tid == 0) {
+      zpipe_tma_rows<L, C>(a, t, per_rhs, S, bar);
+    }
+  };
+  auto stage_slice = [&](int rhs, int ky, int cb) {
+    const int g = a.rhs_per_ghat > 0 ? rhs / a.rhs_per_ghat : 0;
+    const cpx<T>* src = reinterpret_cast<const cpx<T>*>(bmove(a.ghatZ, a.bs_ghatZ * g)) +
+                        ((long long)mirror_index(ky, L) * col_blocks + cb) * kSlice;
+    if (!tma) {
+      for (int k = tid; k < kSlice / 2; k += NT) cp_async16(S + 2 * k, src + 2 * k);
+      cp_async_commit();
+    } else if (tid == 0) {
+      constexpr unsigned bytes = unsigned(kSlice) * unsigned(sizeof(cpx<T>));
+      fence_proxy_async();
+      mbar_expect_tx(bar, bytes);
+      bulk_load(S, src, bytes, bar);
+    }
+  };
+
+  int tile = next_live_tile(a, blockIdx.x, step, per_rhs, ntiles);
+  if (tile < ntiles) stage_rows(tile);
+  while (tile < ntiles) {
+    const int rhs = tile / per_rhs;
+    const int tl = tile - rhs * per_rhs;
+    const int ky = ky_of_slot(tl / col_blocks, L);
+    const int cb = tl % col_blocks;
+    const int next = next_live_tile(a, tile + step, step, per_rhs, ntiles);
+    if (!staged()) return;   // rows visible; the previous tile is done with E
+    cpx<T> r[L1];
+#pragma unroll
+    for (int j1 = 0; j1 < L1; ++j1) {
+      r[j1] = czero<T>();
+      if (j1 < L1 / 2) {
+        const int j = j1 * L2 + jl;
+        if (j < a.n_in) r[j1] = S[j * C + c];
+      }
+    }
+    __syncthreads();   // staging buffer consumed
+    stage_slice(rhs, ky, cb);
+    dft<L1, -1, true>(r);
+    const cpx<T>* tj = TW + jl;
+#pragma unroll
+    for (int k1 = 1; k1 < L1; ++k1) r[k1] = tw_mul_val<-1>(r[k1], tj[k1 * PT]);
+#pragma unroll
+    for (int k1 = 0; k1 < L1; ++k1) E[c * PC + k1 * PK + jl] = r[k1];
+    if (!staged()) return;   // exchange and spectrum slice visible
+    cpx<T> b[NI][L2];
+#pragma unroll
+    for (int it = 0; it < NI; ++it) {
+      const int s = tid + it * NT;
+      const int c2 = s % C, k1 = s / C;
+#pragma unroll
+      for (int j = 0; j < L2; ++j) b[it][j] = E[c2 * PC + k1 * PK + j];
+      dft<L2, -1, false>(b[it]);
+      const cpx<T>* lo = S + k1 * C + c2;          // kz = k1 + L1 k2 below L/2, L - kz from there on
+      const cpx<T>* hi = S + (L - k1) * C + c2;
+#pragma unroll
+      for (int k2 = 0; k2 < L2; ++k2)
+        b[it][k2] = cmul(b[it][k2], k2 < L2 / 2 ? lo[k2 * L1 * C] : hi[-k2 * L1 * C]);
+      dft<L2, +1, false>(b[it]);
+#pragma unroll
+      for (int ja = 1; ja < L2; ++ja)
+        b[it][ja] = tw_mul_val<+1>(b[it][ja], L1 == L2 ? TW[ja * PT + k1] : TW[k1 * PT + ja]);
+    }
+    __syncthreads();   // exchange and slice fully read
+    if (next < ntiles) stage_rows(next);
+#pragma unroll
+    for (int it = 0; it < NI; ++it) {
+      const int s = tid + it * NT;
+      const int c2 = s % C, k1 = s / C;
+#pragma unroll
+      for (int ja = 0; ja < L2; ++ja) E[c2 * PCI + ja * PKI + k1] = b[it][ja];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k1 = 0; k1 < L1; ++k1) r[k1] = E[c * PCI + jl * PKI + k1];
+    dft_low<L1, +1>(r);
+    cpx<T>* out = reinterpret_cast<cpx<T>*>(bmove(a.out, a.bs_out * rhs)) + (long long)ky * a.out_outer + (long long)cb * C;
+#pragma unroll
+    for (int jb = 0; jb < L1 / 2; ++jb) {
+      const int j = jl + L2 * jb;
+      if (j < a.n_out) out[(long long)j * a.out_pt + c] = r[jb];
+    }
+    tile = next;
+  }
+  cp_async_wait_all();
+}
+
+template <int L>
+cudaError_t launch_zconv_mix_L(SArgs a, cudaStream_t s, bool setup, int sm_count) {
+  using Z = ZMix<L>;
+  auto kfn = k_zconv_mix<L>;
+  static int per_sm = 0;   // resident CTAs per SM, measured once at set-up
+  if (setup) {
+    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Z::SMEM_BYTES));
+    if (e != cudaSuccess) return e;
+    int nb = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kfn, Z::NT, Z::SMEM_BYTES);
+    per_sm = (e == cudaSuccess && nb > 0) ? nb : 1;
+    return e;
+  }
+  const long long ntiles = (long long)L * (L / Z::C) * std::max(1, a.nrhs);
+  const int resident = a.cta_cap > 0 ? std::min(std::max(1, per_sm), a.cta_cap) : std::max(1, per_sm);
+  const unsigned gx = unsigned(std::max(1LL, std::min(ntiles, (long long)std::max(1, sm_count) * resident)));
+  kfn<<<gx, Z::NT, Z::SMEM_BYTES, s>>>(a);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -1555,7 +1751,7 @@ __global__ void __launch_bounds__(ZSmem<L, C, T>::NT, ZSmem<L, C, T>::MINB) k_zc
       }
       dft<8, -1, true>(v);
 #pragma unroll
-      for (int t = 1; t < 8; ++t) v[t] = twL_mul<-1>(v[t], TW, (j * t) & (L - 1));
+      for (int t = 1; t < 8; ++t) v[t] = twL_mul<-1>(v[t], TW, j * t);
 #pragma unroll
       for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
     }
@@ -1581,7 +1777,7 @@ __global__ void __launch_bounds__(ZSmem<L, C, T>::NT, ZSmem<L, C, T>::MINB) k_zc
 #pragma unroll
       for (int t = 0; t < 8; ++t) v[t] = ld_stage(X + sidx<C>(j + t * S8, c));
 #pragma unroll
-      for (int t = 1; t < 8; ++t) v[t] = twL_mul<+1>(v[t], TW, (j * t) & (L - 1));
+      for (int t = 1; t < 8; ++t) v[t] = twL_mul<+1>(v[t], TW, j * t);
       dft<8, +1, false>(v);
 #pragma unroll
       for (int t = 0; t < 8; ++t) {
@@ -1895,10 +2091,10 @@ k_yinv_pipe(const __grid_constant__ SArgs a) {
     for (int k1 = 0; k1 < L1; ++k1) r[k1] = B[c * PCI + ja * PKI + k1];
     __syncthreads();   // exchange consumed: the buffer takes the next tile
     if (next < ntiles) stage(next);
-    dft<L1, +1, false>(r);
+    dft_low<L1, +1>(r);
     cpx<T>* out = reinterpret_cast<cpx<T>*>(bmove(a.out, a.bs_out * rhs)) + outer * a.out_outer + (long long)cb * C;
 #pragma unroll
-    for (int jb = 0; jb < L1; ++jb) {
+    for (int jb = 0; jb < L1 / 2; ++jb) {   // n_out <= L/2
       const int j = ja + L2 * jb;
       if (j < a.n_out) out[(long long)j * a.out_pt + c] = r[jb];
     }
@@ -2052,9 +2248,85 @@ cudaError_t launch_zconv_reg_L(SArgs a, cudaStream_t s, bool setup) {
 // stage either has a zero-padded half on input or keeps half its outputs.
 constexpr int kMaxRegL = 1024;
 
+// The mixed lengths (MixRad): FP32 runs the pipelined kernels (and, for the
+// prologues those do not take, the one-tile-per-CTA X kernel), the other
+// arithmetics the shared-memory kernels.  They have one schedule: the TILES
+// and variant fields choose among kernels of the power-of-two lengths.  Full
+// (not half-empty) transforms exist in FP64 alone, for the kernel spectrum.
+template <class T, int L, bool HALF>
+cudaError_t launch_xfwd_mix_L(const XArgs& a, cudaStream_t s, bool setup) {
+  if constexpr (std::is_same<T, float>::value) {
+    if constexpr (HALF) {
+      constexpr int C = xpipe_cols<L>();
+      using TL = Tile<L, C, T>;
+      auto kfn = k_xfwd<T, L, C, HALF>;
+      if (setup) {
+        cudaError_t e = launch_xfwd_pipe_L<L>(a, s, true);
+        if (e != cudaSuccess) return e;
+        return cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(TL::SMEM_BYTES));
+      }
+      if (xfwd_pipe_ok(a, L)) return launch_xfwd_pipe_L<L>(a, s, false);
+      kfn<<<dim3(unsigned((a.nlines + C - 1) / C), unsigned(std::max(1, a.nrhs))), TL::NT, TL::SMEM_BYTES, s>>>(a);
+      return cudaGetLastError();
+    }
+  } else if constexpr (HALF || std::is_same<T, double>::value) {
+    constexpr int CS = 2;   // two lines per CTA, four CTAs per SM, as at the powers of two
+    using LS = LSmem<L, CS, T>;
+    auto kfs = k_xfwd_smem<T, L, CS, HALF>;
+    if (setup) return cudaFuncSetAttribute(kfs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LS::SMEM_BYTES));
+    kfs<<<dim3(unsigned((a.nlines + CS - 1) / CS), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s>>>(a);
+    return cudaGetLastError();
+  }
+  return setup ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+template <class T, int L>
+cudaError_t launch_xinv_mix_L(const XArgs& a, Scalars* sc, int fin, cudaStream_t s, bool setup, unsigned* nblocks) {
+  if constexpr (std::is_same<T, float>::value) {
+    return launch_xinv_pipe_L<L>(a, sc, fin, s, setup, nblocks);
+  } else {
+    constexpr int CS = 2;
+    using LS = LSmem<L, CS, T>;
+    auto kfs = k_xinv_smem<T, L, CS>;
+    const unsigned grid = unsigned((a.nlines + CS - 1) / CS);
+    if (nblocks) *nblocks = grid;
+    if (setup) return cudaFuncSetAttribute(kfs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LS::SMEM_BYTES));
+    kfs<<<dim3(grid, unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s>>>(a, sc, fin);
+    return cudaGetLastError();
+  }
+}
+
+// Columns per tile of the FP32 Y passes at a mixed length: 16 (TMA rows of
+// 128 bytes) where 16 divides the length and two CTAs fit an SM.
+template <int L>
+constexpr int y_mix_cols() { return (L % 16 == 0 && L <= 400) ? 16 : 8; }
+
+template <class T, int L, int SMODE, bool HALF>
+cudaError_t launch_strided_mix_L(SArgs a, cudaStream_t s, bool setup) {
+  if constexpr (std::is_same<T, float>::value) {
+    if constexpr (SMODE == SMODE_FWD && HALF)
+      return launch_yfwd_pipe_V<T, L, y_mix_cols<L>(), Split<L>::L1>(a, s, setup, a.sm_count);
+    else if constexpr (SMODE == SMODE_INV)
+      return launch_yinv_pipe_V<L, y_mix_cols<L>(), Split<L>::L1>(a, s, setup, a.sm_count);
+    else
+      return setup ? cudaSuccess : cudaErrorInvalidValue;
+  } else if constexpr (SMODE == SMODE_INV || HALF || std::is_same<T, double>::value) {
+    constexpr int CS = 4;
+    using LS = LSmem<L, CS, T>;
+    auto kfs = k_strided_smem<T, L, CS, SMODE, (SMODE == SMODE_FWD ? HALF : true)>;
+    if (setup) return cudaFuncSetAttribute(kfs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LS::SMEM_BYTES));
+    a.col_blocks = (a.ncols + CS - 1) / CS;
+    kfs<<<dim3(unsigned(a.nouter) * unsigned(a.col_blocks), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s>>>(a);
+    return cudaGetLastError();
+  }
+  return setup ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 template <class T, int L, bool HALF>
 cudaError_t launch_xfwd_L(const XArgs& a, cudaStream_t s, bool setup) {
-  if constexpr (L > kMaxRegL) {
+  if constexpr (is_mixed_len(L)) {
+    return launch_xfwd_mix_L<T, L, HALF>(a, s, setup);
+  } else if constexpr (L > kMaxRegL) {
     // FP32 solver prologues: the pipelined kernel (4-line tiles, one CTA per SM)
     if constexpr (std::is_same<T, float>::value && HALF) {
       if (setup) {
@@ -2077,7 +2349,9 @@ cudaError_t launch_xfwd_L(const XArgs& a, cudaStream_t s, bool setup) {
 
 template <class T, int L>
 cudaError_t launch_xinv_L(const XArgs& a, Scalars* sc, int fin, cudaStream_t s, bool setup, unsigned* nblocks) {
-  if constexpr (L > kMaxRegL && std::is_same<T, float>::value) {
+  if constexpr (is_mixed_len(L)) {
+    return launch_xinv_mix_L<T, L>(a, sc, fin, s, setup, nblocks);
+  } else if constexpr (L > kMaxRegL && std::is_same<T, float>::value) {
     return launch_xinv_pipe_L<L>(a, sc, fin, s, setup, nblocks);   // as for L <= kMaxRegL
   } else if constexpr (L > kMaxRegL) {
     constexpr int CS = 4;
@@ -2095,7 +2369,9 @@ cudaError_t launch_xinv_L(const XArgs& a, Scalars* sc, int fin, cudaStream_t s, 
 
 template <class T, int L, int SMODE, bool HALF>
 cudaError_t launch_strided_L(SArgs a, cudaStream_t s, bool setup) {
-  if constexpr (L > kMaxRegL) {
+  if constexpr (is_mixed_len(L)) {
+    return launch_strided_mix_L<T, L, SMODE, HALF>(a, s, setup);
+  } else if constexpr (L > kMaxRegL) {
     if constexpr (SMODE == SMODE_ZCONV) {
       return launch_zconv_smem_L<T, L>(a, s, setup, a.sm_count);
     } else {
@@ -2138,7 +2414,10 @@ cudaError_t launch_strided_L(SArgs a, cudaStream_t s, bool setup) {
 // schedule and the kernel of the other arithmetics.
 template <class T, int L>
 cudaError_t launch_zconv_L(SArgs a, cudaStream_t s, bool setup) {
-  if constexpr (L > kMaxRegL) {
+  if constexpr (is_mixed_len(L)) {
+    if constexpr (std::is_same<T, float>::value) return launch_zconv_mix_L<L>(a, s, setup, a.sm_count);
+    else return launch_zconv_smem_L<T, L>(a, s, setup, a.sm_count);
+  } else if constexpr (L > kMaxRegL) {
     if constexpr (std::is_same<T, float>::value) {
       if (setup) {
         cudaError_t e = launch_zconv_pipe_L<T, L>(a, s, true, a.sm_count);
@@ -2153,7 +2432,8 @@ cudaError_t launch_zconv_L(SArgs a, cudaStream_t s, bool setup) {
   }
 }
 
-#define ORI_FOR_EACH_L(X) X(4) X(8) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048)
+#define ORI_FOR_EACH_L(X) \
+  X(4) X(8) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048) X(144) X(200) X(288) X(400) X(576) X(800)
 
 template <class T>
 cudaError_t run_xfwd(int L, bool half, const XArgs& a, cudaStream_t s, bool setup) {

@@ -137,11 +137,10 @@ __global__ void k_spectrum_convert(const cpx<double>* __restrict__ g64, long lon
 }
 
 // FP32 spectrum in the order the Z pass reads it: for each my and each block
-// of 16 kx columns, the entries mz = 0..L/2 as rows of 16 (one contiguous
-// slice per Z tile).  gz[((my * (L/16) + cb) * H + mz) * 16 + c] =
-// g32[(mz * H + my) * H + m(cb*16 + c)].
-__global__ void k_build_ghatZ(const cpx<float>* __restrict__ g32, cpx<float>* gz, int L, int H) {
-  constexpr int G = kZGroup;
+// of G = zgroup(L) kx columns, the entries mz = 0..L/2 as rows of G (one contiguous
+// slice per Z tile).  gz[((my * (L/G) + cb) * H + mz) * G + c] =
+// g32[(mz * H + my) * H + m(cb*G + c)].
+__global__ void k_build_ghatZ(const cpx<float>* __restrict__ g32, cpx<float>* gz, int L, int H, int G) {
   const long long total = (long long)H * (L / G) * H * G;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
