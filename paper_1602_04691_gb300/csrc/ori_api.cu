@@ -604,6 +604,13 @@ static ori_status run_conv(ori_plan_s* p, XArgs pro, XArgs epi, int fin, cudaStr
 
 // Blocks per right-hand side of the vector kernels.
 static int vgrid(const ori_plan_s* p, int nrhs) { return std::max(16, p->vec_grid / std::max(1, nrhs)); }
+// ... of the kernels that end in a grid reduction: at least 4096 cells a
+// block.  A block's FP64 reduction and its arrival at the counter cost about as
+// much as streaming that many cells, so small grids take fewer blocks (COCG
+// update at n = 20: 35 us with 1216 blocks of mostly idle threads).
+static int vgrid_sum(const ori_plan_s* p, int nrhs) {
+  return int(std::max<long long>(1, std::min<long long>(vgrid(p, nrhs), (p->n3 + 4095) / 4096)));
+}
 
 // Control copy on the plan's stream by k_small_copy (rows of `bytes` at the
 // given pitches); dst and src are device addresses (device memory or the
@@ -1225,7 +1232,7 @@ static ori_status cocg_iteration(ori_plan_s* p, int nrhs, int rhs_per_k, cpx<T>*
   epi.bs_xin = bsv;
   epi.bs_out = bsv;
   ORI_TRY(run_conv<T>(p, pro, epi, FIN_ALPHA, p->ps, Mask{&p->sc->done, int(sizeof(Scalars))}, nrhs, rhs_per_k));
-  const int vg = vgrid(p, nrhs);
+  const int vg = vgrid_sum(p, nrhs);
   ORI_VEC(p, ORI_PASS_UPDATE + (sizeof(T) == 4 ? 0 : ORI_PASS_FP64),
           (k_cocg_update<T><<<dim3(vg, nrhs), 256, 0, p->ps>>>(x, pp, r, q, p->n3, p->sc, p->partials)));
   return ORI_OK;
@@ -1268,7 +1275,7 @@ static ori_status cocg_inner(ori_plan_s* p, int nrhs, int rhs_per_k, cpx<T>* x, 
   double* h_tols = p->h_small;
   for (int i = 0; i < nrhs; ++i) h_tols[i] = tols_host[i];
   ORI_TRY(small_copy(p, p->d_tols, p->h_small_d, nrhs * sizeof(double)));   // h_tols is h_small
-  const int vg = vgrid(p, nrhs);
+  const int vg = vgrid_sum(p, nrhs);
   ORI_VEC(p, ORI_PASS_VECTOR + (sizeof(T) == 4 ? 0 : ORI_PASS_FP64),
           (k_cocg_init<T><<<dim3(vg, nrhs), 256, 0, p->ps>>>(r, x, p->n3, p->sc, p->partials, p->d_tols, maxit,
                                                                zero_x ? 1 : 0)));
@@ -1676,7 +1683,7 @@ static ori_status solve_batch(ori_plan_s* p, int nk, int ndir, const double* rhs
               p->d_kv, p->d_dir, p->n, p->d, p->origin[0], p->origin[1], p->origin[2], p->d_phase)));
   // u0 is kept only where S = 0 cells need it for the recovery
   ORI_VEC(p, ORI_PASS_VECTOR,
-          (k_rhs<<<dim3(vg, nrhs), 256, rhs_dev ? 0 : 3 * size_t(p->n) * sizeof(cpx<double>), p->ps>>>(
+          (k_rhs<<<dim3(vgrid_sum(p, nrhs), nrhs), 256, rhs_dev ? 0 : 3 * size_t(p->n) * sizeof(cpx<double>), p->ps>>>(
               reinterpret_cast<const cpx<double>*>(rhs_dev), p->S64, p->zero_S ? p->u0 : nullptr, p->b64, p->n,
               p->d_phase, p->sc, p->partials)));
   ORI_TRY(read_heads(p, nrhs));
@@ -1780,7 +1787,7 @@ ori_status ori_adjoint_solve(ori_plan_t p, const double* u_dev, const double* ec
   ORI_TRY(enter(p, user));
   ORI_CUDA(cudaEventRecord(p->ev0, p->ps));
   ORI_VEC(p, ORI_PASS_VECTOR,
-          (k_adj_rhs<<<p->vec_grid, 256, 0, p->ps>>>(reinterpret_cast<const cpx<double>*>(econj_dev), p->S64, p->b64,
+          (k_adj_rhs<<<vgrid_sum(p, 1), 256, 0, p->ps>>>(reinterpret_cast<const cpx<double>*>(econj_dev), p->S64, p->b64,
                                                       p->n3, p->sc, p->partials)));
   ORI_TRY(read_heads(p, 1));
   const double bnorm = std::sqrt(p->h_sc[0].sum.x);
@@ -1867,7 +1874,7 @@ static ori_status time_fp32_operator(ori_plan_s* p, int nrhs, int reps, float* m
 // Device time of one FP32 COCG vector update over the batch (scalars reset
 // before each launch so that no system is flagged as finished).
 static ori_status time_fp32_update(ori_plan_s* p, int nrhs, int reps, float* ms) {
-  const int vg = vgrid(p, nrhs);
+  const int vg = vgrid_sum(p, nrhs);
   float total = 0.f;
   for (int i = 0; i <= reps; ++i) {
     ORI_CUDA(cudaMemsetAsync(p->sc, 0, size_t(nrhs) * sizeof(Scalars), p->ps));

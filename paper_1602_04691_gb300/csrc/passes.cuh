@@ -244,13 +244,34 @@ __device__ __forceinline__ void map_s(int s, int& c, int& k) {
 // ---------------------------------------------------------------------------
 // Warp + block reduction of a double2 partial into partials[blockIdx.x]
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double2 warp_sum2(double2 v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-    v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-  }
+// FP64 additions run at 2 lanes a cycle and SM, so a block's reductions cost
+// more than its loads when every lane carries every value through all five
+// butterfly steps.  Here the values are split over the lanes first: half the
+// lanes go on with one value, half with the other (5 additions a warp for two
+// values, 6 for four, instead of 10 and 20).
+__device__ __forceinline__ double warp_sum_tail(double v, int from) {
+  for (int o = from; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+__device__ __forceinline__ double2 warp_sum2(double2 v) {
+  const bool up = (threadIdx.x & 16) != 0;
+  double k = up ? v.y : v.x;
+  k += __shfl_xor_sync(0xffffffffu, up ? v.x : v.y, 16);
+  k = warp_sum_tail(k, 8);
+  return make_double2(__shfl_sync(0xffffffffu, k, 0), __shfl_sync(0xffffffffu, k, 16));
+}
+// Sums of a and b over the warp, valid in every lane.
+__device__ __forceinline__ void warp_sum4(double2& a, double2& b) {
+  const bool up = (threadIdx.x & 16) != 0, odd = (threadIdx.x & 8) != 0;
+  double2 k = up ? b : a;
+  const double2 s = up ? a : b;
+  k.x += __shfl_xor_sync(0xffffffffu, s.x, 16);
+  k.y += __shfl_xor_sync(0xffffffffu, s.y, 16);
+  double v = odd ? k.y : k.x;
+  v += __shfl_xor_sync(0xffffffffu, odd ? k.x : k.y, 8);
+  v = warp_sum_tail(v, 4);
+  a = make_double2(__shfl_sync(0xffffffffu, v, 0), __shfl_sync(0xffffffffu, v, 8));
+  b = make_double2(__shfl_sync(0xffffffffu, v, 16), __shfl_sync(0xffffffffu, v, 24));
 }
 
 // All threads of the block must call it.  Uses 32 double2 of scratch smem.

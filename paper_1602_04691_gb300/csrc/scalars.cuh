@@ -12,6 +12,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "passes.cuh"   // warp sums
+
 namespace ori {
 
 enum { FIN_NONE = 0,    // no reduction
@@ -63,31 +65,42 @@ __device__ __forceinline__ bool last_block_arrives(Scalars* sc, int& s_last) {
   return s_last != 0;
 }
 
-// Sum partials[stride*i + which] over i in [0, nparts) in a fixed order.
-// Called by all threads of the last block; result valid in thread 0.
-__device__ __forceinline__ double2 reduce_partials(const double2* partials, int nparts, int stride,
-                                                   int which, double2* red) {
-  double2 acc = make_double2(0.0, 0.0);
+// Sum of the partials over i in [0, nparts) in a fixed order: partials[i]
+// -> a, or with PAIRS partials[2 i] -> a and partials[2 i + 1] -> b in one
+// sweep.  Called by all threads of the last block (whole warps); valid in
+// thread 0.
+template <bool PAIRS>
+__device__ __forceinline__ void reduce_partials(const double2* partials, int nparts, double2* red, double2& a,
+                                                double2& b) {
+  a = make_double2(0.0, 0.0);
+  b = make_double2(0.0, 0.0);
   for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
-    const double2 v = __ldcg(partials + (long long)stride * i + which);
-    acc.x += v.x;
-    acc.y += v.y;
+    const double2 v = __ldcg(partials + (PAIRS ? 2LL * i : i));
+    a.x += v.x;
+    a.y += v.y;
+    if (PAIRS) {
+      const double2 w = __ldcg(partials + 2LL * i + 1);
+      b.x += w.x;
+      b.y += w.y;
+    }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-  }
+  if (PAIRS) warp_sum4(a, b);
+  else a = warp_sum2(a);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int nw = (blockDim.x + 31) >> 5;
+  // the caller's scratch holds 32 double2: pairs take two rounds of it
+  for (int which = 0; which < (PAIRS ? 2 : 1); ++which) {
+    __syncthreads();
+    if (lane == 0) red[w] = which == 0 ? a : b;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double2 t = make_double2(0.0, 0.0);
+      for (int i = 0; i < nw; ++i) { t.x += red[i].x; t.y += red[i].y; }
+      if (which == 0) a = t;
+      else b = t;
+    }
+  }
   __syncthreads();
-  if (lane == 0) red[w] = acc;
-  __syncthreads();
-  double2 s = make_double2(0.0, 0.0);
-  if (threadIdx.x == 0)
-    for (int i = 0; i < nw; ++i) { s.x += red[i].x; s.y += red[i].y; }
-  __syncthreads();
-  return s;
 }
 
 // Scalar update by the last block.  Partials hold one double2 per block
@@ -95,7 +108,8 @@ __device__ __forceinline__ double2 reduce_partials(const double2* partials, int 
 __device__ __forceinline__ void finalize(Scalars* sc, const double2* partials, int nparts, int fin,
                                          double2* red) {
   if (fin == FIN_ALPHA || fin == FIN_SUM) {
-    const double2 s = reduce_partials(partials, nparts, 1, 0, red);
+    double2 s, none;
+    reduce_partials<false>(partials, nparts, red, s, none);
     if (threadIdx.x == 0) {
       if (fin == FIN_SUM) {
         sc->sum = s;
@@ -114,8 +128,8 @@ __device__ __forceinline__ void finalize(Scalars* sc, const double2* partials, i
     }
     return;
   }
-  const double2 rr = reduce_partials(partials, nparts, 2, 0, red);
-  const double2 nn = reduce_partials(partials, nparts, 2, 1, red);
+  double2 rr, nn;
+  reduce_partials<true>(partials, nparts, red, rr, nn);
   if (threadIdx.x == 0) {
     const double rn2 = nn.x;
     if (fin == FIN_INIT) {

@@ -159,8 +159,7 @@ __global__ void k_build_ghatZ(const cpx<float>* __restrict__ g32, cpx<float>* gz
 // Reduction helper for the vector kernels: two double2 partials per block.
 __device__ __forceinline__ void block_partial2(double2 a, double2 b, double2* red,
                                                double2* partials) {
-  a = warp_sum2(a);
-  b = warp_sum2(b);
+  warp_sum4(a, b);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int nw = (blockDim.x + 31) >> 5;
   __syncthreads();
@@ -216,12 +215,16 @@ __global__ void k_rhs(const cpx<double>* __restrict__ rhs, const cpx<double>* __
     __syncthreads();
   }
   double acc = 0.0;
-  // blocks take whole lines (iz, iy): one index division per line, and the
-  // line's phase e_y e_z once per thread; threads run along x
-  for (int line = blockIdx.x; line < n * n; line += gridDim.x) {
+  // a block takes whole lines (iz, iy), several at a time when a line is
+  // shorter than the block (tx threads along x): one index division and the
+  // line's phase e_y e_z once per thread and line
+  int tx = 32;
+  while (tx < n && tx < int(blockDim.x)) tx *= 2;
+  const int rows = blockDim.x / tx, row = threadIdx.x / tx, x0 = threadIdx.x & (tx - 1);
+  for (int line = blockIdx.x * rows + row; line < n * n; line += gridDim.x * rows) {
     const int iz = line / n, iy = line - iz * n;
     const cpx<double> pyz = rhs == nullptr ? cmul(e[n + iy], e[2 * n + iz]) : cpx<double>{0.0, 0.0};
-    for (int ix = threadIdx.x; ix < n; ix += blockDim.x) {
+    for (int ix = x0; ix < n; ix += tx) {
       const long long i = (long long)line * n + ix;
       const cpx<double> u = rhs != nullptr ? rhs[i] : cmul(e[ix], pyz);
       if (u0 != nullptr) u0[i] = u;
