@@ -144,7 +144,7 @@ struct ori_plan_s {
   cpx<double>* d_phase = nullptr;  // 3n plane-wave phase factors per RHS
   double* d_dir = nullptr;         // 3 per RHS (plane waves)
   int* d_skip = nullptr;           // 1 = this RHS takes no part in a pass
-  double* h_small = nullptr;       // pinned: 7 * cap doubles
+  double* h_small = nullptr;       // pinned staging: kSmallSlots * cap doubles (SmallSlot)
   int* h_skip = nullptr;           // pinned: cap ints
   unsigned xinv_blocks = 0;        // largest X-inverse grid of the three arithmetics
   cudaStream_t ps = nullptr;       // private stream (capturable)
@@ -176,6 +176,12 @@ struct ori_plan_s {
   Pend* gpend_cur = nullptr;
   int* ngpend_cur = nullptr;
 };
+
+// Pinned staging of the per-RHS control values, one region (in units of cap
+// doubles) per value, so that the host fills one while the copy of another is
+// in flight: each region is filled again only after a read of the scalar
+// heads (a synchronisation) that followed its copy.
+enum SmallSlot { SLOT_TOLS = 0, SLOT_KV = 1, SLOT_DIR = 2, SLOT_INV = 5, SLOT_ACC = 6, SLOT_COEF = 7, kSmallSlots = 8 };
 
 static constexpr int kEvPool = 4096;
 static constexpr int kMaxVecCtasPerSm = 16;   // bound of ori_schedule.vec_ctas_per_sm
@@ -327,7 +333,7 @@ static ori_status ensure_capacity(ori_plan_s* p, int nrhs) {
   ORI_TRY(alloc_n(p, &p->d_phase, 3 * size_t(p->n) * c));
   ORI_TRY(alloc_n(p, &p->d_skip, c));
   if (cudaMallocHost(&p->h_sc, c * sizeof(Scalars)) != cudaSuccess ||
-      cudaMallocHost(&p->h_small, 7 * c * sizeof(double)) != cudaSuccess ||
+      cudaMallocHost(&p->h_small, size_t(kSmallSlots) * c * sizeof(double)) != cudaSuccess ||
       cudaMallocHost(&p->h_skip, c * sizeof(int)) != cudaSuccess)
     return fail(ORI_ERR_OOM, "cudaMallocHost failed");
   if (cudaHostGetDevicePointer(&p->h_sc_d, p->h_sc, 0) != cudaSuccess ||
@@ -1244,10 +1250,13 @@ struct InnerResult {
   double relres_recur = 0;
 };
 
-// Copy the scalar heads of all right-hand sides to the pinned mirror.
+// Copy the scalar heads of all right-hand sides and the fault flag to their
+// pinned mirrors (one launch) and wait for them.
 static ori_status read_heads(ori_plan_s* p, int nrhs) {
-  ORI_TRY(small_copy(p, p->h_sc_d, p->sc, offsetof(Scalars, hist), nrhs, sizeof(Scalars), sizeof(Scalars)));
-  ORI_TRY(small_copy(p, p->h_fault_d, p->d_fault, sizeof(int)));
+  k_read_heads<<<1, 256, 0, p->ps>>>(p->sc, nrhs, static_cast<unsigned long long*>(p->h_sc_d), p->d_fault,
+                                     static_cast<int*>(p->h_fault_d));
+  ORI_CUDA(cudaGetLastError());
+  launched(p);
   ORI_CUDA(cudaStreamSynchronize(p->ps));
   if (p->timing) t_harvest(p);
   return check_fault(p);
@@ -1279,7 +1288,6 @@ static ori_status cocg_inner(ori_plan_s* p, int nrhs, int rhs_per_k, cpx<T>* x, 
   ORI_VEC(p, ORI_PASS_VECTOR + (sizeof(T) == 4 ? 0 : ORI_PASS_FP64),
           (k_cocg_init<T><<<dim3(vg, nrhs), 256, 0, p->ps>>>(r, x, p->n3, p->sc, p->partials, p->d_tols, maxit,
                                                                zero_x ? 1 : 0)));
-  ORI_TRY(read_heads(p, nrhs));
   auto any_running = [&]() {
     for (int i = 0; i < nrhs; ++i)
       if (p->h_sc[i].done == DONE_RUNNING) return true;
@@ -1290,8 +1298,7 @@ static ori_status cocg_inner(ori_plan_s* p, int nrhs, int rhs_per_k, cpx<T>* x, 
     for (int i = 0; i < nrhs; ++i) m = std::max(m, p->h_sc[i].iter);
     return m;
   };
-  int graph_iters_total = 0;
-  if (any_running() && maxit > 0) {
+  if (maxit > 0) {   // a system that needs no iteration is flagged by k_cocg_init: its kernels return at once
     ORI_TRY(cocg_iteration<T>(p, nrhs, rhs_per_k, x, r, pp, q, S, true));
     const bool f32 = sizeof(T) == 4;
     cudaGraphExec_t& gexec = f32 ? p->graph_f : p->graph_d;
@@ -1330,30 +1337,28 @@ static ori_status cocg_inner(ori_plan_s* p, int nrhs, int rhs_per_k, cpx<T>* x, 
       gtimed = p->timing;
       gkern = p->cap_launches;
     }
+    // the first block goes out behind the first iteration without a look at
+    // the flags: a system that has converged by then leaves its kernels at once
     int launched_iters = 1;
-    bool graph_pending = false;
-    int iter_before = 0;
-    for (;;) {
-      ORI_TRY(read_heads(p, nrhs));
-      const int it_now = max_iter();
-      if (graph_pending) {
-        graph_iters_total += it_now - iter_before;
-        if (p->timing) t_harvest_graph(p, gpend, ngpend, it_now - iter_before);
-      }
-      iter_before = it_now;
-      graph_pending = false;
-      if (!any_running() || launched_iters >= maxit) break;
+    int iter_before = 1;
+    while (launched_iters < maxit) {
       if (use_graph) {
         ORI_CUDA(cudaGraphLaunch(gexec, p->ps));
         p->stats.kernel_launches += gkern;
-        graph_pending = true;
       } else {
         for (int i = 0; i < check_every; ++i) ORI_TRY(cocg_iteration<T>(p, nrhs, rhs_per_k, x, r, pp, q, S, false));
       }
       launched_iters += check_every;
+      ORI_TRY(read_heads(p, nrhs));
+      const int it_now = max_iter();
+      if (use_graph && p->timing) t_harvest_graph(p, gpend, ngpend, std::max(0, it_now - iter_before));
+      iter_before = it_now;
+      if (!any_running()) break;
     }
+    if (launched_iters == 1) ORI_TRY(read_heads(p, nrhs));
+  } else {
+    ORI_TRY(read_heads(p, nrhs));
   }
-  ORI_TRY(read_heads(p, nrhs));
   long long real_matvecs = 0;
   for (int i = 0; i < nrhs; ++i) {
     res[i].iters = p->h_sc[i].iter;
@@ -1367,7 +1372,6 @@ static ori_status cocg_inner(ori_plan_s* p, int nrhs, int rhs_per_k, cpx<T>* x, 
   } else {
     p->stats.fp64_matvecs += real_matvecs;
   }
-  (void)graph_iters_total;
   return ORI_OK;
 }
 
@@ -1418,12 +1422,10 @@ static ori_status push_skip(ori_plan_s* p, int nrhs) {
   ORI_TRY(small_copy(p, p->d_skip, p->h_skip_d, nrhs * sizeof(int)));
   return ORI_OK;
 }
-static ori_status push_doubles(ori_plan_s* p, double* dst, const double* src, int count) {
-  double* stage = p->h_small + 3 * p->cap;   // pinned staging beyond the tolerance slots
-  for (int i = 0; i < count; ++i) stage[i] = src[i];
-  ORI_TRY(small_copy(p, dst, static_cast<double*>(p->h_small_d) + 3 * p->cap, count * sizeof(double)));
-  ORI_CUDA(cudaStreamSynchronize(p->ps));
-  return ORI_OK;
+static ori_status push_doubles(ori_plan_s* p, double* dst, const double* src, int count, SmallSlot slot) {
+  const size_t off = size_t(slot) * size_t(p->cap);
+  for (int i = 0; i < count; ++i) p->h_small[off + i] = src[i];
+  return small_copy(p, dst, static_cast<double*>(p->h_small_d) + off, count * sizeof(double));
 }
 
 // Append COCG's recursive residual after each iteration of the last inner run
@@ -1548,7 +1550,7 @@ static ori_status solve_B(ori_plan_s* p, int nrhs, int rhs_per_k, const double* 
       tin[i] = active[i] ? std::min(0.5, std::max(o.inner_tol, want)) : 1.0;
     }
     if (budget <= 0) break;
-    ORI_TRY(push_doubles(p, p->d_scl, inv.data(), nrhs));
+    ORI_TRY(push_doubles(p, p->d_scl, inv.data(), nrhs, SLOT_INV));
     const int vg = vgrid(p, nrhs);
     ORI_VEC(p, ORI_PASS_VECTOR, (k_normalise_to_f32<<<dim3(vg, nrhs), 256, 0, p->ps>>>(p->r64, p->r32, n3, p->d_scl)));
     ORI_TRY(cocg_inner<float>(p, nrhs, rhs_per_k, p->x32, p->r32, p->p32, p->q32, p->S32, tin.data(), budget,
@@ -1567,7 +1569,7 @@ static ori_status solve_B(ori_plan_s* p, int nrhs, int rhs_per_k, const double* 
       scl[i] = active[i] ? rn[i] : 0.0;
     }
     if (nonfinite_all) break;
-    ORI_TRY(push_doubles(p, p->d_scl, scl.data(), nrhs));
+    ORI_TRY(push_doubles(p, p->d_scl, scl.data(), nrhs, SLOT_ACC));
     ORI_VEC(p, ORI_PASS_VECTOR, (k_accumulate<<<dim3(vg, nrhs), 256, 0, p->ps>>>(p->w, p->x32, n3, p->d_scl)));
     // residual: updated with the FP32 operator when every active RHS allows it
     bool upd = o.resid_update != 0;
@@ -1582,7 +1584,7 @@ static ori_status solve_B(ori_plan_s* p, int nrhs, int rhs_per_k, const double* 
     std::vector<double> rn_new(rn);
     if (upd) {
       // r -= rn B d with the FP32 operator; error <= kFp32OperatorRelErr rn |B d|
-      ORI_TRY(push_doubles(p, p->d_coef, scl.data(), nrhs));
+      ORI_TRY(push_doubles(p, p->d_coef, scl.data(), nrhs, SLOT_COEF));
       const long long bs32 = n3 * (long long)sizeof(cpx<float>), bs64 = n3 * (long long)sizeof(cpx<double>);
       XArgs pro{}, epi{};
       pro.mode = PRO_SCALE;
@@ -1675,8 +1677,8 @@ static ori_status solve_batch(ori_plan_s* p, int nk, int ndir, const double* rhs
       const double an = std::sqrt(a[0] * a[0] + a[1] * a[1] + a[2] * a[2]);
       for (int c = 0; c < 3; ++c) dv[3 * r + c] = an > 0 ? a[c] / an : (c == 2 ? 1.0 : 0.0);
     }
-  ORI_TRY(push_doubles(p, p->d_kv, kv.data(), nrhs));
-  ORI_TRY(push_doubles(p, p->d_dir, dv.data(), 3 * nrhs));
+  ORI_TRY(push_doubles(p, p->d_kv, kv.data(), nrhs, SLOT_KV));
+  ORI_TRY(push_doubles(p, p->d_dir, dv.data(), 3 * nrhs, SLOT_DIR));
   const int vg = vgrid(p, nrhs);
   ORI_VEC(p, ORI_PASS_VECTOR,
           (k_phases<<<dim3(unsigned((3 * p->n + 255) / 256), nrhs), 256, 0, p->ps>>>(

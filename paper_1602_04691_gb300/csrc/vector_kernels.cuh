@@ -4,6 +4,8 @@
 // the mixed-precision refinement steps and the adjoint gradient.
 #pragma once
 
+#include <cstddef>
+
 #include "common.cuh"
 #include "dfloat.cuh"
 #include "passes.cuh"
@@ -99,6 +101,20 @@ __global__ void k_small_copy(const unsigned char* src, unsigned char* dst, long 
       for (long long i = threadIdx.x; i < bytes; i += blockDim.x) dr[i] = sr[i];
     }
   }
+}
+
+// The scalar heads (everything before the history) of nrhs systems and the
+// fault flag, to their mapped mirrors: what the host reads between launches,
+// in one launch.  The mirror of the heads keeps the stride of Scalars.
+__global__ void k_read_heads(const Scalars* sc, int nrhs, unsigned long long* out, const int* fault, int* out_fault) {
+  constexpr int W = int(offsetof(Scalars, hist) / 8), STRIDE = int(sizeof(Scalars) / 8);
+  static_assert(offsetof(Scalars, hist) % 8 == 0 && sizeof(Scalars) % 8 == 0, "whole words");
+  const unsigned long long* in = reinterpret_cast<const unsigned long long*>(sc);
+  for (int i = threadIdx.x; i < nrhs * W; i += blockDim.x) {
+    const int r = i / W, w = i - r * W;
+    out[(long long)r * STRIDE + w] = in[(long long)r * STRIDE + w];
+  }
+  if (threadIdx.x == 0) *out_fault = *fault;
 }
 
 // dst = src for n16 16-byte words of device memory (an SM copy, for the same
