@@ -982,6 +982,11 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
     p->M = spec_M ? spec_M : (o.min_L ? std::max(p->L, o.min_L) : transform_length(p->n, p->L));
     p->L = std::max(p->L, o.min_L);
     p->H = p->M / 2 + 1;
+    // default launch variants: at L = 256 and 1024 the (2 L1) x (L2 / 2) split
+    // was the faster one in all three passes (n = 512: 7.05 -> 6.85 ms an
+    // operator, n = 128: 0.129 -> 0.117 ms), at L = 512 the square-most one
+    // (n = 256: 0.832 against 0.870 ms)
+    if (p->M == 256 || p->M == 1024) p->var_y = p->var_z = p->var_yi = 2;
     p->n3 = (long long)n * n * n;
     p->ks = ks;
     p->side = dom->side;
