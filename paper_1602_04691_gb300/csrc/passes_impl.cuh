@@ -854,7 +854,7 @@ __global__ void __launch_bounds__(Tile<L, C, T>::NT) k_strided(SArgs a0) {
 // ---------------------------------------------------------------------------
 template <int L, int C, class T>
 struct LSmem {
-  static constexpr int NT = C >= 4 ? 256 : 64 * C;
+  static constexpr int NT = is_mixed_len(L) ? stage_threads<L>(C, C >= 4 ? 256 : 160) : (C >= 4 ? 256 : 64 * C);
   static constexpr int MINB = C >= 4 ? 2 : 4;       // narrow tiles: more independent CTAs per SM
   static constexpr size_t X_ELEMS = size_t(L) * C;
   static constexpr size_t SMEM_BYTES = (X_ELEMS + size_t(L)) * sizeof(cpx<T>);
@@ -896,17 +896,24 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_st
       for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
     }
     __syncthreads();
-    dif_rest<L, C>(X, TW, tid, NT);
-    for (int e = tid; e < C * L; e += NT) {
-      const int c = e % C, p = e / C;
-      const int k = digit_rev<L>(p);
-      if (c < colmax && k < a.n_out) out[(long long)k * a.out_pt + c] = ld_stage(X + sidx<C>(p, c));
+    dif_middle<L, C>(X, TW, tid, NT);
+    constexpr int r3 = SRad<L>::r3;
+    for (int g = tid; g < C * (L / r3); g += NT) {
+      const int c = g % C, blk = g / C;
+      cpx<T> v[r3];
+      dif_last<L, C, -1>(X, blk, c, v);
+      const int k0 = freq_of_block<L>(blk);
+#pragma unroll
+      for (int t = 0; t < r3; ++t) {
+        const int k = k0 + (L / r3) * t;
+        if (c < colmax && k < a.n_out) out[(long long)k * a.out_pt + c] = settle(v[t]);
+      }
     }
   } else {
     // the inverse by decimation in frequency with the inverse sign: the first
     // radix-8 stage reads the L input rows in natural order from global
-    // memory, the others run in shared memory, and the n_out kept rows are
-    // gathered from their digit-reversed positions
+    // memory, the middle one runs in shared memory, and the last stores the
+    // n_out kept rows
     __syncthreads();
     for (int g = tid; g < C * S8; g += NT) {
       const int c = g % C, j = g / C;
@@ -923,10 +930,18 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_st
       for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
     }
     __syncthreads();
-    dif_rest<L, C, +1>(X, TW, tid, NT);
-    for (int e = tid; e < C * a.n_out; e += NT) {
-      const int c = e % C, z = e / C;
-      if (c < colmax) out[(long long)z * a.out_pt + c] = ld_stage(X + sidx<C>(inv_digit_rev<L>(z), c));
+    dif_middle<L, C, +1>(X, TW, tid, NT);
+    constexpr int r3 = SRad<L>::r3;
+    for (int g = tid; g < C * (L / r3); g += NT) {
+      const int c = g % C, blk = g / C;
+      cpx<T> v[r3];
+      dif_last<L, C, +1>(X, blk, c, v);
+      const int k0 = freq_of_block<L>(blk);
+#pragma unroll
+      for (int t = 0; t < (r3 + 1) / 2; ++t) {   // n_out <= L/2
+        const int k = k0 + (L / r3) * t;
+        if (c < colmax && k < a.n_out) out[(long long)k * a.out_pt + c] = settle(v[t]);
+      }
     }
   }
 }
@@ -962,21 +977,28 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_xf
     for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
   }
   __syncthreads();
-  dif_rest<L, C>(X, TW, tid, NT);
+  dif_middle<L, C>(X, TW, tid, NT);
   cpx<T>* out = reinterpret_cast<cpx<T>*>(a.fft_out);
-  for (int e = tid; e < C * L; e += NT) {
-    const int k = e % L, c = e / L;
+  // last stage: consecutive threads take consecutive frequencies, so the stores coalesce
+  constexpr int r3 = SRad<L>::r3, B = L / r3;
+  for (int g = tid; g < C * B; g += NT) {
+    const int k0 = g % B, c = g / B;
     const long long line = (long long)blockIdx.x * C + c;
-    if (line < a.nlines) out[line * a.line_len_out + k] = ld_stage(X + sidx<C>(inv_digit_rev<L>(k), c));
+    cpx<T> v[r3];
+    dif_last<L, C, -1>(X, block_of_freq<L>(k0), c, v);
+    if (line < a.nlines) {
+#pragma unroll
+      for (int t = 0; t < r3; ++t) out[line * a.line_len_out + k0 + B * t] = settle(v[t]);
+    }
   }
 }
 
 // The inverse X transform runs by decimation in frequency with the inverse
 // sign: its first radix-8 stage takes each line's L points in natural order
 // straight from global memory (eight independent coalesced loads per thread,
-// no scattered shared-memory stores), the remaining stages run in shared
-// memory, and the epilogue gathers the n kept points x < n from their
-// digit-reversed positions, so its own global reads and writes are coalesced.
+// no scattered shared-memory stores), the middle stage runs in shared memory,
+// and the last one feeds the epilogue with the kept points x < n, consecutive
+// threads taking consecutive x, so its global reads and writes are coalesced.
 template <class T, int L, int C>
 __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_xinv_smem(XArgs a0, Scalars* sc0, int fin) {
   const XArgs a = x_for_rhs(a0, blockIdx.y);
@@ -1007,13 +1029,22 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_xi
     for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
   }
   __syncthreads();
-  dif_rest<L, C, +1>(X, TW, tid, NT);
+  dif_middle<L, C, +1>(X, TW, tid, NT);
   double2 acc = make_double2(0.0, 0.0);
   cpx<T> accT = czero<T>();
-  for (int e = tid; e < C * a.n; e += NT) {
-    const int x = e % a.n, c = e / a.n;
+  constexpr int r3 = SRad<L>::r3, B = L / r3;
+  for (int g = tid; g < C * B; g += NT) {
+    const int k0 = g % B, c = g / B;
     const long long line = (long long)blockIdx.x * C + c;
-    if (line < a.nlines) x_epilogue<T>(a, line * a.n + x, ld_stage(X + sidx<C>(inv_digit_rev<L>(x), c)), accT, acc);
+    cpx<T> v[r3];
+    dif_last<L, C, +1>(X, block_of_freq<L>(k0), c, v);
+    if (line < a.nlines) {
+#pragma unroll
+      for (int t = 0; t < (r3 + 1) / 2; ++t) {   // x < n <= L/2
+        const int x = k0 + B * t;
+        if (x < a.n) x_epilogue<T>(a, line * a.n + x, settle(v[t]), accT, acc);
+      }
+    }
   }
   const cpx<double> accD = c_to_c64(accT);
   acc.x += accD.x;
@@ -1705,11 +1736,15 @@ cudaError_t launch_zconv_mix_L(SArgs a, cudaStream_t s, bool setup, int sm_count
 // ---------------------------------------------------------------------------
 template <int L, int C, class T>
 struct ZSmem {
-  static constexpr int NT = 512;
-  static constexpr int MINB = 1;   // (256 threads, two CTAs per SM measured 9% slower at L = 2048)
   static constexpr size_t X_ELEMS = size_t(L) * C;
   static constexpr size_t S_ELEMS = size_t(L / 2) * C;
   static constexpr size_t SMEM_BYTES = (X_ELEMS + S_ELEMS + size_t(L)) * sizeof(cpx<T>);
+  // one CTA per SM where shared memory holds no more (256 threads, two CTAs
+  // per SM measured 9% slower at L = 2048), else two CTAs of half the threads,
+  // whose phases overlap
+  static constexpr bool TWO = SMEM_BYTES + 1024 <= 114 * 1024;
+  static constexpr int NT = is_mixed_len(L) ? stage_threads<L>(C, TWO ? 256 : 512) : (TWO ? 256 : 512);
+  static constexpr int MINB = TWO ? 2 : 1;
 };
 
 template <class T, int L, int C>
@@ -1757,18 +1792,26 @@ __global__ void __launch_bounds__(ZSmem<L, C, T>::NT, ZSmem<L, C, T>::MINB) k_zc
     }
     __syncthreads();
     if (next < ntiles) zpipe_prefetch_rows<T, L, C, NT>(a, next, per_rhs, S);
-    dif_rest<L, C>(X, TW, tid, NT);
-    // spectrum: position p holds frequency kz = digit_rev(p)
+    dif_middle<L, C>(X, TW, tid, NT);
+    // last forward stage, spectrum and first inverse stage on the same r3 points
     const int my = mirror_index(ky, L);
-    for (int e = tid; e < C * L; e += NT) {
-      const int c = e % C, p = e / C;
-      const int mz = mirror_index(digit_rev<L>(p), L);
+    constexpr int r3 = SRad<L>::r3;
+    for (int g = tid; g < C * (L / r3); g += NT) {
+      const int c = g % C, blk = g / C;
       const int mx = mirror_index(cb * C + c, L);
-      const int si = sidx<C>(p, c);
-      st_stage(X + si, settle(cmul(ld_stage(X + si), ldgc(gh + ((long long)mz * a.H + my) * a.H + mx))));
+      const int k0 = freq_of_block<L>(blk);
+      const cpx<T>* gp = gh + (long long)my * a.H + mx;
+      cpx<T> v[r3];
+      dif_last<L, C, -1>(X, blk, c, v);
+#pragma unroll
+      for (int t = 0; t < r3; ++t)
+        v[t] = settle(cmul(v[t], ldgc(gp + (long long)mirror_index(k0 + (L / r3) * t, L) * a.H * a.H)));
+      dft<r3, +1, false>(v);
+#pragma unroll
+      for (int t = 0; t < r3; ++t) st_stage(X + sidx<C>(blk * r3 + t, c), settle(v[t]));
     }
     __syncthreads();
-    dit_head<L, C>(X, TW, tid, NT);
+    dit_middle<L, C>(X, TW, tid, NT);
     // last inverse stage (M = L), keep rows z < n_out
     cpx<T>* out = reinterpret_cast<cpx<T>*>(bmove(a.out, a.bs_out * rhs)) + (long long)ky * a.out_outer + (long long)cb * C;
     for (int g = tid; g < C * S8; g += NT) {
