@@ -1287,7 +1287,7 @@ static ori_status cocg_iteration(ori_plan_s* p, int nrhs, int rhs_per_k, cpx<T>*
   ORI_TRY(run_conv<T>(p, pro, epi, FIN_ALPHA, p->ps, Mask{&p->sc->done, int(sizeof(Scalars))}, nrhs, rhs_per_k));
   const int vg = vgrid_sum(p, nrhs);
   ORI_VEC(p, ORI_PASS_UPDATE + (sizeof(T) == 4 ? 0 : ORI_PASS_FP64),
-          (k_cocg_update<T><<<dim3(vg, nrhs), 256, 0, p->ps>>>(x, pp, r, q, p->n3, p->sc, p->partials)));
+          (launch_dep(k_cocg_update<T>, dim3(vg, nrhs), 256, 0, p->ps, x, pp, r, q, p->n3, p->sc, p->partials)));
   return ORI_OK;
 }
 

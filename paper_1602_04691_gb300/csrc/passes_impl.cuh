@@ -172,6 +172,7 @@ __device__ __forceinline__ cpx<T> x_prologue(const XArgs& a, long long line, int
 // ---------------------------------------------------------------------------
 template <class T, int L, int C, bool HALF>
 __global__ void __launch_bounds__(Tile<L, C, T>::NT, Tile<L, C, T>::MINB) k_xfwd(XArgs a0) {
+  dep_wait();
   const XArgs a = x_for_rhs(a0, blockIdx.y);
   using TL = Tile<L, C, T>;
   constexpr int L1 = TL::L1, L2 = TL::L2, NT = TL::NT;
@@ -273,8 +274,9 @@ __global__ void __launch_bounds__(XFwdPipe<L, C>::NT, L > 1024 ? 1 : 2) k_xfwd_p
   cpx<T>* P = R + XP::STAGE / 3;
   cpx<T>* G = P + XP::STAGE / 3;
   cpx<T>* TW = G + XP::STAGE / 3;
-  if (a.done != nullptr && *a.done != 0) return;
   fill_tw2<L>(TW, reinterpret_cast<const cpx<T>*>(a.twL), threadIdx.x, NT);   // [k1][j] layout
+  dep_wait();
+  if (a.done != nullptr && *a.done != 0) return;
   const int tid = threadIdx.x;
   const int ntiles = int((a.nlines + C - 1) / C);
   const cpx<T> beta = x_beta<T>(a);
@@ -406,6 +408,7 @@ __device__ __forceinline__ void x_epilogue(const XArgs& a, long long i, cpx<T> v
 // ---------------------------------------------------------------------------
 template <class T, int L, int C>
 __global__ void __launch_bounds__(Tile<L, C, T>::NT, Tile<L, C, T>::MINB) k_xinv(XArgs a0, Scalars* sc0, int fin) {
+  dep_wait();
   const XArgs a = x_for_rhs(a0, blockIdx.y);
   Scalars* sc = sc0 == nullptr ? nullptr : sc0 + blockIdx.y;
   using TL = Tile<L, C, T>;
@@ -541,6 +544,7 @@ template <int L, int C>
 __global__ void __launch_bounds__(XInvPipe<L, C>::NT, L > 1024 ? 1 : 3) k_xinv_pipe(XArgs a0, Scalars* sc0, int fin) {
   using T = float;
   using XP = XInvPipe<L, C>;
+  dep_wait();
   const XArgs a = x_for_rhs(a0, blockIdx.y);
   Scalars* sc = sc0 == nullptr ? nullptr : sc0 + blockIdx.y;
   using TL = Tile<L, C, T>;
@@ -735,6 +739,7 @@ __device__ __forceinline__ int mirror_index(int k, int L) { return k <= L / 2 ? 
 
 template <class T, int L, int C, int SMODE, bool HALF>
 __global__ void __launch_bounds__(Tile<L, C, T>::NT) k_strided(SArgs a0) {
+  dep_wait();
   const SArgs a = s_for_rhs(a0, blockIdx.y);
   using TL = Tile<L, C, T>;
   constexpr int L1 = TL::L1, L2 = TL::L2, NT = TL::NT;
@@ -868,10 +873,11 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_st
   extern __shared__ __align__(16) unsigned char smraw[];
   cpx<T>* X = reinterpret_cast<cpx<T>*>(smraw);
   cpx<T>* TW = X + LS::X_ELEMS;
-  if (a.done != nullptr && *a.done != 0) return;
   const cpx<T>* twg = reinterpret_cast<const cpx<T>*>(a.twL);
   const int tid = threadIdx.x;
   for (int i = tid; i < L; i += NT) TW[i] = twg[i];
+  dep_wait();
+  if (a.done != nullptr && *a.done != 0) return;
   const int outer = blockIdx.x / a.col_blocks;
   const int cb = blockIdx.x - outer * a.col_blocks;
   const cpx<T>* in = reinterpret_cast<const cpx<T>*>(a.in) + outer * a.in_outer + (long long)cb * C;
@@ -954,10 +960,11 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_xf
   extern __shared__ __align__(16) unsigned char smraw[];
   cpx<T>* X = reinterpret_cast<cpx<T>*>(smraw);
   cpx<T>* TW = X + LS::X_ELEMS;
-  if (a.done != nullptr && *a.done != 0) return;
   const cpx<T>* twg = reinterpret_cast<const cpx<T>*>(a.twL);
   const int tid = threadIdx.x;
   for (int i = tid; i < L; i += NT) TW[i] = twg[i];
+  dep_wait();
+  if (a.done != nullptr && *a.done != 0) return;
   __syncthreads();
   const cpx<T> beta = x_beta<T>(a);
   // first stage: consecutive threads take consecutive points of one line
@@ -1001,6 +1008,7 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_xf
 // threads taking consecutive x, so its global reads and writes are coalesced.
 template <class T, int L, int C>
 __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_xinv_smem(XArgs a0, Scalars* sc0, int fin) {
+  dep_wait();
   const XArgs a = x_for_rhs(a0, blockIdx.y);
   Scalars* sc = sc0 == nullptr ? nullptr : sc0 + blockIdx.y;
   using LS = LSmem<L, C, T>;
@@ -1081,8 +1089,7 @@ cudaError_t launch_xfwd_pipe_L(const XArgs& a, cudaStream_t s, bool setup) {
   const long long ntiles = (a.nlines + C - 1) / C;
   const int nb = std::max(1, a.nrhs);
   const unsigned gx = unsigned(std::max(1LL, std::min(ntiles, (long long)std::max(1, a.sm_count) * std::max(1, per_sm) / nb)));
-  kfn<<<dim3(gx, unsigned(nb)), XP::NT, XP::SMEM_BYTES, s>>>(a);
-  return cudaGetLastError();
+  return launch_dep(kfn, dim3(gx, unsigned(nb)), XP::NT, XP::SMEM_BYTES, s, a);
 }
 
 // The pipelined kernel serves the solver's prologues on whole contiguous lines
@@ -1108,16 +1115,14 @@ cudaError_t launch_xfwd_reg_L(const XArgs& a, cudaStream_t s, bool setup) {
     using LS = LSmem<L, CS, T>;
     auto kfs = k_xfwd_smem<T, L, CS>;
     if (setup) return cudaFuncSetAttribute(kfs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LS::SMEM_BYTES));
-    kfs<<<dim3(unsigned((a.nlines + CS - 1) / CS), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s>>>(a);
-    return cudaGetLastError();
+    return launch_dep(kfs, dim3(unsigned((a.nlines + CS - 1) / CS), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s, a);
   }
   constexpr int C = lines_contig<T, L>();
   using TL = Tile<L, C, T>;
   auto kfn = k_xfwd<T, L, C, HALF>;
   if (setup) return cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(TL::SMEM_BYTES));
   const dim3 grid(unsigned((a.nlines + C - 1) / C), unsigned(std::max(1, a.nrhs)));
-  kfn<<<grid, TL::NT, TL::SMEM_BYTES, s>>>(a);
-  return cudaGetLastError();
+  return launch_dep(kfn, dim3(grid), TL::NT, TL::SMEM_BYTES, s, a);
 }
 
 template <int L>
@@ -1140,8 +1145,7 @@ cudaError_t launch_xinv_pipe_L(const XArgs& a, Scalars* sc, int fin, cudaStream_
   const int nb = std::max(1, a.nrhs);
   const unsigned gx = unsigned(std::max(1LL, std::min(ntiles, (long long)std::max(1, a.sm_count) * std::max(1, per_sm) / nb)));
   if (nblocks) *nblocks = gx;
-  kfn<<<dim3(gx, unsigned(nb)), XP::NT, XP::SMEM_BYTES, s>>>(a, sc, fin);
-  return cudaGetLastError();
+  return launch_dep(kfn, dim3(gx, unsigned(nb)), XP::NT, XP::SMEM_BYTES, s, a, sc, fin);
 }
 
 template <class T, int L>
@@ -1155,8 +1159,7 @@ cudaError_t launch_xinv_reg_L(const XArgs& a, Scalars* sc, int fin, cudaStream_t
     const unsigned grid = unsigned((a.nlines + CS - 1) / CS);
     if (nblocks) *nblocks = grid;
     if (setup) return cudaFuncSetAttribute(kfs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LS::SMEM_BYTES));
-    kfs<<<dim3(grid, unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s>>>(a, sc, fin);
-    return cudaGetLastError();
+    return launch_dep(kfs, dim3(grid, unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s, a, sc, fin);
   } else {
     constexpr int C = lines_contig<T, L>();
     using TL = Tile<L, C, T>;
@@ -1164,8 +1167,7 @@ cudaError_t launch_xinv_reg_L(const XArgs& a, Scalars* sc, int fin, cudaStream_t
     const unsigned grid = unsigned((a.nlines + C - 1) / C);
     if (nblocks) *nblocks = grid;
     if (setup) return cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(TL::SMEM_BYTES));
-    kfn<<<dim3(grid, unsigned(std::max(1, a.nrhs))), TL::NT, TL::SMEM_BYTES, s>>>(a, sc, fin);
-    return cudaGetLastError();
+    return launch_dep(kfn, dim3(grid, unsigned(std::max(1, a.nrhs))), TL::NT, TL::SMEM_BYTES, s, a, sc, fin);
   }
 }
 
@@ -1203,8 +1205,7 @@ cudaError_t launch_strided_reg_L(SArgs a, cudaStream_t s, bool setup) {
     auto kfs = k_strided_smem<T, L, CS, SMODE>;
     if (setup) return cudaFuncSetAttribute(kfs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LS::SMEM_BYTES));
     a.col_blocks = (a.ncols + CS - 1) / CS;
-    kfs<<<dim3(unsigned(a.nouter) * unsigned(a.col_blocks), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s>>>(a);
-    return cudaGetLastError();
+    return launch_dep(kfs, dim3(unsigned(a.nouter) * unsigned(a.col_blocks), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s, a);
   }
   constexpr int C = cols_strided<T>();
   using TL = Tile<L, C, T>;
@@ -1212,8 +1213,7 @@ cudaError_t launch_strided_reg_L(SArgs a, cudaStream_t s, bool setup) {
   if (setup) return cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(TL::SMEM_BYTES));
   a.col_blocks = (a.ncols + C - 1) / C;
   const dim3 grid(unsigned(a.nouter) * unsigned(a.col_blocks), unsigned(std::max(1, a.nrhs)));
-  kfn<<<grid, TL::NT, TL::SMEM_BYTES, s>>>(a);
-  return cudaGetLastError();
+  return launch_dep(kfn, dim3(grid), TL::NT, TL::SMEM_BYTES, s, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -1427,6 +1427,7 @@ k_zconv_pipe(const __grid_constant__ SArgs a) {
     zpipe_prefetch<T, L, C, L1X>(a, t, per_rhs, S);
   };
 
+  dep_wait();
   int tile = next_live_tile(a, blockIdx.x, step, per_rhs, ntiles);
   if (tile < ntiles) stage_rows(tile);
   while (tile < ntiles) {
@@ -1639,6 +1640,7 @@ __global__ void __launch_bounds__(ZMix<L>::NT, ZMix<L>::MINB) k_zconv_mix(const 
     }
   };
 
+  dep_wait();
   int tile = next_live_tile(a, blockIdx.x, step, per_rhs, ntiles);
   if (tile < ntiles) stage_rows(tile);
   while (tile < ntiles) {
@@ -1724,8 +1726,7 @@ cudaError_t launch_zconv_mix_L(SArgs a, cudaStream_t s, bool setup, int sm_count
   const long long ntiles = (long long)L * (L / Z::C) * std::max(1, a.nrhs);
   const int resident = a.cta_cap > 0 ? std::min(std::max(1, per_sm), a.cta_cap) : std::max(1, per_sm);
   const unsigned gx = unsigned(std::max(1LL, std::min(ntiles, (long long)std::max(1, sm_count) * resident)));
-  kfn<<<gx, Z::NT, Z::SMEM_BYTES, s>>>(a);
-  return cudaGetLastError();
+  return launch_dep(kfn, dim3(gx), Z::NT, Z::SMEM_BYTES, s, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -1764,6 +1765,7 @@ __global__ void __launch_bounds__(ZSmem<L, C, T>::NT, ZSmem<L, C, T>::MINB) k_zc
   const int step = gridDim.x;
   const int tid = threadIdx.x;
 
+  dep_wait();
   int tile = next_live_tile(a, blockIdx.x, step, per_rhs, ntiles);
   if (tile < ntiles) zpipe_prefetch_rows<T, L, C, NT>(a, tile, per_rhs, S);
   while (tile < ntiles) {
@@ -1849,8 +1851,7 @@ cudaError_t launch_zconv_smem_L(SArgs a, cudaStream_t s, bool setup, int sm_coun
   }
   const long long ntiles = (long long)L * (L / C) * std::max(1, a.nrhs);
   const unsigned gx = unsigned(std::max(1LL, std::min(ntiles, (long long)std::max(1, sm_count) * std::max(1, per_sm))));
-  kfn<<<gx, ZS::NT, ZS::SMEM_BYTES, s>>>(a);
-  return cudaGetLastError();
+  return launch_dep(kfn, dim3(gx), ZS::NT, ZS::SMEM_BYTES, s, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -1950,6 +1951,7 @@ k_yfwd_pipe(const __grid_constant__ SArgs a) {
     }
     ypipe_prefetch<T, L, C, L1X>(a, t, per_rhs, S);
   };
+  dep_wait();
   int tile = next_live_tile(a, blockIdx.x, step, per_rhs, ntiles);
   if (tile < ntiles) stage(tile);
   while (tile < ntiles) {
@@ -2088,6 +2090,7 @@ k_yinv_pipe(const __grid_constant__ SArgs a) {
     }
     yinv_prefetch<L, C, L1X>(a, t, per_rhs, B);
   };
+  dep_wait();
   int tile = next_live_tile(a, blockIdx.x, step, per_rhs, ntiles);
   if (tile < ntiles) stage(tile);
   while (tile < ntiles) {
@@ -2164,8 +2167,7 @@ cudaError_t launch_yinv_pipe_V(SArgs a, cudaStream_t s, bool setup, int sm_count
   const long long ntiles = (long long)a.nouter * a.col_blocks * std::max(1, a.nrhs);
   const int resident = a.cta_cap > 0 ? std::min(std::max(1, per_sm), a.cta_cap) : std::max(1, per_sm);
   const unsigned gx = unsigned(std::max(1LL, std::min(ntiles, (long long)std::max(1, sm_count) * resident)));
-  kfn<<<gx, YP::NT, YP::SMEM_BYTES, s>>>(a);
-  return cudaGetLastError();
+  return launch_dep(kfn, dim3(gx), YP::NT, YP::SMEM_BYTES, s, a);
 }
 
 template <class T, int L, int C, int L1X>
@@ -2185,8 +2187,7 @@ cudaError_t launch_yfwd_pipe_V(SArgs a, cudaStream_t s, bool setup, int sm_count
   const long long ntiles = (long long)a.nouter * a.col_blocks * std::max(1, a.nrhs);
   const int resident = a.cta_cap > 0 ? std::min(std::max(1, per_sm), a.cta_cap) : std::max(1, per_sm);
   const unsigned gx = unsigned(std::max(1LL, std::min(ntiles, (long long)std::max(1, sm_count) * resident)));
-  kfn<<<gx, YP::NT, YP::SMEM_BYTES, s>>>(a);
-  return cudaGetLastError();
+  return launch_dep(kfn, dim3(gx), YP::NT, YP::SMEM_BYTES, s, a);
 }
 
 template <class T, int L, int C, int L1X>
@@ -2205,8 +2206,7 @@ cudaError_t launch_zconv_pipe_V(SArgs a, cudaStream_t s, bool setup, int sm_coun
   const long long ntiles = (long long)L * (L / C) * std::max(1, a.nrhs);
   const int resident = a.cta_cap > 0 ? std::min(std::max(1, per_sm), a.cta_cap) : std::max(1, per_sm);
   const unsigned gx = unsigned(std::max(1LL, std::min(ntiles, (long long)std::max(1, sm_count) * resident)));
-  kfn<<<gx, ZP::NT, ZP::SMEM_BYTES, s>>>(a);
-  return cudaGetLastError();
+  return launch_dep(kfn, dim3(gx), ZP::NT, ZP::SMEM_BYTES, s, a);
 }
 
 // Dispatch on the launch variant (has_pipe_variants): the set-up call
@@ -2309,16 +2309,14 @@ cudaError_t launch_xfwd_mix_L(const XArgs& a, cudaStream_t s, bool setup) {
         return cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(TL::SMEM_BYTES));
       }
       if (xfwd_pipe_ok(a, L)) return launch_xfwd_pipe_L<L>(a, s, false);
-      kfn<<<dim3(unsigned((a.nlines + C - 1) / C), unsigned(std::max(1, a.nrhs))), TL::NT, TL::SMEM_BYTES, s>>>(a);
-      return cudaGetLastError();
+      return launch_dep(kfn, dim3(unsigned((a.nlines + C - 1) / C), unsigned(std::max(1, a.nrhs))), TL::NT, TL::SMEM_BYTES, s, a);
     }
   } else if constexpr (HALF || std::is_same<T, double>::value) {
     constexpr int CS = 2;   // two lines per CTA, four CTAs per SM, as at the powers of two
     using LS = LSmem<L, CS, T>;
     auto kfs = k_xfwd_smem<T, L, CS, HALF>;
     if (setup) return cudaFuncSetAttribute(kfs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LS::SMEM_BYTES));
-    kfs<<<dim3(unsigned((a.nlines + CS - 1) / CS), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s>>>(a);
-    return cudaGetLastError();
+    return launch_dep(kfs, dim3(unsigned((a.nlines + CS - 1) / CS), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s, a);
   }
   return setup ? cudaSuccess : cudaErrorInvalidValue;
 }
@@ -2334,8 +2332,7 @@ cudaError_t launch_xinv_mix_L(const XArgs& a, Scalars* sc, int fin, cudaStream_t
     const unsigned grid = unsigned((a.nlines + CS - 1) / CS);
     if (nblocks) *nblocks = grid;
     if (setup) return cudaFuncSetAttribute(kfs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LS::SMEM_BYTES));
-    kfs<<<dim3(grid, unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s>>>(a, sc, fin);
-    return cudaGetLastError();
+    return launch_dep(kfs, dim3(grid, unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s, a, sc, fin);
   }
 }
 
@@ -2359,8 +2356,7 @@ cudaError_t launch_strided_mix_L(SArgs a, cudaStream_t s, bool setup) {
     auto kfs = k_strided_smem<T, L, CS, SMODE, (SMODE == SMODE_FWD ? HALF : true)>;
     if (setup) return cudaFuncSetAttribute(kfs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LS::SMEM_BYTES));
     a.col_blocks = (a.ncols + CS - 1) / CS;
-    kfs<<<dim3(unsigned(a.nouter) * unsigned(a.col_blocks), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s>>>(a);
-    return cudaGetLastError();
+    return launch_dep(kfs, dim3(unsigned(a.nouter) * unsigned(a.col_blocks), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s, a);
   }
   return setup ? cudaSuccess : cudaErrorInvalidValue;
 }
@@ -2383,8 +2379,7 @@ cudaError_t launch_xfwd_L(const XArgs& a, cudaStream_t s, bool setup) {
     using LS = LSmem<L, CS, T>;
     auto kfs = k_xfwd_smem<T, L, CS, HALF>;
     if (setup) return cudaFuncSetAttribute(kfs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LS::SMEM_BYTES));
-    kfs<<<dim3(unsigned((a.nlines + CS - 1) / CS), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s>>>(a);
-    return cudaGetLastError();
+    return launch_dep(kfs, dim3(unsigned((a.nlines + CS - 1) / CS), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s, a);
   } else {
     return launch_xfwd_reg_L<T, L, HALF>(a, s, setup);
   }
@@ -2403,8 +2398,7 @@ cudaError_t launch_xinv_L(const XArgs& a, Scalars* sc, int fin, cudaStream_t s, 
     const unsigned grid = unsigned((a.nlines + CS - 1) / CS);
     if (nblocks) *nblocks = grid;
     if (setup) return cudaFuncSetAttribute(kfs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LS::SMEM_BYTES));
-    kfs<<<dim3(grid, unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s>>>(a, sc, fin);
-    return cudaGetLastError();
+    return launch_dep(kfs, dim3(grid, unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s, a, sc, fin);
   } else {
     return launch_xinv_reg_L<T, L>(a, sc, fin, s, setup, nblocks);
   }
@@ -2442,8 +2436,7 @@ cudaError_t launch_strided_L(SArgs a, cudaStream_t s, bool setup) {
       auto kfs = k_strided_smem<T, L, CS, SMODE, (SMODE == SMODE_FWD ? HALF : true)>;
       if (setup) return cudaFuncSetAttribute(kfs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LS::SMEM_BYTES));
       a.col_blocks = (a.ncols + CS - 1) / CS;
-      kfs<<<dim3(unsigned(a.nouter) * unsigned(a.col_blocks), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s>>>(a);
-      return cudaGetLastError();
+      return launch_dep(kfs, dim3(unsigned(a.nouter) * unsigned(a.col_blocks), unsigned(std::max(1, a.nrhs))), LS::NT, LS::SMEM_BYTES, s, a);
     }
   } else {
     return launch_strided_reg_L<T, L, SMODE, HALF>(a, s, setup);

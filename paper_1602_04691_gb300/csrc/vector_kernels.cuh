@@ -330,6 +330,7 @@ template <class T>
 __global__ void k_cocg_update(cpx<T>* __restrict__ x, const cpx<T>* __restrict__ p,
                               cpx<T>* __restrict__ r, const cpx<T>* __restrict__ q, long long n3,
                               Scalars* sc0, double2* partials0) {
+  dep_wait();
   __shared__ double2 red[64];
   __shared__ int s_last;
   const int rb = blockIdx.y;
@@ -375,6 +376,7 @@ template <>
 __global__ void k_cocg_update<float>(cpx<float>* __restrict__ x, const cpx<float>* __restrict__ p,
                                      cpx<float>* __restrict__ r, const cpx<float>* __restrict__ q,
                                      long long n3, Scalars* sc0, double2* partials0) {
+  dep_wait();
   __shared__ double2 red[64];
   __shared__ int s_last;
   const int rb = blockIdx.y;
