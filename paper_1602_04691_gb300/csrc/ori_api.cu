@@ -2079,10 +2079,15 @@ extern "C" ori_status ori_field(ori_plan_t p, const double* u_dev, int64_t npts,
   ORI_VEC(p, ORI_PASS_VECTOR,
           (k_charges<<<p->vec_grid, 256, 0, p->ps>>>(reinterpret_cast<const cpx<double>*>(u_dev), p->h, p->N, coef,
                                                       p->p64, p->n3)));
-  // slices per point: enough blocks to fill the GPU; partials in the FP64 scratch cube
+  // slices per point: enough blocks to fill the GPU, of 256 cells or more; with
+  // 2048 cells or more to a block (its coordinate table and reduction are then
+  // below a tenth of its work) about 32 blocks an SM, so that the last ones to
+  // run leave few SMs idle.  Partials in the FP64 scratch cube.
   const long long cap_entries = (long long)t1_elems(p) * p->cap;
-  int S = int(std::max<long long>(1, std::min<long long>(256, (4LL * p->sm_count + npts - 1) / npts)));
-  S = int(std::min<long long>(S, std::max<long long>(1, p->n3 / 256)));
+  auto slices = [&](long long per_sm, long long cells) {
+    return std::min<long long>((per_sm * p->sm_count + npts - 1) / npts, p->n3 / cells);
+  };
+  const int S = int(std::max<long long>(1, std::min<long long>(256, std::max(slices(4, 256), slices(32, 2048)))));
   const long long chunk = std::max<long long>(1, std::min<long long>(npts, cap_entries / S));
   double2* partials = reinterpret_cast<double2*>(p->T1d);
   for (long long c0 = 0; c0 < npts; c0 += chunk) {
@@ -2090,7 +2095,7 @@ extern "C" ori_status ori_field(ori_plan_t p, const double* u_dev, int64_t npts,
     const double* pts = points_dev + 3 * c0;
     const dim3 grid(unsigned(std::min<long long>(np, 65535)), unsigned(S));
     ORI_VEC(p, ORI_PASS_VECTOR,
-            (k_field_partial<<<grid, 256, 0, p->ps>>>(p->p64, pts, np, p->n, p->d, p->origin[0], p->origin[1],
+            (k_field_partial<<<grid, 256, 3 * size_t(p->n) * sizeof(double), p->ps>>>(p->p64, pts, np, p->n, p->d, p->origin[0], p->origin[1],
                                                        p->origin[2], p->ks[0], partials)));
     ORI_VEC(p, ORI_PASS_VECTOR,
             (k_field_finish<<<unsigned((np + 255) / 256), 256, 0, p->ps>>>(
