@@ -731,9 +731,11 @@ static ori_status set_medium(ori_plan_s* p, const double* h_dev, const double* N
 // (zero at the origin and beyond offsets n - 1) is even along each axis, so
 // its DFT is even too and only the octant kx, ky, kz <= L/2 (H = L/2 + 1 per
 // axis) is kept.  Planes z = 0..H-1 (the others repeat them) are transformed
-// along x and y in batches, keeping kx, ky < H, into an H^3 buffer; the z
-// transform then reads row L - z for z > L/2 (the even extension) and keeps
-// kz < H in place.  FP64 throughout; the octant is stored in FP64, FP32 and
+// in batches: the x transform of the lines y = 0..H-1 (half of a plane: the
+// FP64 sines, cosines and butterflies of the x pass are three quarters of the
+// build), the y transform reading row L - y for y > L/2 (the even extension)
+// and keeping kx, ky < H, into an H^3 buffer; the z transform then extends
+// and keeps kz < H in the same way, in place.  FP64 throughout; the octant is stored in FP64, FP32 and
 // paired FP32 with c_S |Delta| / L^3 folded in, plus the Z-tile-ordered FP32
 // copy.  Transient memory: the H^3 octant and a batch of L^2 planes.
 static ori_status build_spectrum(ori_plan_s* p) {
@@ -742,7 +744,7 @@ static ori_status build_spectrum(ori_plan_s* p) {
   const long long L3 = (long long)L * L * L;
   const long long H3 = (long long)H * H * H;
   const long long HZ = (long long)H * H * L;
-  const long long plane = (long long)L * L;
+  const long long plane = (long long)L * H;   // a plane's lines y = 0..H-1
   const int nz = int(std::max<long long>(1, std::min<long long>(H, (1LL << 26) / plane)));   // <= 1 GiB per batch
   cpx<double>* oct = nullptr;
   cpx<double>* planes = nullptr;
@@ -766,11 +768,11 @@ static ori_status build_spectrum(ori_plan_s* p) {
       a.d = p->d;
       a.k = p->ks[ik];
       a.n = n;
-      a.nlines = (long long)nzb * L;
+      a.nlines = nzb * H;
       a.n_in = L;
       a.line_len_in = L;
       a.line_len_out = L;
-      a.lines_per_plane = L;
+      a.lines_per_plane = H;
       a.plane0 = z0;
       a.fft_out = planes;
       a.twL = p->tw64;
@@ -781,6 +783,7 @@ static ori_status build_spectrum(ori_plan_s* p) {
       y.out = oct + (long long)z0 * H * H;
       y.in_outer = plane; y.out_outer = (long long)H * H;
       y.in_pt = L; y.out_pt = H; y.ncols = H; y.n_in = L; y.n_out = H; y.nouter = nzb;
+      y.mirror_in = 1;
       y.twL = p->tw64;
       y.sm_count = p->sm_count;
       check(run_strided<double>(L, SMODE_FWD, false, y, p->ps, false), "plan Y pass");

@@ -80,7 +80,7 @@ struct XArgs {
   int n_in;             // valid input points (forward)
   int line_len_in;      // elements between lines in the input
   int line_len_out;     // elements between lines in the output
-  int lines_per_plane;  // PRO_KERNEL: lines in one z plane (= L)
+  int lines_per_plane;  // PRO_KERNEL: lines of one z plane (L, or the L/2 + 1 of the even half)
   int plane0;           // PRO_KERNEL: z index of the first plane of the launch
   int mode;             // PRO_* or EPI_*
   const void* twL;      // twiddle table for length L
