@@ -75,6 +75,11 @@ struct ori_plan_s {
   std::vector<std::vector<double>> history;   // per system: residual estimates of the last solve
                                               // run with ori_solve_opts.history
   size_t bytes = 0, mem_cap = 0;
+  void* mem = nullptr;             // the plan's arrays, and those of the batch capacity: one
+  void* cap_mem = nullptr;         // allocation each (Carve)
+  size_t cap_bytes = 0;            // of the capacity, counted in bytes
+  void* pin = nullptr;             // pinned mirrors of the plan and of the capacity
+  void* cap_pin = nullptr;
   int sm_count = 0;
   unsigned long long zero_S = 0;
   // medium
@@ -244,31 +249,63 @@ static void t_harvest_graph(ori_plan_s* p, const ori_plan_s::Pend* g, int ng, in
   cudaGetLastError();
 }
 
-static ori_status plan_alloc(ori_plan_s* p, void** ptr, size_t bytes) {
-  if (p->mem_cap && p->bytes + bytes > p->mem_cap)
+// Arrays laid out in one allocation.  The first sweep (base null) adds up
+// the sizes, the second hands out the pointers, each on 256 bytes.  A plan
+// holds some forty arrays; at small grids allocating and freeing them one by
+// one took half of a one-call solve (n = 64: 2.3 of 4.2 ms).
+struct Carve {
+  char* base = nullptr;
+  size_t off = 0;      // bytes of the allocation
+  size_t bytes = 0;    // bytes of the arrays
+  template <class P>
+  void take(P*& ptr, size_t count) {
+    off = (off + 255) & ~size_t(255);
+    ptr = base ? reinterpret_cast<P*>(base + off) : nullptr;
+    off += count * sizeof(P);
+    bytes += count * sizeof(P);
+  }
+};
+
+// Allocate what `layout` takes; *mem is the allocation, *bytes what its arrays hold.
+template <class F>
+static ori_status carve_device(ori_plan_s* p, void** mem, size_t* bytes, F layout) {
+  Carve c;
+  layout(c);
+  if (p->mem_cap && p->bytes + c.bytes > p->mem_cap)
     return fail(ORI_ERR_OOM, "plan memory would exceed opts->mem_cap");
-  cudaError_t e = cudaMalloc(ptr, bytes);
+  cudaError_t e = cudaMalloc(mem, c.off);
   if (e != cudaSuccess) {
-    *ptr = nullptr;
+    *mem = nullptr;
     cudaGetLastError();
     return fail(ORI_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   }
-  p->bytes += bytes;
+  *bytes = c.bytes;
+  p->bytes += c.bytes;
+  Carve g;
+  g.base = static_cast<char*>(*mem);
+  layout(g);
   return ORI_OK;
 }
 
-template <class P>
-static ori_status alloc_n(ori_plan_s* p, P** ptr, size_t count) {
-  return plan_alloc(p, reinterpret_cast<void**>(ptr), count * sizeof(P));
-}
-
-template <class P>
-static void free_n(ori_plan_s* p, P*& ptr, size_t count) {
-  if (ptr) {
-    cudaFree(ptr);
-    p->bytes -= count * sizeof(P);
-    ptr = nullptr;
+// Pinned host memory (zeroed) for what `layout` takes; *dev_delta: device address minus host address.
+template <class F>
+static ori_status carve_pinned(void** mem, ptrdiff_t* dev_delta, F layout) {
+  Carve c;
+  layout(c);
+  if (cudaMallocHost(mem, c.off) != cudaSuccess) {
+    *mem = nullptr;
+    cudaGetLastError();
+    return fail(ORI_ERR_OOM, "cudaMallocHost failed");
   }
+  void* dev = nullptr;
+  if (cudaHostGetDevicePointer(&dev, *mem, 0) != cudaSuccess)
+    return fail(ORI_ERR_CUDA, "cudaHostGetDevicePointer failed (pinned memory not mapped)");
+  std::memset(*mem, 0, c.off);
+  *dev_delta = static_cast<char*>(dev) - static_cast<char*>(*mem);
+  Carve g;
+  g.base = static_cast<char*>(*mem);
+  layout(g);
+  return ORI_OK;
 }
 
 static void drop_graphs(ori_plan_s* p) {
@@ -283,26 +320,11 @@ static size_t t2_elems(const ori_plan_s* p) { return size_t(p->n) * p->M * p->M;
 
 // Release the batch-sized buffers.
 static void free_capacity(ori_plan_s* p) {
-  const size_t c = size_t(p->cap), n3 = size_t(p->n3);
-  p->T1f = nullptr;   // the FP32 cubes live inside the FP64-class ones
-  p->T2f = nullptr;
-  free_n(p, p->T1d, c * t1_elems(p));
-  free_n(p, p->T2d, c * t2_elems(p));
-  free_n(p, p->sc, c);
-  free_n(p, p->partials, c * p->part_per_rhs);
-  for (cpx<double>** v : {&p->b64, &p->w, &p->r64, &p->u0, &p->p64, &p->q64}) free_n(p, *v, c * n3);
-  for (cpx<float>** v : {&p->x32, &p->r32, &p->p32, &p->q32}) free_n(p, *v, c * n3);
-  for (double** v : {&p->d_tols, &p->d_scl, &p->d_coef, &p->d_kv}) free_n(p, *v, c);
-  free_n(p, p->d_dir, 3 * c);
-  free_n(p, p->d_phase, 3 * size_t(p->n) * c);
-  free_n(p, p->d_skip, c);
-  if (p->h_sc) cudaFreeHost(p->h_sc);
-  if (p->h_small) cudaFreeHost(p->h_small);
-  if (p->h_skip) cudaFreeHost(p->h_skip);
-  p->h_sc = nullptr;
-  p->h_small = nullptr;
-  p->h_skip = nullptr;
-  p->h_sc_d = p->h_small_d = p->h_skip_d = nullptr;
+  if (p->cap_mem) cudaFree(p->cap_mem);
+  if (p->cap_pin) cudaFreeHost(p->cap_pin);
+  p->cap_mem = p->cap_pin = nullptr;
+  p->bytes -= p->cap_bytes;
+  p->cap_bytes = 0;
   p->cap = 0;
   drop_graphs(p);
 }
@@ -315,35 +337,38 @@ static ori_status ensure_capacity(ori_plan_s* p, int nrhs) {
   sync_plan(p);
   free_capacity(p);
   const size_t c = size_t(nrhs), n3 = size_t(p->n3);
-  // FP32 passes and FP64-class passes never run at the same time (one
-  // stream, one operator application after another), so the FP32 cubes
-  // (half the bytes) share the FP64-class allocations
-  ORI_TRY(alloc_n(p, &p->T1d, c * t1_elems(p)));
-  ORI_TRY(alloc_n(p, &p->T2d, c * t2_elems(p)));
-  p->T1f = reinterpret_cast<cpx<float>*>(p->T1d);
-  p->T2f = reinterpret_cast<cpx<float>*>(p->T2d);
-  ORI_TRY(alloc_n(p, &p->sc, c));
-  ORI_CUDA(cudaMemsetAsync(p->sc, 0, c * sizeof(Scalars), p->ps));
   // partials of the X-inverse reductions, or two per block of the widest vector grid
   p->part_per_rhs = std::max<size_t>(size_t(p->xinv_blocks), size_t(2) * std::max(1, p->sm_count) * kMaxVecCtasPerSm) + 16;
-  ORI_TRY(alloc_n(p, &p->partials, c * p->part_per_rhs));
-  for (cpx<double>** v : {&p->b64, &p->w, &p->r64}) ORI_TRY(alloc_n(p, v, c * n3));
-  if (!p->lean)   // FP64 COCG vectors and the incident field kept for S = 0 cells
-    for (cpx<double>** v : {&p->u0, &p->p64, &p->q64}) ORI_TRY(alloc_n(p, v, c * n3));
-  for (cpx<float>** v : {&p->x32, &p->r32, &p->p32, &p->q32}) ORI_TRY(alloc_n(p, v, c * n3));
-  for (double** v : {&p->d_tols, &p->d_scl, &p->d_coef, &p->d_kv}) ORI_TRY(alloc_n(p, v, c));
-  ORI_TRY(alloc_n(p, &p->d_dir, 3 * c));
-  ORI_TRY(alloc_n(p, &p->d_phase, 3 * size_t(p->n) * c));
-  ORI_TRY(alloc_n(p, &p->d_skip, c));
-  if (cudaMallocHost(&p->h_sc, c * sizeof(Scalars)) != cudaSuccess ||
-      cudaMallocHost(&p->h_small, size_t(kSmallSlots) * c * sizeof(double)) != cudaSuccess ||
-      cudaMallocHost(&p->h_skip, c * sizeof(int)) != cudaSuccess)
-    return fail(ORI_ERR_OOM, "cudaMallocHost failed");
-  if (cudaHostGetDevicePointer(&p->h_sc_d, p->h_sc, 0) != cudaSuccess ||
-      cudaHostGetDevicePointer(&p->h_small_d, p->h_small, 0) != cudaSuccess ||
-      cudaHostGetDevicePointer(&p->h_skip_d, p->h_skip, 0) != cudaSuccess)
-    return fail(ORI_ERR_CUDA, "cudaHostGetDevicePointer failed (pinned memory not mapped)");
-  std::memset(p->h_sc, 0, c * sizeof(Scalars));
+  ORI_TRY(carve_device(p, &p->cap_mem, &p->cap_bytes, [&](Carve& m) {
+    // FP32 passes and FP64-class passes never run at the same time (one
+    // stream, one operator application after another), so the FP32 cubes
+    // (half the bytes) share the FP64-class allocations
+    m.take(p->T1d, c * t1_elems(p));
+    m.take(p->T2d, c * t2_elems(p));
+    m.take(p->sc, c);
+    m.take(p->partials, c * p->part_per_rhs);
+    for (cpx<double>** v : {&p->b64, &p->w, &p->r64}) m.take(*v, c * n3);
+    if (!p->lean)   // FP64 COCG vectors and the incident field kept for S = 0 cells
+      for (cpx<double>** v : {&p->u0, &p->p64, &p->q64}) m.take(*v, c * n3);
+    for (cpx<float>** v : {&p->x32, &p->r32, &p->p32, &p->q32}) m.take(*v, c * n3);
+    for (double** v : {&p->d_tols, &p->d_scl, &p->d_coef, &p->d_kv}) m.take(*v, c);
+    m.take(p->d_dir, 3 * c);
+    m.take(p->d_phase, 3 * size_t(p->n) * c);
+    m.take(p->d_skip, c);
+  }));
+  p->T1f = reinterpret_cast<cpx<float>*>(p->T1d);
+  p->T2f = reinterpret_cast<cpx<float>*>(p->T2d);
+  p->zmap_ptr = p->ymap_ptr = nullptr;   // the tensor maps hold the old addresses
+  ptrdiff_t delta = 0;
+  ORI_TRY(carve_pinned(&p->cap_pin, &delta, [&](Carve& m) {
+    m.take(p->h_sc, c);
+    m.take(p->h_small, size_t(kSmallSlots) * c);
+    m.take(p->h_skip, c);
+  }));
+  p->h_sc_d = reinterpret_cast<char*>(p->h_sc) + delta;
+  p->h_small_d = reinterpret_cast<char*>(p->h_small) + delta;
+  p->h_skip_d = reinterpret_cast<char*>(p->h_skip) + delta;
+  ORI_CUDA(cudaMemsetAsync(p->sc, 0, c * sizeof(Scalars), p->ps));
   p->cap = nrhs;
   return ORI_OK;
 }
@@ -355,13 +380,8 @@ static void plan_free(ori_plan_s* p) {
   cudaSetDevice(p->device);
   cudaDeviceSynchronize();
   free_capacity(p);
-  void* ptrs[] = {p->h, p->N, p->w64, p->S64, p->Sinv, p->w32, p->S32, p->wdf, p->Sdf,
-                  p->ghat64, p->ghat32, p->ghatdf, p->ghatZ32, p->tw64, p->tw32, p->twdf, p->d_count,
-                  p->d_fault};
-  for (void* q : ptrs)
-    if (q) cudaFree(q);
-  if (p->h_fault) cudaFreeHost(p->h_fault);
-  if (p->h_count) cudaFreeHost(p->h_count);
+  if (p->mem) cudaFree(p->mem);
+  if (p->pin) cudaFreeHost(p->pin);
   if (p->ev0) cudaEventDestroy(p->ev0);
   if (p->ev1) cudaEventDestroy(p->ev1);
   if (p->evj) cudaEventDestroy(p->evj);
@@ -378,12 +398,11 @@ static void plan_free(ori_plan_s* p) {
 
 // Host twiddle table tab[m] = (cos, sin)(2 pi m / L), from the compile-time
 // evaluable series in common.cuh on a fine circle (2^20 points; 8 L at the mixed lengths).
-template <class T>
-static void host_twiddles(int L, cpx<T>* out) {
+static void host_twiddles(int L, cpx<double>* out) {
   const long long M = is_mixed_len(L) ? 8LL * L : 1LL << 20;
   for (int m = 0; m < L; ++m) {
     CosSin v = turn_cos_sin((long long)m * (M / L), M);
-    out[m] = cpx<T>{T(v.c), T(v.s)};
+    out[m] = cpx<double>{v.c, v.s};
   }
 }
 
@@ -737,7 +756,7 @@ static ori_status set_medium(ori_plan_s* p, const double* h_dev, const double* N
 // and keeping kx, ky < H, into an H^3 buffer; the z transform then extends
 // and keeps kz < H in the same way, in place.  FP64 throughout; the octant is stored in FP64, FP32 and
 // paired FP32 with c_S |Delta| / L^3 folded in, plus the Z-tile-ordered FP32
-// copy.  Transient memory: the H^3 octant and a batch of L^2 planes.
+// copy.
 static ori_status build_spectrum(ori_plan_s* p) {
   NvtxRange nvtx("ori plan spectrum");
   const int L = p->M, n = p->n, H = p->H;
@@ -745,16 +764,23 @@ static ori_status build_spectrum(ori_plan_s* p) {
   const long long H3 = (long long)H * H * H;
   const long long HZ = (long long)H * H * L;
   const long long plane = (long long)L * H;   // a plane's lines y = 0..H-1
-  const int nz = int(std::max<long long>(1, std::min<long long>(H, (1LL << 26) / plane)));   // <= 1 GiB per batch
-  cpx<double>* oct = nullptr;
-  cpx<double>* planes = nullptr;
-  cudaError_t e = cudaMalloc(&oct, size_t(H3) * sizeof(cpx<double>));
-  if (e == cudaSuccess) e = cudaMalloc(&planes, size_t(nz) * size_t(plane) * sizeof(cpx<double>));
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    if (oct) cudaFree(oct);
-    return fail(ORI_ERR_OOM, std::string("cudaMalloc (spectrum build): ") + cudaGetErrorString(e));
+  int nz = int(std::max<long long>(1, std::min<long long>(H, (1LL << 26) / plane)));   // <= 1 GiB per batch
+  // The octant and the planes live in the pass scratch (T2, idle until the
+  // first operator), in transient memory where min_L makes them larger.
+  cpx<double>* oct = p->T2d;
+  cpx<double>* own = nullptr;
+  const long long room = (long long)t2_elems(p) * p->cap;
+  if (room >= H3 + plane) {
+    nz = int(std::min<long long>(nz, (room - H3) / plane));
+  } else {
+    const cudaError_t e = cudaMalloc(&own, size_t(H3 + nz * plane) * sizeof(cpx<double>));
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return fail(ORI_ERR_OOM, std::string("cudaMalloc (spectrum build): ") + cudaGetErrorString(e));
+    }
+    oct = own;
   }
+  cpx<double>* planes = oct + H3;
   ori_status st = ORI_OK;
   auto check = [&](cudaError_t err, const char* what) {
     if (err != cudaSuccess && st == ORI_OK) st = fail(ORI_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(err));
@@ -809,8 +835,7 @@ static ori_status build_spectrum(ori_plan_s* p) {
     check(cudaStreamSynchronize(p->ps), "plan spectrum");
   }
   cudaStreamSynchronize(p->ps);
-  cudaFree(planes);
-  cudaFree(oct);
+  if (own) cudaFree(own);
   return st;
 }
 
@@ -841,7 +866,9 @@ static ori_status load_spectrum(ori_plan_s* p, const unsigned char* buf) {
   // a lean plan has no FP64 spectrum: the entries go through a bounded staging buffer
   const long long chunk = p->ghat64 ? H3 : std::min<long long>(H3, 1LL << 26);
   cpx<double>* stage = nullptr;
-  if (!p->ghat64) {
+  const bool own = !p->ghat64 && (long long)t2_elems(p) * p->cap < chunk;
+  if (!p->ghat64 && !own) stage = p->T2d;   // the pass scratch
+  if (own) {
     cudaError_t e = cudaMalloc(&stage, size_t(chunk) * sizeof(cpx<double>));
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -869,7 +896,7 @@ static ori_status load_spectrum(ori_plan_s* p, const unsigned char* buf) {
       if (e != cudaSuccess) st = fail(ORI_ERR_CUDA, std::string("spectrum load: ") + cudaGetErrorString(e));
     }
   }
-  if (stage) cudaFree(stage);
+  if (own) cudaFree(stage);
   return st;
 }
 
@@ -1010,26 +1037,42 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
     const size_t n3 = size_t(p->n3), nk = ks.size();
     const size_t H3 = size_t(p->H) * p->H * p->H;
     const bool full = !p->lean;   // arrays of the FP64 and A-form operations, the adjoint and the field
-    if ((full && ((st = alloc_n(p, &p->h, n3)) || (st = alloc_n(p, &p->N, n3)) || (st = alloc_n(p, &p->w64, n3)) ||
-                  (st = alloc_n(p, &p->Sinv, n3)) || (st = alloc_n(p, &p->w32, n3)) || (st = alloc_n(p, &p->wdf, n3)) ||
-                  (st = alloc_n(p, &p->ghat64, nk * H3)))) ||
-        (st = alloc_n(p, &p->S64, n3)) || (st = alloc_n(p, &p->S32, n3)) || (st = alloc_n(p, &p->Sdf, n3)) ||
-        (st = alloc_n(p, &p->ghat32, nk * H3)) ||
-        (st = alloc_n(p, &p->ghatdf, nk * H3)) ||
-        (st = alloc_n(p, &p->ghatZ32, nk * size_t(p->H) * p->H * p->M)) ||
-        (st = alloc_n(p, &p->tw64, size_t(p->M))) || (st = alloc_n(p, &p->tw32, size_t(p->M))) ||
-        (st = alloc_n(p, &p->twdf, size_t(p->M))) || (st = alloc_n(p, &p->d_count, 1)) ||
-        (st = alloc_n(p, &p->d_fault, 1)))
+    size_t plan_bytes = 0;
+    if ((st = carve_device(p, &p->mem, &plan_bytes, [&](Carve& m) {
+           if (full) {
+             m.take(p->h, n3);
+             m.take(p->N, n3);
+             m.take(p->w64, n3);
+             m.take(p->Sinv, n3);
+             m.take(p->w32, n3);
+             m.take(p->wdf, n3);
+             m.take(p->ghat64, nk * H3);
+           }
+           m.take(p->S64, n3);
+           m.take(p->S32, n3);
+           m.take(p->Sdf, n3);
+           m.take(p->ghat32, nk * H3);
+           m.take(p->ghatdf, nk * H3);
+           m.take(p->ghatZ32, nk * size_t(p->H) * p->H * p->M);
+           m.take(p->tw64, size_t(p->M));
+           m.take(p->tw32, size_t(p->M));
+           m.take(p->twdf, size_t(p->M));
+           m.take(p->d_count, 1);
+           m.take(p->d_fault, 1);
+         })))
       break;
-    if (cudaMemset(p->d_fault, 0, sizeof(int)) != cudaSuccess || cudaMallocHost(&p->h_fault, sizeof(int)) != cudaSuccess ||
-        cudaMallocHost(&p->h_count, sizeof(unsigned long long)) != cudaSuccess ||
-        cudaHostGetDevicePointer(&p->h_fault_d, p->h_fault, 0) != cudaSuccess ||
-        cudaHostGetDevicePointer(&p->h_count_d, p->h_count, 0) != cudaSuccess) {
+    ptrdiff_t delta = 0;
+    if ((st = carve_pinned(&p->pin, &delta, [&](Carve& m) {
+           m.take(p->h_fault, 1);
+           m.take(p->h_count, 1);
+         })))
+      break;
+    p->h_fault_d = reinterpret_cast<char*>(p->h_fault) + delta;
+    p->h_count_d = reinterpret_cast<char*>(p->h_count) + delta;
+    if (cudaMemset(p->d_fault, 0, sizeof(int)) != cudaSuccess) {
       st = fail(ORI_ERR_CUDA, "fault flag");
       break;
     }
-    *p->h_fault = 0;
-    *p->h_count = 0;
     unsigned bx32 = 0, bx64 = 0, bxdf = 0;
     if ((st = setup_kernels<float>(p->M, &bx32, p->n, p->sm_count)) ||
         (st = setup_kernels<double>(p->M, &bx64, p->n, p->sm_count)) ||
@@ -1041,9 +1084,9 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
       cpx<double>* twd = new cpx<double>[p->M];
       cpx<float>* twf = new cpx<float>[p->M];
       cpx<dfl>* twdf = new cpx<dfl>[p->M];
-      host_twiddles<double>(p->M, twd);
-      host_twiddles<float>(p->M, twf);
+      host_twiddles(p->M, twd);
       for (int m = 0; m < p->M; ++m) {   // the stage layout of paired FP32: (re.hi, im.hi, re.lo, im.lo)
+        twf[m] = cpx<float>{float(twd[m].x), float(twd[m].y)};
         const dfl re = df_from_double_host(twd[m].x), im = df_from_double_host(twd[m].y);
         float* f = reinterpret_cast<float*>(twdf + m);
         f[0] = re.hi;
@@ -1060,8 +1103,8 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
       if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) { st = fail(ORI_ERR_CUDA, "twiddle upload failed"); break; }
     }
     if ((st = set_medium(p, h_dev, N_dev))) break;
+    if ((st = ensure_capacity(p, 1))) break;   // before the spectrum build, which uses its cubes
     if ((st = spec ? load_spectrum(p, static_cast<const unsigned char*>(spec)) : build_spectrum(p))) break;
-    if ((st = ensure_capacity(p, 1))) break;   // after the spectrum build: lower peak memory
     if ((st = leave(p, user))) break;
   } while (0);
   if (st != ORI_OK) {
