@@ -170,14 +170,14 @@ constexpr int even_box(int rows) {
 // waits in dep_wait until the previous kernel has completed and its writes
 // are visible.  Every kernel launched this way calls dep_wait before it
 // touches anything another kernel writes or reads (all but the plan's
-// twiddle tables), in every thread, and then lets its own successor start.
-// FP32 operator (five passes) at n = 100: 79.9 -> 71.2 us; FP64 operator at
-// n = 12: 44.0 -> 34.4 us; mixed solve at n = 20: 0.83 -> 0.74 ms.
+// twiddle tables), in every thread.  The successor's launch is not triggered
+// early: CTAs waiting on an SM from the start of their predecessor cost more
+// than the overlap gives (n = 400: FP32 operator 4.14 ms with an early trigger,
+// 3.92 without, 3.93 with plain launches; n = 128: 0.112, 0.103 and 0.118 ms).
+// FP32 operator (five passes) at n = 100: 79.9 -> 66.7 us; FP64 operator at
+// n = 12: 44.0 -> 34.4 us; mixed solve at n = 20: 0.83 -> 0.72 ms.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void dep_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... P, class... A>
 inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
                               const A&... args) {
