@@ -376,7 +376,8 @@ typedef struct {
                            columns with the transform split L = L1 * L2,
                            L1 = 2^ceil(log2(L) / 2); 1: tiles of 8 columns;
                            2: 16 columns, split (2 L1) * (L2 / 2).  The default is
-                           2 at transform lengths 256 and 1024, else 0.  Other lengths
+                           2 at transform lengths 256 and 1024 (Z pass: at
+                           256), else 0.  Other lengths
                            have variant 0 only.  A plan whose transform length M
                            is not a power of two runs one persistent kernel per
                            pass whatever these fields say (zconv_variant 1: its

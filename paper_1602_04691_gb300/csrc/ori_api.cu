@@ -115,7 +115,7 @@ struct ori_plan_s {
   // and a batch of zmap_R right-hand sides
   CUtensorMap zmap{};
   const void* zmap_ptr = nullptr;
-  int zmap_R = 0, zmap_ok = 0, zbox = 0;
+  int zmap_R = 0, zmap_ok = 0, zbox = 0, zmap_w = 0;   // zmap_w: columns of a box
   // tensor maps of the FP32 Y passes' input rows: T1f rows (Y forward) and
   // T2f rows (Y inverse), 16 columns by ybox rows a box
   CUtensorMap ymap_f{}, ymap_i{};
@@ -492,34 +492,38 @@ static bool z_bulk_staged(const ori_plan_s* p) {
   return !(has_pipe_variants(L) && p->var_z == 1);
 }
 
-// The tensor map of the FP32 Z pass's input: T2f seen as [rhs][z][ky][kx]
-// with dims (kx: L, ky: L, z: n, rhs: R), 8-byte elements, boxes of
+// The tensor map of the FP32 Z pass's input T2f, [rhs][ky / B][z][ky % B][kx]
+// with dims (kx: L, ky % B: B, (ky / B) n + z: n L / B, rhs: R), 8-byte elements, boxes of
 // 16 x 1 x zbox x 1 (128-byte rows; zbox = min(L / 2, 256), so that the boxes
 // covering z < n end within the tile's L / 2 + 1 staged rows).  Encoded when
 // T2f or the batch size changes; without an encoder, an aligned base or a
 // length the kernel stages by bulk copies, the kernel keeps cp.async.
 static void z_tensor_map(ori_plan_s* p, SArgs& z, int nrhs) {
   const int R = std::max(1, nrhs);
-  if (p->zmap_ptr != p->T2f || p->zmap_R != R) {
+  // columns of a box: a group's where the pass works in groups (zconv_groups), else 16
+  const int w = is_mixed_len(p->M) || p->var_z == 0 ? zgroup(p->M) : kZGroup;
+  if (p->zmap_ptr != p->T2f || p->zmap_R != R || p->zmap_w != w) {
     p->zmap_ok = 0;
     p->zmap_ptr = p->T2f;
     p->zmap_R = R;
+    p->zmap_w = w;
     const int L = p->M;
     const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (enc != nullptr && L >= 64 && L <= 1024 && (reinterpret_cast<uintptr_t>(p->T2f) & 15u) == 0) {
       const cuuint64_t es = sizeof(cpx<float>);
-      const cuuint64_t dims[4] = {cuuint64_t(L), cuuint64_t(L), cuuint64_t(p->n), cuuint64_t(R)};
-      const cuuint64_t strides[3] = {cuuint64_t(L) * es, cuuint64_t(L) * L * es, cuuint64_t(t2_elems(p)) * es};
+      const cuuint64_t B = cuuint64_t(yblk(L));
+      const cuuint64_t dims[4] = {cuuint64_t(L), B, cuuint64_t(p->n) * (L / B), cuuint64_t(R)};
+      const cuuint64_t strides[3] = {cuuint64_t(L) * es, B * L * es, cuuint64_t(t2_elems(p)) * es};
       const int zbox = std::min(L / 2, 256);
       const cuuint32_t box[4] = {cuuint32_t(kZGroup), 1, cuuint32_t(zbox), 1};
-      const cuuint32_t mbox[4] = {cuuint32_t(zgroup(L)), 1, cuuint32_t(even_box(L / 2)), 1};   // mixed lengths
+      const cuuint32_t gbox[4] = {cuuint32_t(w), 1, cuuint32_t(even_box(L / 2)), 1};
       const cuuint32_t estr[4] = {1, 1, 1, 1};
       if (enc(&p->zmap, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, p->T2f, dims, strides,
-              is_mixed_len(L) ? mbox : box, estr,
+              w == kZGroup ? box : gbox, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS) {
         p->zmap_ok = 1;
-        p->zbox = is_mixed_len(L) ? even_box(L / 2) : zbox;
+        p->zbox = w == kZGroup ? zbox : even_box(L / 2);
       }
     }
   }
@@ -533,8 +537,8 @@ static void z_tensor_map(ori_plan_s* p, SArgs& z, int nrhs) {
 // FP32 columns = 128 bytes a row): the Y-forward input T1f, dims (kx, y, z,
 // right-hand side) and box (16, ybox_f, 1, 1), ybox_f = even_box(L/2) (it
 // divides L/2: the zero-filled rows past n stay within the L/2 staged rows);
-// the Y-inverse input T2f, dims (kx, ky, z, right-hand side) and box
-// (16, ybox_i, 1, 1), ybox_i = even_box(L).
+// the Y-inverse input T2f, dims (kx, ky % B, ky / B, z, right-hand side) and
+// boxes of ybox_i rows: whole blocks, at most 256 rows.
 static void y_tensor_maps(ori_plan_s* p, SArgs& y, SArgs& yi, int nrhs) {
   const int R = std::max(1, nrhs);
   if (p->ymap_ptr != p->T1f || p->ymap_R != R) {
@@ -546,18 +550,25 @@ static void y_tensor_maps(ori_plan_s* p, SArgs& y, SArgs& yi, int nrhs) {
     if (enc != nullptr && L >= 64 && L <= 1024 && ((reinterpret_cast<uintptr_t>(p->T1f) |
                                                     reinterpret_cast<uintptr_t>(p->T2f)) & 15u) == 0) {
       const cuuint64_t es = sizeof(cpx<float>);
-      const int bf = even_box(L / 2), bi = even_box(L);
+      const int B = yblk(L), nblk = L / B;
+      int nb = 1;   // blocks of ky per Y-inverse box (L < 256: the one block in boxes of even_box(L) rows)
+      for (int q = 1; q <= nblk; ++q)
+        if (nblk % q == 0 && q * B <= 256) nb = q;
+      const int bf = even_box(L / 2), bi = B == L ? even_box(L) : nb * B;
       const cuuint32_t estr[4] = {1, 1, 1, 1};
       const cuuint64_t dims_f[4] = {cuuint64_t(L), cuuint64_t(n), cuuint64_t(n), cuuint64_t(R)};
       const cuuint64_t str_f[3] = {cuuint64_t(L) * es, cuuint64_t(n) * L * es, cuuint64_t(t1_elems(p)) * es};
       const cuuint32_t box_f[4] = {cuuint32_t(kZGroup), cuuint32_t(bf), 1, 1};
-      const cuuint64_t dims_i[4] = {cuuint64_t(L), cuuint64_t(L), cuuint64_t(n), cuuint64_t(R)};
-      const cuuint64_t str_i[3] = {cuuint64_t(L) * es, cuuint64_t(L) * L * es, cuuint64_t(t2_elems(p)) * es};
-      const cuuint32_t box_i[4] = {cuuint32_t(kZGroup), cuuint32_t(bi), 1, 1};
+      const cuuint64_t dims_i[5] = {cuuint64_t(L), cuuint64_t(B), cuuint64_t(nblk), cuuint64_t(n), cuuint64_t(R)};
+      const cuuint64_t str_i[4] = {cuuint64_t(L) * es, cuuint64_t(n) * B * L * es, cuuint64_t(B) * L * es,
+                                   cuuint64_t(t2_elems(p)) * es};
+      const cuuint32_t box_i[5] = {cuuint32_t(kZGroup), cuuint32_t(std::min(B, bi)),
+                                   cuuint32_t(B == L ? 1 : nb), 1, 1};
+      const cuuint32_t estr_i[5] = {1, 1, 1, 1, 1};
       if (enc(&p->ymap_f, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, p->T1f, dims_f, str_f, box_f, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS &&
-          enc(&p->ymap_i, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, p->T2f, dims_i, str_i, box_i, estr,
+          enc(&p->ymap_i, CU_TENSOR_MAP_DATA_TYPE_UINT64, 5, p->T2f, dims_i, str_i, box_i, estr_i,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS) {
         p->ymap_ok = 1;
@@ -600,7 +611,9 @@ static ori_status run_conv(ori_plan_s* p, XArgs pro, XArgs epi, int fin, cudaStr
 
   SArgs y{};
   y.in = T1; y.out = T2;
-  y.in_outer = (long long)n * L; y.out_outer = (long long)L * L;
+  // T2 in blocks of B values of ky: [ky / B][z][ky % B][kx]
+  const long long BL = (long long)yblk(L) * L, blk = n * BL;
+  y.in_outer = (long long)n * L; y.out_outer = BL; y.out_blk = blk;
   y.in_pt = L; y.out_pt = L; y.ncols = L; y.n_in = n; y.n_out = L; y.nouter = n;
   y.twL = tw; y.done = mask.flags; y.done_stride = mask.stride; y.sm_count = p->sm_count;
   y.nrhs = nrhs; y.bs_in = bsT1; y.bs_out = bsT2;
@@ -613,8 +626,8 @@ static ori_status run_conv(ori_plan_s* p, XArgs pro, XArgs epi, int fin, cudaStr
 
   SArgs z{};
   z.in = T2; z.out = T2;
-  z.in_outer = L; z.out_outer = L;
-  z.in_pt = (long long)L * L; z.out_pt = (long long)L * L;
+  z.in_outer = L; z.out_outer = L; z.in_blk = blk; z.out_blk = blk;
+  z.in_pt = BL; z.out_pt = BL;
   z.ncols = L; z.n_in = n; z.n_out = n; z.nouter = L;
   z.twL = tw; z.ghat = gh; z.ghatZ = p->ghatZ32; z.H = p->H;
   z.done = mask.flags; z.done_stride = mask.stride; z.sm_count = p->sm_count;
@@ -629,7 +642,7 @@ static ori_status run_conv(ori_plan_s* p, XArgs pro, XArgs epi, int fin, cudaStr
   e1 = t_rec(p, s); t_pair(p, ORI_PASS_ZCONV + K, e0, e1); e0 = e1;
 
   yi.in = T2; yi.out = T1;
-  yi.in_outer = (long long)L * L; yi.out_outer = (long long)n * L;
+  yi.in_outer = BL; yi.out_outer = (long long)n * L; yi.in_blk = blk;
   yi.in_pt = L; yi.out_pt = L; yi.ncols = L; yi.n_in = L; yi.n_out = n; yi.nouter = n;
   yi.twL = tw; yi.done = mask.flags; yi.done_stride = mask.stride;
   yi.nrhs = nrhs; yi.bs_in = bsT2; yi.bs_out = bsT1;
@@ -809,6 +822,7 @@ static ori_status build_spectrum(ori_plan_s* p) {
       y.out = oct + (long long)z0 * H * H;
       y.in_outer = plane; y.out_outer = (long long)H * H;
       y.in_pt = L; y.out_pt = H; y.ncols = H; y.n_in = L; y.n_out = H; y.nouter = nzb;
+      y.out_blk = (long long)yblk(L) * y.out_pt;   // plain order
       y.mirror_in = 1;
       y.twL = p->tw64;
       y.sm_count = p->sm_count;
@@ -820,6 +834,7 @@ static ori_status build_spectrum(ori_plan_s* p) {
     z.in_outer = H; z.out_outer = H;
     z.in_pt = (long long)H * H; z.out_pt = (long long)H * H;
     z.ncols = H; z.n_in = L; z.n_out = H; z.nouter = H;
+    z.out_blk = (long long)yblk(L) * z.out_pt;
     z.mirror_in = 1;
     z.twL = p->tw64;
     z.sm_count = p->sm_count;
@@ -1013,10 +1028,11 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
     p->L = std::max(p->L, o.min_L);
     p->H = p->M / 2 + 1;
     // default launch variants: at L = 256 and 1024 the (2 L1) x (L2 / 2) split
-    // was the faster one in all three passes (n = 512: 7.05 -> 6.85 ms an
-    // operator, n = 128: 0.129 -> 0.117 ms), at L = 512 the square-most one
-    // (n = 256: 0.832 against 0.870 ms)
-    if (p->M == 256 || p->M == 1024) p->var_y = p->var_z = p->var_yi = 2;
+    // was the faster one in the Y passes, and at L = 256 in the Z pass (n = 128:
+    // 0.129 -> 0.117 ms an operator; n = 512: Y 1.08 + 1.10 -> 1.01 + 1.04 ms),
+    // at L = 512 the square-most one (n = 256: 0.832 against 0.870 ms)
+    if (p->M == 256 || p->M == 1024) p->var_y = p->var_yi = 2;
+    if (p->M == 256) p->var_z = 2;
     p->n3 = (long long)n * n * n;
     p->ks = ks;
     p->side = dom->side;

@@ -11,7 +11,13 @@
 //   Y inv : T2[z][0..L)[kx]                                 ->  T1[z][0..n)[kx]
 //   X inv : T1[z][y][0..L) -> keep x < n --(epilogue: y = x + s conv, dots)--> y
 //
-// T1 is [n][n][L] and T2 is [n][L][L] (C-order, x fastest).  The spectrum is
+// T1 is [n][n][L] (C-order, x fastest).  T2 holds its [z][ky][kx] points in
+// blocks of B = yblk(L) values of ky, [ky / B][z][ky % B][kx] (below L = 256
+// B = L, the plain order).  The Y passes walk ky at a fixed z and the Z pass z
+// at a fixed ky; in the plain order a Z tile's n rows lie L^2 points apart
+// (8 MB at L = 1024), every one in another page, and the address translation
+// was what a tile of narrow rows waited for (8-column Z tiles, n = 512: 3.59 ms
+// plain, 3.13 ms in blocks of 128; n = 288: 0.58 and 0.52 ms).  The spectrum is
 // stored once for the (L/2+1)^3 distinct entries (the kernel cube is even
 // along each axis); column (kx, ky, kz) reads entry (m(kz), m(ky), m(kx)),
 // m(k) = min(k, L - k), and already carries c_S |Delta| / L^3.
@@ -101,6 +107,9 @@ struct SArgs {
   void* out;
   long long in_outer, out_outer;   // elements between outer indices
   long long in_pt, out_pt;         // elements between points of a line
+  // elements between blocks of yblk(L): of the output points of a forward
+  // pass, the input points of an inverse pass, the outer index of the Z pass
+  long long in_blk, out_blk;
   int ncols;                       // columns per outer index (stride 1)
   int col_blocks;                  // ceil(ncols / C)
   int n_in, n_out;
@@ -127,10 +136,11 @@ struct SArgs {
   int cta_cap;
   int variant;                     // pipelined FP32 kernels: launch variant (has_pipe_variants)
   // FP32 Z and Y passes with 16-column tiles: the input rows of a tile
-  // arrive by TMA (cp.async.bulk.tensor) through this map of the input cube,
-  // dims (kx, ky, z, right-hand side) and box (16, 1, zbox, 1) for the Z
-  // pass, (kx, y, z, right-hand side) and box (16, zbox, 1, 1) for the Y
-  // passes; zrows_ok = 0 keeps cp.async
+  // arrive by TMA (cp.async.bulk.tensor) through this map of the input cube:
+  // Z pass, dims (kx, ky % B, (ky / B) n + z, right-hand side) of T2 and box
+  // (16, 1, zbox, 1); Y forward, dims (kx, y, z, right-hand side) of T1 and box
+  // (16, zbox, 1, 1); Y inverse, dims (kx, ky % B, ky / B, z, right-hand side)
+  // of T2 and box (16, B, zbox / B, 1, 1); zrows_ok = 0 keeps cp.async
   CUtensorMap zrows;
   int zrows_ok;
   int zbox;
@@ -141,8 +151,9 @@ enum { SCHED_PERSISTENT = 0, SCHED_TILES = 1 };
 
 // Columns per group of the Z-tile-ordered FP32 spectrum [my][kx / kZGroup][mz][kZGroup].
 constexpr int kZGroup = 16;
-// ... at transform length L: the mixed lengths (MixRad) group by the 8 columns of their Z tiles.
-constexpr int zgroup(int L) { return is_mixed_len(L) ? 8 : kZGroup; }
+// ... at transform length L, where the Z pass works in groups of fewer columns
+// (zconv_groups): their number.
+constexpr int zgroup(int L) { return is_mixed_len(L) || L == 1024 ? 8 : kZGroup; }
 
 // Transform length of a grid: the smallest instantiated length >= 2n.  Any
 // length >= 2n - 1 gives the same operator, and the work of a pass grows with
@@ -153,6 +164,36 @@ constexpr int transform_length(int n, int pow2) {
   for (int m : {144, 200, 288, 400, 576, 800})
     if (m >= 2 * n && m > pow2 / 2 && m < pow2) return m;
   return pow2;
+}
+
+// Values of ky per block of T2 at transform length L.  Narrow Z tiles want few
+// (rows of a tile within tens of pages), the Y passes many: n = 512, Y forward +
+// Z + Y inverse 1.01 + 2.86 + 1.05 ms in blocks of 32, 1.10 + 2.98 + 1.05 in
+// blocks of 128; n = 400: 0.67 + 1.73 + 0.59 in blocks of 40, 0.67 + 1.84 + 0.59
+// plain; n = 260: what the Z pass gains (0.55 -> 0.53) the Y passes lose.
+constexpr int yblk(int L) {
+  if (L < 256) return L;
+  if (is_mixed_len(L)) return L == 800 ? 40 : L;
+  return L == 256 ? 64 : 32;
+}
+// Offset of point k of a line laid out in blocks: `blk` elements between blocks, `pt` between points of one.
+template <int L>
+__device__ __forceinline__ long long blk_off(int k, long long blk, long long pt) {
+  constexpr int B = yblk(L);
+  static_assert(L % B == 0, "whole blocks");
+  return (long long)(k / B) * blk + (long long)(k % B) * pt;
+}
+
+// Offset of point k + STEP t from that of point k < STEP (`at` = blk_off<L>(k)):
+// the block and the place in it move by compile-time amounts when STEP is
+// whole blocks or divides one.
+template <int L, int STEP>
+__device__ __forceinline__ long long blk_at(long long at, int k, int t, long long blk, long long pt) {
+  constexpr int B = yblk(L);
+  if constexpr (B == L) return at + t * (STEP * pt);
+  else if constexpr (STEP % B == 0) return at + t * (STEP / B * blk);
+  else if constexpr (B % STEP == 0) return at + (STEP * t / B) * blk + (STEP * t % B) * pt;
+  else return blk_off<L>(k + STEP * t, blk, pt);
 }
 
 // Rows of one TMA box when boxes of equal size cover exactly `rows` staged rows (at most 256 each).

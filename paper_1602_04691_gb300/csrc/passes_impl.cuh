@@ -64,6 +64,13 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, i
       ::"r"(smem_addr(dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_addr(bar))
       : "memory");
 }
+__device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, int x, int y, int z, int w, int v,
+                                            unsigned long long* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
+      ::"r"(smem_addr(dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(v), "r"(smem_addr(bar))
+      : "memory");
+}
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar))
@@ -752,8 +759,10 @@ __global__ void __launch_bounds__(Tile<L, C, T>::NT) k_strided(SArgs a0) {
   const int tid = threadIdx.x;
   const int outer = blockIdx.x / a.col_blocks;
   const int cb = blockIdx.x - outer * a.col_blocks;
-  const cpx<T>* in = reinterpret_cast<const cpx<T>*>(a.in) + outer * a.in_outer + (long long)cb * C;
-  cpx<T>* out = reinterpret_cast<cpx<T>*>(a.out) + outer * a.out_outer + (long long)cb * C;
+  const cpx<T>* in = reinterpret_cast<const cpx<T>*>(a.in) + (long long)cb * C +
+                     (SMODE == SMODE_ZCONV ? blk_off<L>(outer, a.in_blk, a.in_outer) : outer * a.in_outer);
+  cpx<T>* out = reinterpret_cast<cpx<T>*>(a.out) + (long long)cb * C +
+                (SMODE == SMODE_ZCONV ? blk_off<L>(outer, a.out_blk, a.out_outer) : outer * a.out_outer);
   const int colmax = a.ncols - cb * C;
 
   cpx<T> b[NI][L2];
@@ -790,10 +799,11 @@ __global__ void __launch_bounds__(Tile<L, C, T>::NT) k_strided(SArgs a0) {
         int c2, k1;
         map_s<LAYOUT_STRIDED, C, L1>(tid + it * NT, c2, k1);
         if (c2 < colmax) {
+          const long long o = blk_off<L>(k1, a.out_blk, a.out_pt) + c2;
 #pragma unroll
           for (int k2 = 0; k2 < L2; ++k2) {
             const int k = k1 + L1 * k2;
-            if (k < a.n_out) out[(long long)k * a.out_pt + c2] = settle(b[it][k2]);
+            if (k < a.n_out) out[blk_at<L, L1>(o, k1, k2, a.out_blk, a.out_pt)] = settle(b[it][k2]);
           }
         }
       }
@@ -820,9 +830,10 @@ __global__ void __launch_bounds__(Tile<L, C, T>::NT) k_strided(SArgs a0) {
     for (int it = 0; it < NI; ++it) {
       int c2, k1;
       map_s<LAYOUT_STRIDED, C, L1>(tid + it * NT, c2, k1);
+      const long long o = blk_off<L>(k1, a.in_blk, a.in_pt) + c2;
 #pragma unroll
       for (int k2 = 0; k2 < L2; ++k2)
-        b[it][k2] = c2 < colmax ? in[(long long)(k1 + L1 * k2) * a.in_pt + c2] : czero<T>();
+        b[it][k2] = c2 < colmax ? in[blk_at<L, L1>(o, k1, k2, a.in_blk, a.in_pt)] : czero<T>();
     }
   }
   // inverse stage A: DFT over k2, twiddle, exchange
@@ -909,10 +920,11 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_st
       cpx<T> v[r3];
       dif_last<L, C, -1>(X, blk, c, v);
       const int k0 = freq_of_block<L>(blk);
+      const long long o = blk_off<L>(k0, a.out_blk, a.out_pt);
 #pragma unroll
       for (int t = 0; t < r3; ++t) {
         const int k = k0 + (L / r3) * t;
-        if (c < colmax && k < a.n_out) out[(long long)k * a.out_pt + c] = settle(v[t]);
+        if (c < colmax && k < a.n_out) out[blk_at<L, L / r3>(o, k0, t, a.out_blk, a.out_pt) + c] = settle(v[t]);
       }
     }
   } else {
@@ -924,10 +936,11 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_st
     for (int g = tid; g < C * S8; g += NT) {
       const int c = g % C, j = g / C;
       cpx<T> v[8];
+      const long long o = blk_off<L>(j, a.in_blk, a.in_pt);
 #pragma unroll
       for (int t = 0; t < 8; ++t) {
         const int jj = j + t * S8;
-        v[t] = (c < colmax && jj < a.n_in) ? in[(long long)jj * a.in_pt + c] : czero<T>();
+        v[t] = (c < colmax && jj < a.n_in) ? in[blk_at<L, S8>(o, j, t, a.in_blk, a.in_pt) + c] : czero<T>();
       }
       dft<8, +1, false>(v);
 #pragma unroll
@@ -1248,6 +1261,8 @@ __device__ __forceinline__ int next_live_tile(const SArgs& a, int t, int step, i
   return t;
 }
 
+template <int L, int C, int G> struct ZGroups;
+
 template <int L, int C, class T, int L1X = Split<L>::L1>
 struct ZPipe {
   using TL = Tile<L, C, T, L1X>;
@@ -1261,7 +1276,12 @@ struct ZPipe {
   static constexpr size_t TW_ELEMS = GZ ? size_t(L) : 0;                // twiddle table copy
   // with TMA: 128 bytes of slack to align the tile to 128 bytes, and the mbarrier
   static constexpr size_t TMA_BYTES = TMA ? 128 + 16 : 0;
-  static constexpr size_t SMEM_BYTES = (E_ELEMS + S_ELEMS + TW_ELEMS) * sizeof(cpx<T>) + TMA_BYTES;
+  // 16-column tiles at the default split of the lengths whose spectrum is
+  // grouped by fewer columns: the tile's groups run apart (zconv_groups)
+  static constexpr int GC = zgroup(L);
+  static constexpr bool GROUPS = TMA && GC < C && L1X == Split<L>::L1;
+  static constexpr size_t SMEM_BYTES = GROUPS ? ZGroups<L, GC, C / GC>::SMEM_BYTES
+                                              : (E_ELEMS + S_ELEMS + TW_ELEMS) * sizeof(cpx<T>) + TMA_BYTES;
 };
 
 // Bulk-copy staging of the FP32 Z pass (ZPipe::TMA).  Thread 0 issues the
@@ -1280,22 +1300,30 @@ __device__ __forceinline__ void zpipe_tma_rows(const SArgs& a, int tile, int per
   const int nbox = (a.n_in + a.zbox - 1) / a.zbox;
   fence_proxy_async();
   mbar_expect_tx(bar, unsigned(nbox * a.zbox * C * int(sizeof(cpx<float>))));
-  for (int q = 0; q < nbox; ++q) tma_load_4d(S + q * a.zbox * C, &a.zrows, cb * C, ky, q * a.zbox, rhs, bar);
+  if constexpr (yblk(L) == L) {
+    for (int q = 0; q < nbox; ++q) tma_load_4d(S + q * a.zbox * C, &a.zrows, cb * C, ky, q * a.zbox, rhs, bar);
+  } else {   // rows past n_in belong to the next block of ky (or are zero-filled): staged, not used
+    const int kb = ky / yblk(L), z0 = kb * a.n_in;
+    for (int q = 0; q < nbox; ++q)
+      tma_load_4d(S + q * a.zbox * C, &a.zrows, cb * C, ky - kb * yblk(L), z0 + q * a.zbox, rhs, bar);
+  }
 }
-// The spectrum slice of a tile: with C == kZGroup the L / 2 + 1 rows of C
-// entries are one contiguous run of the Z-tile-ordered spectrum.
+// The spectrum slice of a tile: the L / 2 + 1 rows of its columns are C / W
+// contiguous runs of the Z-tile-ordered spectrum, one per group of W = zgroup(L)
+// columns, staged one after another.
 template <int L, int C>
 __device__ __forceinline__ void zpipe_tma_ghat(const SArgs& a, int rhs, int ky, int cb, cpx<float>* S,
                                                unsigned long long* bar) {
-  static_assert(C == kZGroup, "one contiguous run per tile");
+  constexpr int W = zgroup(L), run = (L / 2 + 1) * W;
+  static_assert(C % W == 0, "whole groups");
   const int my = mirror_index(ky, L);
   const int g = a.rhs_per_ghat > 0 ? rhs / a.rhs_per_ghat : 0;
   const cpx<float>* src = reinterpret_cast<const cpx<float>*>(bmove(a.ghatZ, a.bs_ghatZ * g)) +
-                          ((long long)my * (L / kZGroup) + cb) * (L / 2 + 1) * kZGroup;
+                          ((long long)my * (L / W) + cb * (C / W)) * run;
   constexpr unsigned bytes = unsigned(L / 2 + 1) * C * unsigned(sizeof(cpx<float>));
   fence_proxy_async();
   mbar_expect_tx(bar, bytes);
-  bulk_load(S, src, bytes, bar);
+  bulk_load(S, src, bytes, bar);   // the runs of neighbouring groups follow one another
 }
 
 template <class T, int L, int C, int L1X>
@@ -1307,8 +1335,8 @@ __device__ __forceinline__ void zpipe_prefetch(const SArgs& a, int tile, int per
   const int t = tile - rhs * per_rhs;
   const int ky = ky_of_slot(t / col_blocks, L);
   const int cb = t % col_blocks;
-  const cpx<T>* src = reinterpret_cast<const cpx<T>*>(bmove(a.in, a.bs_in * rhs)) + (long long)ky * a.in_outer +
-                      (long long)cb * C;
+  const cpx<T>* src = reinterpret_cast<const cpx<T>*>(bmove(a.in, a.bs_in * rhs)) +
+                      blk_off<L>(ky, a.in_blk, a.in_outer) + (long long)cb * C;
   const int chunks = a.n_in * PER_ROW;
   constexpr int EPC = 16 / int(sizeof(cpx<T>));             // elements per chunk
   for (int k = threadIdx.x; k < chunks; k += NT) {
@@ -1320,7 +1348,7 @@ __device__ __forceinline__ void zpipe_prefetch(const SArgs& a, int tile, int per
 
 // Stage the n_in input rows of a Z tile (C columns) into S, NT threads.
 template <class T, int L, int C, int NT>
-__device__ __forceinline__ void zpipe_prefetch_rows(const SArgs& a, int tile, int per_rhs, cpx<T>* S) {
+__device__ __forceinline__ void zpipe_prefetch_rows(const SArgs& a, int tile, int per_rhs, cpx<T>* S, int tid) {
   constexpr int PER_ROW = C * int(sizeof(cpx<T>)) / 16;
   constexpr int EPC = 16 / int(sizeof(cpx<T>));
   const int col_blocks = L / C;
@@ -1328,10 +1356,10 @@ __device__ __forceinline__ void zpipe_prefetch_rows(const SArgs& a, int tile, in
   const int tl = tile - rhs * per_rhs;
   const int ky = ky_of_slot(tl / col_blocks, L);
   const int cb = tl % col_blocks;
-  const cpx<T>* src = reinterpret_cast<const cpx<T>*>(bmove(a.in, a.bs_in * rhs)) + (long long)ky * a.in_outer +
-                      (long long)cb * C;
+  const cpx<T>* src = reinterpret_cast<const cpx<T>*>(bmove(a.in, a.bs_in * rhs)) +
+                      blk_off<L>(ky, a.in_blk, a.in_outer) + (long long)cb * C;
   const int chunks = a.n_in * PER_ROW;
-  for (int k = threadIdx.x; k < chunks; k += NT) {
+  for (int k = tid; k < chunks; k += NT) {
     const int j = k / PER_ROW, cc = (k - j * PER_ROW) * EPC;
     cp_async16(S + j * C + cc, src + (long long)j * a.in_pt + cc);
   }
@@ -1339,27 +1367,239 @@ __device__ __forceinline__ void zpipe_prefetch_rows(const SArgs& a, int tile, in
 }
 
 // The spectrum slice of a tile: entries (mz, my(ky), kx) for mz in [0, L/2]
-// and kx in the tile, copied to S as [mz][C].  The Z-tile order stores the
-// FP32 spectrum in groups of kZGroup columns, [my][kx / kZGroup][mz][kZGroup];
-// a tile of C columns (C divides kZGroup) reads C of each group row.
+// and kx in the tile.  The Z-tile order stores the FP32 spectrum in groups of
+// W = zgroup(L) columns, [my][kx / W][mz][W]; a tile of whole groups is copied
+// as it lies ([group][mz][W]), a tile of C < W columns as [mz][C].
 template <class T, int L, int C, int L1X>
 __device__ __forceinline__ void zpipe_prefetch_ghat(const SArgs& a, int rhs, int ky, int cb, cpx<T>* S) {
-  static_assert(kZGroup % C == 0, "tile width must divide the spectrum group");
+  constexpr int W = zgroup(L), H = L / 2 + 1;
+  static_assert(W % C == 0 || C % W == 0, "tile width and spectrum group");
   constexpr int NT = ZPipe<L, C, T, L1X>::NT;
   const int my = mirror_index(ky, L);
   const int g = a.rhs_per_ghat > 0 ? rhs / a.rhs_per_ghat : 0;
   const int kx0 = cb * C;
-  const int grp = kx0 / kZGroup, off = kx0 - grp * kZGroup;
+  const int grp = kx0 / W, off = kx0 - grp * W;
   const cpx<T>* src = reinterpret_cast<const cpx<T>*>(bmove(a.ghatZ, a.bs_ghatZ * g)) +
-                      ((long long)my * (L / kZGroup) + grp) * (L / 2 + 1) * kZGroup + off;
+                      ((long long)my * (L / W) + grp) * H * W + off;
   constexpr int EPC = 16 / int(sizeof(cpx<T>));
-  constexpr int PER_ROW = C / EPC;
-  constexpr int chunks = (L / 2 + 1) * PER_ROW;
+  constexpr int PER_ROW = (C < W ? C : W) / EPC;
+  constexpr int chunks = H * C / EPC;
   for (int k = threadIdx.x; k < chunks; k += NT) {
-    const int row = k / PER_ROW, cc = (k - row * PER_ROW) * EPC;
-    cp_async16(S + row * C + cc, src + row * kZGroup + cc);
+    if constexpr (C < W) {
+      const int row = k / PER_ROW, cc = (k - row * PER_ROW) * EPC;
+      cp_async16(S + row * C + cc, src + row * W + cc);
+    } else {
+      cp_async16(S + k * EPC, src + k * EPC);
+    }
   }
   cp_async_commit();
+}
+
+// ---------------------------------------------------------------------------
+// FP32 Z convolution in groups of C columns that do not wait for one another:
+// the G groups of a CTA share the twiddle table and nothing else, each with its
+// own exchange buffer, staging buffer, barriers and tiles.  With the whole CTA
+// in step the FMA pipe and the shared-memory pipe of an SM took turns (59% and
+// 50% busy, the sum of their times); groups out of phase overlap them (67% and
+// 68%).  Tile by tile it is k_zconv_pipe's two stages; the column pitch of the
+// exchange spreads the columns and rows of a half warp over 16 different 8-byte
+// banks (2 modulo 4 for 8 columns, 4 modulo 8 for 4), and the twiddle table is
+// padded to L2 + 1 entries a row for the same reason (a square split reads it
+// by its symmetry instead).  The spectrum is grouped by C columns (zgroup), so
+// a tile's slice is one contiguous run.
+//   L = 1024, 2 groups of 8: n = 512 3.18 -> 2.94 ms
+//   mixed lengths, 1 group of 8 and several CTAs per SM: n = 260 (576 points) 0.55 ms,
+//   where the 1024-point pass on the same grid takes 3.06 ms
+// At L = 512 two 16-column CTAs in step each are faster (n = 256: 0.362 ms,
+// groups of 8 0.378, of 4 0.379), and so are four at L = 256.
+// ---------------------------------------------------------------------------
+template <int L, int C, int G>
+struct ZGroups {
+  static constexpr int L1 = Split<L>::L1, L2 = Split<L>::L2;
+  static constexpr int NT = C * L2, NI = L1 / L2;                     // threads of a group
+  static constexpr int PK = L2 + 1, PKI = L1 + 1;
+  static constexpr int MOD = C == 8 ? 4 : 8, REM = MOD / 2;
+  static constexpr int pitch(int v) { return v + ((REM - v % MOD) + MOD) % MOD; }
+  static constexpr int PC = pitch(L1 * PK), PCI = pitch(L2 * PKI);
+  static constexpr int PT = L1 == L2 ? L2 : L2 + 1;
+  static constexpr int r16(int v) { return (v + 15) / 16 * 16; }      // regions start on 128 bytes
+  static constexpr int E_ELEMS = r16(C * (PC > PCI ? PC : PCI));
+  static constexpr int S_ELEMS = r16((L / 2 + 1) * C);
+  static constexpr int TW_ELEMS = r16(L1 * PT);
+  static constexpr size_t SMEM_BYTES =
+      (size_t(TW_ELEMS) + size_t(G) * (E_ELEMS + S_ELEMS)) * sizeof(cpx<float>) + 128 + 8 * G + 8;
+  // one group per CTA: CTAs per SM the register budget is set for: as many as
+  // shared memory holds, at 96 registers a thread or more
+  static constexpr int fit = int(227 * 1024 / (SMEM_BYTES + 1024));
+  static constexpr int warps = (G * NT + 31) / 32;
+  static constexpr int MINB = fit * warps > 21 ? 21 / warps : fit;
+};
+
+// Barrier of the NT threads of group g (the CTA's own barrier when it is the only group).
+template <int G, int NT>
+__device__ __forceinline__ void group_sync(int g) {
+  if constexpr (G == 1) __syncthreads();
+  else asm volatile("barrier.cta.sync %0, %1;" ::"r"(1 + g), "r"(NT) : "memory");
+}
+template <int G, int NT>
+__device__ __forceinline__ bool group_sync_or(int g, bool v) {
+  if constexpr (G == 1) return __syncthreads_or(v) != 0;
+  unsigned r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.or.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"(unsigned(v)), "r"(1 + g), "r"(NT)
+      : "memory");
+  return r != 0;
+}
+
+template <int L, int C, int G>
+__device__ __forceinline__ void zconv_groups(const SArgs& a) {
+  using T = float;
+  using Z = ZGroups<L, C, G>;
+  constexpr int L1 = Z::L1, L2 = Z::L2, NT = Z::NT, NI = Z::NI;
+  constexpr int PK = Z::PK, PC = Z::PC, PKI = Z::PKI, PCI = Z::PCI, PT = Z::PT;
+  constexpr int kSlice = (L / 2 + 1) * C;
+  static_assert(C == zgroup(L) && (G == 1 || NT % 32 == 0), "one run of the spectrum per tile; whole warps");
+  extern __shared__ __align__(128) unsigned char smraw[];
+  unsigned char* base = smraw + ((128u - (smem_addr(smraw) & 127u)) & 127u);
+  const int g = G == 1 ? 0 : int(threadIdx.x) / NT;
+  const int tid = G == 1 ? int(threadIdx.x) : int(threadIdx.x) - g * NT;
+  cpx<T>* TW = reinterpret_cast<cpx<T>*>(base);
+  cpx<T>* E = TW + Z::TW_ELEMS + g * (Z::E_ELEMS + Z::S_ELEMS);
+  cpx<T>* S = E + Z::E_ELEMS;
+  unsigned long long* bar =
+      reinterpret_cast<unsigned long long*>(TW + Z::TW_ELEMS + G * (Z::E_ELEMS + Z::S_ELEMS)) + g;
+  const int c = tid % C, jl = tid / C;
+  const cpx<T>* twg = reinterpret_cast<const cpx<T>*>(a.twL);
+  for (int i = threadIdx.x; i < L; i += G * NT) {
+    const int k1 = i / L2, j = i - k1 * L2;
+    TW[k1 * PT + j] = twg[j * k1];
+  }
+  constexpr int col_blocks = L / C;
+  constexpr int per_rhs = L * col_blocks;
+  const int ntiles = per_rhs * (a.nrhs > 1 ? a.nrhs : 1);
+  const int step = gridDim.x * G;
+  const bool tma = a.zrows_ok != 0;   // uniform over the grid
+  unsigned phase = 0;
+  if (tma && tid == 0) {
+    mbar_init(bar, 1);
+    fence_mbar_init();
+  }
+  __syncthreads();   // the table; from here on the groups go their own ways
+  // Wait for the staged copy, bounded as in k_zconv_pipe; false: the group leaves.
+  auto staged = [&]() -> bool {
+    if (tma) {
+      const bool ok = mbar_wait(bar, phase);
+      if (group_sync_or<G, NT>(g, !ok)) {
+        if (tid == 0 && a.err != nullptr) atomicExch(a.err, 1);
+        if (!ok) mbar_wait(bar, phase);
+        return false;
+      }
+      phase ^= 1u;
+      return true;
+    }
+    cp_async_wait_all();
+    group_sync<G, NT>(g);
+    return true;
+  };
+  auto stage_rows = [&](int t) {
+    if (!tma) {
+      zpipe_prefetch_rows<T, L, C, NT>(a, t, per_rhs, S, tid);
+    } else if (tid == 0) {
+      zpipe_tma_rows<L, C>(a, t, per_rhs, S, bar);
+    }
+  };
+  auto stage_slice = [&](int rhs, int ky, int cb) {
+    const int gk = a.rhs_per_ghat > 0 ? rhs / a.rhs_per_ghat : 0;
+    const cpx<T>* src = reinterpret_cast<const cpx<T>*>(bmove(a.ghatZ, a.bs_ghatZ * gk)) +
+                        ((long long)mirror_index(ky, L) * col_blocks + cb) * kSlice;
+    if (!tma) {
+      for (int k = tid; k < kSlice / 2; k += NT) cp_async16(S + 2 * k, src + 2 * k);
+      cp_async_commit();
+    } else if (tid == 0) {
+      constexpr unsigned bytes = unsigned(kSlice) * unsigned(sizeof(cpx<T>));
+      fence_proxy_async();
+      mbar_expect_tx(bar, bytes);
+      bulk_load(S, src, bytes, bar);
+    }
+  };
+
+  dep_wait();
+  int tile = next_live_tile(a, blockIdx.x * G + g, step, per_rhs, ntiles);
+  if (tile < ntiles) stage_rows(tile);
+  while (tile < ntiles) {
+    const int rhs = tile / per_rhs;
+    const int tl = tile - rhs * per_rhs;
+    const int ky = ky_of_slot(tl / col_blocks, L);
+    const int cb = tl % col_blocks;
+    const int next = next_live_tile(a, tile + step, step, per_rhs, ntiles);
+    if (!staged()) return;   // rows visible; the previous tile is done with E
+    cpx<T> r[L1];
+#pragma unroll
+    for (int j1 = 0; j1 < L1; ++j1) {
+      r[j1] = czero<T>();
+      if (j1 < L1 / 2) {
+        const int j = j1 * L2 + jl;
+        if (j < a.n_in) r[j1] = S[j * C + c];
+      }
+    }
+    group_sync<G, NT>(g);   // staging buffer consumed
+    stage_slice(rhs, ky, cb);
+    dft<L1, -1, true>(r);
+    const cpx<T>* tj = TW + jl;
+#pragma unroll
+    for (int k1 = 1; k1 < L1; ++k1) r[k1] = tw_mul_val<-1>(r[k1], tj[k1 * PT]);
+#pragma unroll
+    for (int k1 = 0; k1 < L1; ++k1) E[c * PC + k1 * PK + jl] = r[k1];
+    if (!staged()) return;   // exchange and spectrum slice visible
+    cpx<T> b[NI][L2];
+#pragma unroll
+    for (int it = 0; it < NI; ++it) {
+      const int s = tid + it * NT;
+      const int c2 = s % C, k1 = s / C;
+#pragma unroll
+      for (int j = 0; j < L2; ++j) b[it][j] = E[c2 * PC + k1 * PK + j];
+      dft<L2, -1, false>(b[it]);
+      const cpx<T>* lo = S + k1 * C + c2;          // kz = k1 + L1 k2 below L/2, L - kz from there on
+      const cpx<T>* hi = S + (L - k1) * C + c2;
+#pragma unroll
+      for (int k2 = 0; k2 < L2; ++k2)
+        b[it][k2] = cmul(b[it][k2], k2 < L2 / 2 ? lo[k2 * L1 * C] : hi[-k2 * L1 * C]);
+      dft<L2, +1, false>(b[it]);
+#pragma unroll
+      for (int ja = 1; ja < L2; ++ja)
+        b[it][ja] = tw_mul_val<+1>(b[it][ja], L1 == L2 ? TW[ja * PT + k1] : TW[k1 * PT + ja]);
+    }
+    group_sync<G, NT>(g);   // exchange and slice fully read
+    if (next < ntiles) stage_rows(next);
+#pragma unroll
+    for (int it = 0; it < NI; ++it) {
+      const int s = tid + it * NT;
+      const int c2 = s % C, k1 = s / C;
+#pragma unroll
+      for (int ja = 0; ja < L2; ++ja) E[c2 * PCI + ja * PKI + k1] = b[it][ja];
+    }
+    group_sync<G, NT>(g);
+#pragma unroll
+    for (int k1 = 0; k1 < L1; ++k1) r[k1] = E[c * PCI + jl * PKI + k1];
+    dft_low<L1, +1>(r);
+    cpx<T>* out = reinterpret_cast<cpx<T>*>(bmove(a.out, a.bs_out * rhs)) + blk_off<L>(ky, a.out_blk, a.out_outer) + (long long)cb * C;
+#pragma unroll
+    for (int jb = 0; jb < L1 / 2; ++jb) {
+      const int j = jl + L2 * jb;
+      if (j < a.n_out) out[(long long)j * a.out_pt + c] = r[jb];
+    }
+    tile = next;
+  }
+  cp_async_wait_all();
+}
+
+// The mixed lengths: one group per CTA, several CTAs per SM.
+template <int L>
+__global__ void __launch_bounds__(ZGroups<L, 8, 1>::NT, ZGroups<L, 8, 1>::MINB)
+k_zconv_mix(const __grid_constant__ SArgs a) {
+  zconv_groups<L, 8, 1>(a);
 }
 
 template <class T, int L, int C, int L1X = Split<L>::L1>
@@ -1368,6 +1608,9 @@ __global__ void __launch_bounds__(ZPipe<L, C, T, L1X>::NT,
 k_zconv_pipe(const __grid_constant__ SArgs a) {
   using TL = Tile<L, C, T, L1X>;
   using ZP = ZPipe<L, C, T, L1X>;
+  if constexpr (ZP::GROUPS) {
+    zconv_groups<L, ZP::GC, C / ZP::GC>(a);
+  } else {
   constexpr bool GZ = ZP::GZ;
   constexpr int L1 = TL::L1, L2 = TL::L2, NT = TL::NT, NI = L1 / L2;
   constexpr int PK = TL::PK, PC = TL::PC, PKI = TL::PKI, PCI = TL::PCI;
@@ -1491,11 +1734,22 @@ k_zconv_pipe(const __grid_constant__ SArgs a) {
         // kz = k1 + L1 k2 has mirror index kz below L/2 and L - kz from L/2 on
         // (k2 >= L2/2), so the slice [mz][C] is read at constant offsets from
         // two base pointers
-        const cpx<T>* lo = S + k1 * C + c2;
-        const cpx<T>* hi = S + (L - k1) * C + c2;
+        // (the slice lies as [mz][C], or as one such run per group of W columns)
+        constexpr int W = zgroup(L) < C ? zgroup(L) : C;
+        if constexpr (W == C) {
+          const cpx<T>* lo = S + k1 * C + c2;
+          const cpx<T>* hi = S + (L - k1) * C + c2;
 #pragma unroll
-        for (int k2 = 0; k2 < L2; ++k2)
-          b[it][k2] = cmul(b[it][k2], k2 < L2 / 2 ? lo[k2 * L1 * C] : hi[-k2 * L1 * C]);
+          for (int k2 = 0; k2 < L2; ++k2)
+            b[it][k2] = cmul(b[it][k2], k2 < L2 / 2 ? lo[k2 * L1 * C] : hi[-k2 * L1 * C]);
+        } else {
+          const cpx<T>* run = S + (c2 / W) * (L / 2 + 1) * W + c2 % W;
+          const cpx<T>* lo = run + k1 * W;
+          const cpx<T>* hi = run + (L - k1) * W;
+#pragma unroll
+          for (int k2 = 0; k2 < L2; ++k2)
+            b[it][k2] = cmul(b[it][k2], k2 < L2 / 2 ? lo[k2 * L1 * W] : hi[-k2 * L1 * W]);
+        }
       } else {
         const int mx = mirror_index(cb * C + c2, L);
 #pragma unroll
@@ -1528,7 +1782,7 @@ k_zconv_pipe(const __grid_constant__ SArgs a) {
 #pragma unroll
     for (int k1 = 0; k1 < L1; ++k1) r[k1] = E[c * PCI + jl * PKI + k1];
     dft<L1, +1, false>(r);
-    cpx<T>* out = reinterpret_cast<cpx<T>*>(bmove(a.out, a.bs_out * rhs)) + (long long)ky * a.out_outer + (long long)cb * C;
+    cpx<T>* out = reinterpret_cast<cpx<T>*>(bmove(a.out, a.bs_out * rhs)) + blk_off<L>(ky, a.out_blk, a.out_outer) + (long long)cb * C;
 #pragma unroll
     for (int jb = 0; jb < L1 / 2; ++jb) {
       const int j = jl + L2 * jb;
@@ -1537,182 +1791,12 @@ k_zconv_pipe(const __grid_constant__ SArgs a) {
     tile = next;
   }
   cp_async_wait_all();
-}
-
-// ---------------------------------------------------------------------------
-// FP32 Z convolution at the mixed lengths: k_zconv_pipe's stages on 8-column
-// tiles, several small CTAs per SM (their arithmetic and shared-memory phases
-// overlap; one 16-column CTA per SM would take turns).  The column pitch of
-// the exchange is 2 modulo 4, so that the 8 columns x 2 rows of a half warp
-// fall into 16 different 8-byte banks, and the twiddle table is padded to
-// L2 + 1 entries a row for the same reason (square splits read it by its
-// symmetry instead).  The spectrum is grouped by 8 columns (zgroup), so a
-// tile's slice is one contiguous run.  n = 260, 576 points: 0.56 ms, where
-// the 1024-point pass on the same grid takes 3.06 ms.
-// ---------------------------------------------------------------------------
-template <int L>
-struct ZMix {
-  static constexpr int C = 8;
-  static constexpr int L1 = Split<L>::L1, L2 = Split<L>::L2;
-  static constexpr int NT = C * L2, NI = L1 / L2;
-  static constexpr int PK = L2 + 1, PKI = L1 + 1;
-  static constexpr int pitch(int v) { return v + (6 - v % 4) % 4; }   // next v = 2 (mod 4)
-  static constexpr int PC = pitch(L1 * PK), PCI = pitch(L2 * PKI);
-  static constexpr int PT = L1 == L2 ? L2 : L2 + 1;
-  static constexpr int r16(int v) { return (v + 15) / 16 * 16; }      // regions start on 128 bytes
-  static constexpr int E_ELEMS = r16(C * (PC > PCI ? PC : PCI));
-  static constexpr int S_ELEMS = r16((L / 2 + 1) * C);
-  static constexpr int TW_ELEMS = r16(L1 * PT);
-  static constexpr size_t SMEM_BYTES = size_t(E_ELEMS + S_ELEMS + TW_ELEMS) * sizeof(cpx<float>) + 128 + 16;
-  // CTAs per SM the register budget is set for: as many as shared memory holds,
-  static constexpr int fit = int(227 * 1024 / (SMEM_BYTES + 1024));
-  // at 96 registers a thread or more
-  static constexpr int warps = (NT + 31) / 32;
-  static constexpr int MINB = fit * warps > 21 ? 21 / warps : fit;
-};
-
-template <int L>
-__global__ void __launch_bounds__(ZMix<L>::NT, ZMix<L>::MINB) k_zconv_mix(const __grid_constant__ SArgs a) {
-  using T = float;
-  using Z = ZMix<L>;
-  constexpr int C = Z::C, L1 = Z::L1, L2 = Z::L2, NT = Z::NT, NI = Z::NI;
-  constexpr int PK = Z::PK, PC = Z::PC, PKI = Z::PKI, PCI = Z::PCI, PT = Z::PT;
-  constexpr int kSlice = (L / 2 + 1) * C;
-  extern __shared__ __align__(128) unsigned char smraw[];
-  unsigned char* base = smraw + ((128u - (smem_addr(smraw) & 127u)) & 127u);
-  cpx<T>* E = reinterpret_cast<cpx<T>*>(base);
-  cpx<T>* S = E + Z::E_ELEMS;
-  cpx<T>* TW = S + Z::S_ELEMS;
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(TW + Z::TW_ELEMS);
-  const int tid = threadIdx.x;
-  const int c = tid % C, jl = tid / C;
-  const cpx<T>* twg = reinterpret_cast<const cpx<T>*>(a.twL);
-  for (int i = tid; i < L; i += NT) {
-    const int k1 = i / L2, j = i - k1 * L2;
-    TW[k1 * PT + j] = twg[j * k1];
   }
-  constexpr int col_blocks = L / C;
-  constexpr int per_rhs = L * col_blocks;
-  const int ntiles = per_rhs * (a.nrhs > 1 ? a.nrhs : 1);
-  const int step = gridDim.x;
-  const bool tma = a.zrows_ok != 0;   // uniform over the grid
-  unsigned phase = 0;
-  if (tma && tid == 0) {
-    mbar_init(bar, 1);
-    fence_mbar_init();
-  }
-  __syncthreads();
-  // Wait for the staged copy, bounded as in k_zconv_pipe; false: leave.
-  auto staged = [&]() -> bool {
-    if (tma) {
-      const bool ok = mbar_wait(bar, phase);
-      if (__syncthreads_or(!ok)) {
-        if (tid == 0 && a.err != nullptr) atomicExch(a.err, 1);
-        if (!ok) mbar_wait(bar, phase);
-        return false;
-      }
-      phase ^= 1u;
-      return true;
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    return true;
-  };
-  auto stage_rows = [&](int t) {
-    if (!tma) {
-      zpipe_prefetch_rows<T, L, C, NT>(a, t, per_rhs, S);
-    } else if (tid == 0) {
-      zpipe_tma_rows<L, C>(a, t, per_rhs, S, bar);
-    }
-  };
-  auto stage_slice = [&](int rhs, int ky, int cb) {
-    const int g = a.rhs_per_ghat > 0 ? rhs / a.rhs_per_ghat : 0;
-    const cpx<T>* src = reinterpret_cast<const cpx<T>*>(bmove(a.ghatZ, a.bs_ghatZ * g)) +
-                        ((long long)mirror_index(ky, L) * col_blocks + cb) * kSlice;
-    if (!tma) {
-      for (int k = tid; k < kSlice / 2; k += NT) cp_async16(S + 2 * k, src + 2 * k);
-      cp_async_commit();
-    } else if (tid == 0) {
-      constexpr unsigned bytes = unsigned(kSlice) * unsigned(sizeof(cpx<T>));
-      fence_proxy_async();
-      mbar_expect_tx(bar, bytes);
-      bulk_load(S, src, bytes, bar);
-    }
-  };
-
-  dep_wait();
-  int tile = next_live_tile(a, blockIdx.x, step, per_rhs, ntiles);
-  if (tile < ntiles) stage_rows(tile);
-  while (tile < ntiles) {
-    const int rhs = tile / per_rhs;
-    const int tl = tile - rhs * per_rhs;
-    const int ky = ky_of_slot(tl / col_blocks, L);
-    const int cb = tl % col_blocks;
-    const int next = next_live_tile(a, tile + step, step, per_rhs, ntiles);
-    if (!staged()) return;   // rows visible; the previous tile is done with E
-    cpx<T> r[L1];
-#pragma unroll
-    for (int j1 = 0; j1 < L1; ++j1) {
-      r[j1] = czero<T>();
-      if (j1 < L1 / 2) {
-        const int j = j1 * L2 + jl;
-        if (j < a.n_in) r[j1] = S[j * C + c];
-      }
-    }
-    __syncthreads();   // staging buffer consumed
-    stage_slice(rhs, ky, cb);
-    dft<L1, -1, true>(r);
-    const cpx<T>* tj = TW + jl;
-#pragma unroll
-    for (int k1 = 1; k1 < L1; ++k1) r[k1] = tw_mul_val<-1>(r[k1], tj[k1 * PT]);
-#pragma unroll
-    for (int k1 = 0; k1 < L1; ++k1) E[c * PC + k1 * PK + jl] = r[k1];
-    if (!staged()) return;   // exchange and spectrum slice visible
-    cpx<T> b[NI][L2];
-#pragma unroll
-    for (int it = 0; it < NI; ++it) {
-      const int s = tid + it * NT;
-      const int c2 = s % C, k1 = s / C;
-#pragma unroll
-      for (int j = 0; j < L2; ++j) b[it][j] = E[c2 * PC + k1 * PK + j];
-      dft<L2, -1, false>(b[it]);
-      const cpx<T>* lo = S + k1 * C + c2;          // kz = k1 + L1 k2 below L/2, L - kz from there on
-      const cpx<T>* hi = S + (L - k1) * C + c2;
-#pragma unroll
-      for (int k2 = 0; k2 < L2; ++k2)
-        b[it][k2] = cmul(b[it][k2], k2 < L2 / 2 ? lo[k2 * L1 * C] : hi[-k2 * L1 * C]);
-      dft<L2, +1, false>(b[it]);
-#pragma unroll
-      for (int ja = 1; ja < L2; ++ja)
-        b[it][ja] = tw_mul_val<+1>(b[it][ja], L1 == L2 ? TW[ja * PT + k1] : TW[k1 * PT + ja]);
-    }
-    __syncthreads();   // exchange and slice fully read
-    if (next < ntiles) stage_rows(next);
-#pragma unroll
-    for (int it = 0; it < NI; ++it) {
-      const int s = tid + it * NT;
-      const int c2 = s % C, k1 = s / C;
-#pragma unroll
-      for (int ja = 0; ja < L2; ++ja) E[c2 * PCI + ja * PKI + k1] = b[it][ja];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k1 = 0; k1 < L1; ++k1) r[k1] = E[c * PCI + jl * PKI + k1];
-    dft_low<L1, +1>(r);
-    cpx<T>* out = reinterpret_cast<cpx<T>*>(bmove(a.out, a.bs_out * rhs)) + (long long)ky * a.out_outer + (long long)cb * C;
-#pragma unroll
-    for (int jb = 0; jb < L1 / 2; ++jb) {
-      const int j = jl + L2 * jb;
-      if (j < a.n_out) out[(long long)j * a.out_pt + c] = r[jb];
-    }
-    tile = next;
-  }
-  cp_async_wait_all();
 }
 
 template <int L>
 cudaError_t launch_zconv_mix_L(SArgs a, cudaStream_t s, bool setup, int sm_count) {
-  using Z = ZMix<L>;
+  using Z = ZGroups<L, 8, 1>;
   auto kfn = k_zconv_mix<L>;
   static int per_sm = 0;   // resident CTAs per SM, measured once at set-up
   if (setup) {
@@ -1723,7 +1807,7 @@ cudaError_t launch_zconv_mix_L(SArgs a, cudaStream_t s, bool setup, int sm_count
     per_sm = (e == cudaSuccess && nb > 0) ? nb : 1;
     return e;
   }
-  const long long ntiles = (long long)L * (L / Z::C) * std::max(1, a.nrhs);
+  const long long ntiles = (long long)L * (L / 8) * std::max(1, a.nrhs);
   const int resident = a.cta_cap > 0 ? std::min(std::max(1, per_sm), a.cta_cap) : std::max(1, per_sm);
   const unsigned gx = unsigned(std::max(1LL, std::min(ntiles, (long long)std::max(1, sm_count) * resident)));
   return launch_dep(kfn, dim3(gx), Z::NT, Z::SMEM_BYTES, s, a);
@@ -1767,7 +1851,7 @@ __global__ void __launch_bounds__(ZSmem<L, C, T>::NT, ZSmem<L, C, T>::MINB) k_zc
 
   dep_wait();
   int tile = next_live_tile(a, blockIdx.x, step, per_rhs, ntiles);
-  if (tile < ntiles) zpipe_prefetch_rows<T, L, C, NT>(a, tile, per_rhs, S);
+  if (tile < ntiles) zpipe_prefetch_rows<T, L, C, NT>(a, tile, per_rhs, S, tid);
   while (tile < ntiles) {
     const int rhs = tile / per_rhs;
     const int tl = tile - rhs * per_rhs;
@@ -1793,7 +1877,7 @@ __global__ void __launch_bounds__(ZSmem<L, C, T>::NT, ZSmem<L, C, T>::MINB) k_zc
       for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
     }
     __syncthreads();
-    if (next < ntiles) zpipe_prefetch_rows<T, L, C, NT>(a, next, per_rhs, S);
+    if (next < ntiles) zpipe_prefetch_rows<T, L, C, NT>(a, next, per_rhs, S, tid);
     dif_middle<L, C>(X, TW, tid, NT);
     // last forward stage, spectrum and first inverse stage on the same r3 points
     const int my = mirror_index(ky, L);
@@ -1815,7 +1899,7 @@ __global__ void __launch_bounds__(ZSmem<L, C, T>::NT, ZSmem<L, C, T>::MINB) k_zc
     __syncthreads();
     dit_middle<L, C>(X, TW, tid, NT);
     // last inverse stage (M = L), keep rows z < n_out
-    cpx<T>* out = reinterpret_cast<cpx<T>*>(bmove(a.out, a.bs_out * rhs)) + (long long)ky * a.out_outer + (long long)cb * C;
+    cpx<T>* out = reinterpret_cast<cpx<T>*>(bmove(a.out, a.bs_out * rhs)) + blk_off<L>(ky, a.out_blk, a.out_outer) + (long long)cb * C;
     for (int g = tid; g < C * S8; g += NT) {
       const int c = g % C, j = g / C;
       cpx<T> v[8];
@@ -1861,6 +1945,17 @@ cudaError_t launch_zconv_smem_L(SArgs a, cudaStream_t s, bool setup, int sm_coun
 // through a tensor map of T1 for 16-column tiles (boxes of up to 256 rows)
 // and by cp.async otherwise.
 // ---------------------------------------------------------------------------
+// CTAs per SM the register budget of a Y kernel at a mixed length is set for:
+// what shared memory holds, at 96 registers a thread or more (with 40-point
+// stages 160 in the forward, 128 in the inverse pass: n = 400 0.64 and 0.59 ms,
+// against 0.67 at 128 and 0.66 at 160).
+template <int L>
+constexpr int y_mix_minb(int nt, size_t smem, bool inv) {
+  const int fit = int(227 * 1024 / (smem + 1024)), warps = (nt + 31) / 32;
+  const int most = (L == 800 ? (inv ? 15 : 12) : 21) / warps;
+  return fit < most ? fit : most;
+}
+
 template <int L, int C, class T, int L1X = Split<L>::L1>
 struct YPipe {
   using TL = Tile<L, C, T, L1X>;
@@ -1908,7 +2003,8 @@ __device__ __forceinline__ void ypipe_prefetch(const SArgs& a, int tile, int per
 
 template <class T, int L, int C, int L1X = Split<L>::L1>
 __global__ void __launch_bounds__(YPipe<L, C, T, L1X>::NT,
-                                  (L > 1024 || L1X >= 64 || YPipe<L, C, T, L1X>::NT >= 512)
+                                  is_mixed_len(L) ? y_mix_minb<L>(YPipe<L, C, T, L1X>::NT, YPipe<L, C, T, L1X>::SMEM_BYTES, false)
+                                  : (L > 1024 || L1X >= 64 || YPipe<L, C, T, L1X>::NT >= 512)
                                       ? 1 : (YPipe<L, C, T, L1X>::NT >= 256 ? 2 : 512 / YPipe<L, C, T, L1X>::NT))
 k_yfwd_pipe(const __grid_constant__ SArgs a) {
   using TL = Tile<L, C, T, L1X>;
@@ -1998,10 +2094,11 @@ k_yfwd_pipe(const __grid_constant__ SArgs a) {
 #pragma unroll
       for (int j = 0; j < L2; ++j) b[j] = E[c2 * PC + k1 * PK + j];
       dft<L2, -1, false>(b);
+      const long long o = blk_off<L>(k1, a.out_blk, a.out_pt) + c2;
 #pragma unroll
       for (int k2 = 0; k2 < L2; ++k2) {
         const int k = k1 + L1 * k2;
-        if (k < a.n_out) out[(long long)k * a.out_pt + c2] = b[k2];
+        if (k < a.n_out) out[blk_at<L, L1>(o, k1, k2, a.out_blk, a.out_pt)] = b[k2];
       }
     }
     tile = next;
@@ -2039,14 +2136,28 @@ __device__ __forceinline__ void yinv_prefetch(const SArgs& a, int tile, int per_
                           (long long)cb * C;
   for (int k = threadIdx.x; k < L * PER_ROW; k += NT) {
     const int j = k / PER_ROW, cc = (k - j * PER_ROW) * 2;
-    cp_async16(B + j * C + cc, src + (long long)j * a.in_pt + cc);
+    cp_async16(B + j * C + cc, src + blk_off<L>(j, a.in_blk, a.in_pt) + cc);
   }
   cp_async_commit();
 }
 
+// The L input rows of a Y-inverse tile: boxes of a.zbox rows, whole blocks of ky.
+template <int L, int C>
+__device__ __forceinline__ void yinv_tma_rows(const SArgs& a, int rhs, int outer, int cb, cpx<float>* S,
+                                              unsigned long long* bar) {
+  constexpr int BK = yblk(L);
+  const int nbox = L / a.zbox;
+  fence_proxy_async();
+  mbar_expect_tx(bar, unsigned(L * C * int(sizeof(cpx<float>))));
+  for (int q = 0; q < nbox; ++q)
+    tma_load_5d(S + q * a.zbox * C, &a.zrows, cb * C, BK == L ? q * a.zbox : 0, BK == L ? 0 : q * (a.zbox / BK), outer,
+                rhs, bar);
+}
+
 template <int L, int C, int L1X = Split<L>::L1>
 __global__ void __launch_bounds__(YInvPipe<L, C, L1X>::NT,
-                                  (L > 1024 || L1X >= 64 || YInvPipe<L, C, L1X>::NT >= 512)
+                                  is_mixed_len(L) ? y_mix_minb<L>(YInvPipe<L, C, L1X>::NT, YInvPipe<L, C, L1X>::SMEM_BYTES, true)
+                                  : (L > 1024 || L1X >= 64 || YInvPipe<L, C, L1X>::NT >= 512)
                                       ? 1 : (YInvPipe<L, C, L1X>::NT >= 256 ? 2 : 512 / YInvPipe<L, C, L1X>::NT))
 k_yinv_pipe(const __grid_constant__ SArgs a) {
   using T = float;
@@ -2083,7 +2194,7 @@ k_yinv_pipe(const __grid_constant__ SArgs a) {
         if (tid == 0) {
           const int rt = t / per_rhs, tt = t - rt * per_rhs;
           const int o = tt / a.col_blocks;
-          ypipe_tma_rows<C>(a, rt, o, tt - o * a.col_blocks, L, B, bar);
+          yinv_tma_rows<L, C>(a, rt, o, tt - o * a.col_blocks, B, bar);
         }
         return;
       }

@@ -47,18 +47,21 @@ def test_sources_define_the_restated_lengths():
         assert 8 * r2 * r3 == L and L1 % (L // L1) == 0 and (L // L1) % 2 == 0
 
 
-@pytest.mark.parametrize("L", MIX)
-def test_zconv_mix_indices(L):
-    L1 = MIX[L][2]
-    L2, C = L // L1, 8
+@pytest.mark.parametrize("L,C,G", [(L, 8, 1) for L in MIX] + [(1024, 8, 2)])
+def test_zconv_group_indices(L, C, G):
+    """Z pass in G groups of C columns per CTA (zconv_groups)."""
+    L1 = MIX[L][2] if L in MIX else 32
+    L2 = L // L1
     NT, NI = C * L2, L1 // L2
     r16 = lambda v: -(-v // 16) * 16                                    # noqa: E731
-    pitch = lambda v: v + (6 - v % 4) % 4                               # noqa: E731
+    mod = 4 if C == 8 else 8
+    pitch = lambda v: v + (mod // 2 - v % mod + mod) % mod              # noqa: E731
     PK, PKI = L2 + 1, L1 + 1
     PC, PCI = pitch(L1 * PK), pitch(L2 * PKI)
     PT = L2 if L1 == L2 else L2 + 1
     E, S, TW = r16(C * max(PC, PCI)), r16((L // 2 + 1) * C), r16(L1 * PT)
-    assert PC % 4 == 2 and PCI % 4 == 2 and (E + S + TW) * 8 + 144 <= SMEM_MAX and L % C == 0
+    assert (TW + G * (E + S)) * 8 + 136 + 8 * G <= SMEM_MAX and L % (C * G) == 0
+    assert G == 1 or NT % 32 == 0 and G < 16                            # whole warps; named barriers 1..G
     tid, j1 = grid(NT, L1 // 2)
     assert ((j1 * L2 + tid // C) * C + tid % C).max() < (L // 2) * C
     tid, k1 = grid(NT, L1)
@@ -147,6 +150,42 @@ def test_prime_factor_map(R):
     t = np.fft.fft(np.fft.fft(a[(Q * n1 + P * n2) % R], axis=1), axis=0)
     k = np.arange(R)
     assert np.allclose(t[k % Q, k % P], np.fft.fft(a))
+
+
+def yblk(L):
+    if L < 256:
+        return L
+    if L & (L - 1):
+        return 40 if L == 800 else L
+    return 64 if L == 256 else 32
+
+
+@pytest.mark.parametrize("L", [64, 128, 144, 200, 256, 288, 400, 512, 576, 800, 1024, 2048])
+def test_blocked_scratch_layout(L):
+    """T2 in blocks of yblk(L) values of ky: every point has its own place, the
+    steps of the kernels move the block and the place in it by constant amounts
+    where they are whole blocks or divide one, and the boxes
+    of the Y-inverse rows are whole blocks of at most 256 rows."""
+    B, n = yblk(L), 3
+    assert L % B == 0
+    ky, z = grid(L, n)
+    off = (ky // B) * n * B * L + z * B * L + (ky % B) * L
+    assert len(np.unique(off)) == off.size and off.max() == (n * L - 1) * L
+    if B == L:
+        return
+    lg = L.bit_length() - 1
+    L1 = MIX[L][2] if L in MIX else 1 << ((lg + 1) // 2)
+    assert L1 % B == 0 or B % L1 == 0
+    for step in (L1, 2 * L1, L // 8, L // 4, L // 16):                  # blk_at
+        if L % step or not (step % B == 0 or B % step == 0):
+            continue
+        k = np.arange(step)
+        for t in range(L // step):
+            kk = k + step * t
+            move = t * (step // B) * 7919 if step % B == 0 else (step * t // B) * 7919 + step * t % B
+            assert np.array_equal((kk // B) * 7919 + kk % B, (k // B) * 7919 + k % B + move)
+    nb = max(q for q in range(1, L // B + 1) if (L // B) % q == 0 and (q * B <= 256 or q == 1))
+    assert nb * B <= 256 and L % (nb * B) == 0
 
 
 def test_transform_lengths():
