@@ -1080,7 +1080,11 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_xi
 // Launchers (dispatch on the padded length)
 // ---------------------------------------------------------------------------
 template <class T> constexpr int cols_strided() { return sizeof(T) == 4 ? 8 : 4; }
+// Lines per CTA of the one-tile X kernels.  Up to L = 32 one warp: a grid of
+// n <= 16 has at most 256 lines, which blocks of 128 or 256 threads put on a
+// handful of SMs (n = 12: FP64 X passes 5 CTAs of 32 lines, 8.4 us a pass).
 template <class T, int L> constexpr int lines_contig() {
+  if (L <= 32) return 32 / Split<L>::L2;
   constexpr int want = (sizeof(T) == 4 ? 256 : 128) / Split<L>::L2;
   return want < 1 ? 1 : want;
 }
