@@ -1636,11 +1636,10 @@ static ori_status solve_B(ori_plan_s* p, int nrhs, int rhs_per_k, const double* 
     }
     return ORI_OK;
   }
-  // mixed: FP32 COCG on the normalised residual, FP64-class refinement
-  if (!warm) {
-    ORI_CUDA(cudaMemsetAsync(p->w, 0, bytes64, p->ps));
-    ORI_TRY(dev_copy(p, p->r64, p->b64, bytes64));
-  }
+  // mixed: FP32 COCG on the normalised residual, FP64-class refinement.  From
+  // a cold start w = 0 and the residual is b, neither of which is written out:
+  // the first step reads b64 and sets w (w_set), unless it ends before.
+  bool w_set = warm;
   std::vector<double> rn(rn0), err(nrhs, 0.0), recur(nrhs, 0.0);
   if (warm)
     for (int i = 0; i < nrhs; ++i) err[i] = (o.residual == ORI_DF ? kDfOperatorRelErr : 1e-14) * bnorm[i];
@@ -1661,7 +1660,8 @@ static ori_status solve_B(ori_plan_s* p, int nrhs, int rhs_per_k, const double* 
     if (budget <= 0) break;
     ORI_TRY(push_doubles(p, p->d_scl, inv.data(), nrhs, SLOT_INV));
     const int vg = vgrid(p, nrhs);
-    ORI_VEC(p, ORI_PASS_VECTOR, (k_normalise_to_f32<<<dim3(vg, nrhs), 256, 0, p->ps>>>(p->r64, p->r32, n3, p->d_scl)));
+    ORI_VEC(p, ORI_PASS_VECTOR, (k_normalise_to_f32<<<dim3(vg, nrhs), 256, 0, p->ps>>>(w_set ? p->r64 : p->b64, p->r32, n3,
+                                                                                       p->d_scl)));
     ORI_TRY(cocg_inner<float>(p, nrhs, rhs_per_k, p->x32, p->r32, p->p32, p->q32, p->S32, tin.data(), budget,
                               o.check_every, graph, ir.data()));
     if (o.history) ORI_TRY(record_history(p, nrhs, ir.data(), rn.data(), bnorm, active));
@@ -1679,7 +1679,7 @@ static ori_status solve_B(ori_plan_s* p, int nrhs, int rhs_per_k, const double* 
     }
     if (nonfinite_all) break;
     ORI_TRY(push_doubles(p, p->d_scl, scl.data(), nrhs, SLOT_ACC));
-    ORI_VEC(p, ORI_PASS_VECTOR, (k_accumulate<<<dim3(vg, nrhs), 256, 0, p->ps>>>(p->w, p->x32, n3, p->d_scl)));
+    ORI_VEC(p, ORI_PASS_VECTOR, (k_accumulate<<<dim3(vg, nrhs), 256, 0, p->ps>>>(p->w, p->x32, n3, p->d_scl, w_set ? 0 : 1)));
     // residual: updated with the FP32 operator when every active RHS allows it
     bool upd = o.resid_update != 0;
     std::vector<double> upd_err(nrhs, 0.0);
@@ -1691,6 +1691,8 @@ static ori_status solve_B(ori_plan_s* p, int nrhs, int rhs_per_k, const double* 
     for (int i = 0; i < nrhs; ++i) p->h_skip[i] = active[i] ? 0 : 1;
     ORI_TRY(push_skip(p, nrhs));
     std::vector<double> rn_new(rn);
+    if (upd && !w_set) ORI_TRY(dev_copy(p, p->r64, p->b64, bytes64));   // updated in place
+    w_set = true;
     if (upd) {
       // r -= rn B d with the FP32 operator; error <= kFp32OperatorRelErr rn |B d|
       ORI_TRY(push_doubles(p, p->d_coef, scl.data(), nrhs, SLOT_COEF));
@@ -1732,6 +1734,7 @@ static ori_status solve_B(ori_plan_s* p, int nrhs, int rhs_per_k, const double* 
       if (total[i] >= o.maxit) active[i] = 0;
     }
   }
+  if (!w_set) ORI_CUDA(cudaMemsetAsync(p->w, 0, bytes64, p->ps));
   for (int i = 0; i < nrhs; ++i) {
     info[i].iters = total[i];
     info[i].outer_iters = outer[i];

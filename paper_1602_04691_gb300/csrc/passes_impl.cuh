@@ -378,7 +378,9 @@ __device__ __forceinline__ void x_epilogue(const XArgs& a, long long i, cpx<T> v
         const cpx<double> w = reinterpret_cast<const cpx<double>*>(a.xin)[i];
         const cpx<double> b = reinterpret_cast<const cpx<double>*>(a.bvec)[i];
         const cpx<double> s = ldgc(reinterpret_cast<const cpx<double>*>(a.scale) + i);
-        const cpx<double> rr = b - (w + cmul(s, c_to_c64(v)));
+        // b - w - s v with the products fused into the sums: FP64 operations are what this epilogue costs
+        const cpx<double> vd = c_to_c64(v);
+        const cpx<double> rr = {fma(-s.x, vd.x, fma(s.y, vd.y, b.x - w.x)), fma(-s.x, vd.y, fma(-s.y, vd.x, b.y - w.y))};
         reinterpret_cast<cpx<double>*>(a.out)[i] = rr;
         acc.x += rr.x * rr.x + rr.y * rr.y;
       } break;

@@ -449,20 +449,24 @@ __global__ void k_normalise_to_f32(const cpx<double>* __restrict__ r64, cpx<floa
   }
 }
 
-// Mixed refinement: w += scale * d32.
+// Mixed refinement: w += scale * d32, or w = scale * d32 when `set` (the first
+// step from w = 0).
 __global__ void k_accumulate(cpx<double>* w, const cpx<float>* __restrict__ d32, long long n3,
-                             const double* __restrict__ scales) {
+                             const double* __restrict__ scales, int set) {
   const int rb = blockIdx.y;
   const double scale = scales[rb];
-  if (scale == 0.0) return;
+  if (scale == 0.0 && !set) return;
   w += rb * n3;
   d32 += rb * n3;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n3;
        i += (long long)gridDim.x * blockDim.x) {
-    const cpx<float> dv = d32[i];
-    cpx<double> wv = w[i];
-    wv.x += scale * double(dv.x);
-    wv.y += scale * double(dv.y);
+    cpx<double> wv = czero<double>();
+    if (!set) wv = w[i];
+    if (scale != 0.0) {   // a system left out of the step: w = 0 whatever d32 holds
+      const cpx<float> dv = d32[i];
+      wv.x += scale * double(dv.x);
+      wv.y += scale * double(dv.y);
+    }
     w[i] = wv;
   }
 }
