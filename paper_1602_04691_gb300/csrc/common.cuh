@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace ori {
 
 // ---------------------------------------------------------------------------
@@ -270,10 +272,17 @@ template <int SIGN, class T>
 __device__ __forceinline__ void dft3(cpx<T>& a, cpx<T>& b, cpx<T>& c) {
   constexpr T half = TwR<3, T>::c(1), sn = TwR<3, T>::s(1);   // cos = -1/2
   const cpx<T> t = b + c, d = b - c;
-  const cpx<T> m = axpy_r(half, t, a), n = {sn * d.x, sn * d.y};
+  const cpx<T> m = axpy_r(half, t, a);
   a = a + t;
-  b = add_i<SIGN>(m, n);
-  c = add_i<-SIGN>(m, n);
+  if constexpr (std::is_floating_point<T>::value) {   // m +- i s d with the products fused into the sums
+    constexpr T s = SIGN > 0 ? sn : -sn;
+    b = {m.x - s * d.y, m.y + s * d.x};
+    c = {m.x + s * d.y, m.y - s * d.x};
+  } else {
+    const cpx<T> n = {sn * d.x, sn * d.y};
+    b = add_i<SIGN>(m, n);
+    c = add_i<-SIGN>(m, n);
+  }
 }
 
 template <int SIGN, class T>

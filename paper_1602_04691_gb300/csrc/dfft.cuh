@@ -49,75 +49,97 @@ __device__ __forceinline__ int block_of_freq(int k0) {   // k0 < L / r3
   return (k0 & 7) * SRad<L>::r2 + (k0 >> 3);
 }
 
-// Shared-memory index of point j of column c: rows of C columns, the column
-// index swizzled by the row so that both row-wise and column-wise warp
-// accesses avoid bank conflicts.
-template <int C>
-__device__ __forceinline__ int sidx(int j, int c) { return j * C + (c ^ (j & (C - 1))); }
+// Layout of a tile in shared memory: idx(j, c, q) is the place of point j of
+// column c, q = j / (L / 8); item(g) splits a work item of `per` items a column.
+// Columns (Y and Z passes): rows of C columns, neighbouring threads on
+// neighbouring columns, the column index swizzled by the row so that both
+// row-wise and column-wise warp accesses avoid bank conflicts.
+template <int L, int C>
+struct ColTile {
+  static constexpr int ELEMS = L * C;
+  __device__ __forceinline__ static int idx(int j, int c, int) { return j * C + (c ^ (j & (C - 1))); }
+  template <int PER>
+  __device__ __forceinline__ static void item(int g, int& c, int& i) { c = g % C; i = g / C; }
+};
+// Lines (X passes): every line on its own, neighbouring threads along the line.
+// The last stage takes consecutive frequencies, whose points lie L / 8 apart:
+// one element of padding every L / 8 points puts them on different banks (in
+// rows of columns 77% of the X passes' shared loads were conflicts).
+template <int L, int C>
+struct LineTile {
+  static constexpr int ELEMS = (L + 8) * C;
+  __device__ __forceinline__ static int idx(int j, int c, int q) { return c * (L + 8) + j + q; }
+  template <int PER>
+  __device__ __forceinline__ static void item(int g, int& c, int& i) { c = g / PER; i = g - c * PER; }
+};
 
 // One in-place decimation-in-frequency stage of radix R on all C columns:
 // blocks of M points, span s = M / R; outputs multiplied by w_M^(j t').
-template <int R, int M, int SIGN, int L, int C, class T>
+template <int R, int M, int SIGN, int L, int C, template <int, int> class Lay, class T>
 __device__ __forceinline__ void dif_stage(cpx<T>* X, const cpx<T>* tw, int tid, int nt) {
+  static_assert(M == L / 8, "the middle stage: one block per eighth of the points");
   constexpr int s = M / R, step = L / M;
   for (int g = tid; g < C * (L / R); g += nt) {
-    const int c = g % C, bi = g / C;
+    int c, bi;
+    Lay<L, C>::template item<L / R>(g, c, bi);
     const int blk = bi / s, j = bi - blk * s;
     const int base = blk * M + j;
     cpx<T> v[R];
 #pragma unroll
-    for (int t = 0; t < R; ++t) v[t] = ld_stage(X + sidx<C>(base + t * s, c));
+    for (int t = 0; t < R; ++t) v[t] = ld_stage(X + Lay<L, C>::idx(base + t * s, c, blk));
     dft<R, SIGN, false>(v);
 #pragma unroll
     for (int t = 1; t < R; ++t) v[t] = twL_mul<SIGN>(v[t], tw, j * t * step);   // j t < M
 #pragma unroll
-    for (int t = 0; t < R; ++t) st_stage(X + sidx<C>(base + t * s, c), settle(v[t]));
+    for (int t = 0; t < R; ++t) st_stage(X + Lay<L, C>::idx(base + t * s, c, blk), settle(v[t]));
   }
 }
 
 // One in-place decimation-in-time stage: inputs multiplied by w_M^(j t), then
 // the radix-R butterfly.
-template <int R, int M, int SIGN, int L, int C, class T>
+template <int R, int M, int SIGN, int L, int C, template <int, int> class Lay, class T>
 __device__ __forceinline__ void dit_stage(cpx<T>* X, const cpx<T>* tw, int tid, int nt) {
+  static_assert(M == L / 8, "the middle stage: one block per eighth of the points");
   constexpr int s = M / R, step = L / M;
   for (int g = tid; g < C * (L / R); g += nt) {
-    const int c = g % C, bi = g / C;
+    int c, bi;
+    Lay<L, C>::template item<L / R>(g, c, bi);
     const int blk = bi / s, j = bi - blk * s;
     const int base = blk * M + j;
     cpx<T> v[R];
 #pragma unroll
-    for (int t = 0; t < R; ++t) v[t] = ld_stage(X + sidx<C>(base + t * s, c));
+    for (int t = 0; t < R; ++t) v[t] = ld_stage(X + Lay<L, C>::idx(base + t * s, c, blk));
 #pragma unroll
     for (int t = 1; t < R; ++t) v[t] = twL_mul<SIGN>(v[t], tw, j * t * step);   // j t < M
     dft<R, SIGN, false>(v);
 #pragma unroll
-    for (int t = 0; t < R; ++t) st_stage(X + sidx<C>(base + t * s, c), settle(v[t]));
+    for (int t = 0; t < R; ++t) st_stage(X + Lay<L, C>::idx(base + t * s, c, blk), settle(v[t]));
   }
 }
 
 // The middle stage (radix r2), forward (DIF, either sign) and inverse (DIT).
-template <int L, int C, int SIGN = -1, class T>
+template <int L, int C, int SIGN = -1, template <int, int> class Lay = ColTile, class T>
 __device__ __forceinline__ void dif_middle(cpx<T>* X, const cpx<T>* tw, int tid, int nt) {
   if constexpr (SRad<L>::r2 > 1) {
-    dif_stage<SRad<L>::r2, L / 8, SIGN, L, C>(X, tw, tid, nt);
+    dif_stage<SRad<L>::r2, L / 8, SIGN, L, C, Lay>(X, tw, tid, nt);
     __syncthreads();
   }
 }
-template <int L, int C, class T>
+template <int L, int C, template <int, int> class Lay = ColTile, class T>
 __device__ __forceinline__ void dit_middle(cpx<T>* X, const cpx<T>* tw, int tid, int nt) {
   if constexpr (SRad<L>::r2 > 1) {
-    dit_stage<SRad<L>::r2, L / 8, +1, L, C>(X, tw, tid, nt);
+    dit_stage<SRad<L>::r2, L / 8, +1, L, C, Lay>(X, tw, tid, nt);
     __syncthreads();
   }
 }
 
 // The last DIF stage of block `blk` of column c, in registers: v[t] is the
 // transform at frequency freq_of_block(blk) + (L / r3) t.
-template <int L, int C, int SIGN, class T>
+template <int L, int C, int SIGN, template <int, int> class Lay = ColTile, class T>
 __device__ __forceinline__ void dif_last(const cpx<T>* X, int blk, int c, cpx<T> (&v)[SRad<L>::r3]) {
   constexpr int r3 = SRad<L>::r3;
 #pragma unroll
-  for (int t = 0; t < r3; ++t) v[t] = ld_stage(X + sidx<C>(blk * r3 + t, c));
+  for (int t = 0; t < r3; ++t) v[t] = ld_stage(X + Lay<L, C>::idx(blk * r3 + t, c, blk / SRad<L>::r2));
   dft<r3, SIGN, false>(v);
 }
 

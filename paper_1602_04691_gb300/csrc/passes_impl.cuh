@@ -874,7 +874,7 @@ template <int L, int C, class T>
 struct LSmem {
   static constexpr int NT = is_mixed_len(L) ? stage_threads<L>(C, C >= 4 ? 256 : 160) : (C >= 4 ? 256 : 64 * C);
   static constexpr int MINB = C >= 4 ? 2 : 4;       // narrow tiles: more independent CTAs per SM
-  static constexpr size_t X_ELEMS = size_t(L) * C;
+  static constexpr size_t X_ELEMS = LineTile<L, C>::ELEMS;   // the larger of the two layouts
   static constexpr size_t SMEM_BYTES = (X_ELEMS + size_t(L)) * sizeof(cpx<T>);
 };
 
@@ -912,7 +912,7 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_st
 #pragma unroll
       for (int t = 1; t < 8; ++t) v[t] = twL_mul<-1>(v[t], TW, j * t);
 #pragma unroll
-      for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
+      for (int t = 0; t < 8; ++t) st_stage(X + ColTile<L, C>::idx(j + t * S8, c, t), settle(v[t]));
     }
     __syncthreads();
     dif_middle<L, C>(X, TW, tid, NT);
@@ -948,7 +948,7 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_st
 #pragma unroll
       for (int t = 1; t < 8; ++t) v[t] = twL_mul<+1>(v[t], TW, j * t);
 #pragma unroll
-      for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
+      for (int t = 0; t < 8; ++t) st_stage(X + ColTile<L, C>::idx(j + t * S8, c, t), settle(v[t]));
     }
     __syncthreads();
     dif_middle<L, C, +1>(X, TW, tid, NT);
@@ -996,10 +996,10 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_xf
 #pragma unroll
     for (int t = 1; t < 8; ++t) v[t] = twL_mul<-1>(v[t], TW, j * t);
 #pragma unroll
-    for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
+    for (int t = 0; t < 8; ++t) st_stage(X + LineTile<L, C>::idx(j + t * S8, c, t), settle(v[t]));
   }
   __syncthreads();
-  dif_middle<L, C>(X, TW, tid, NT);
+  dif_middle<L, C, -1, LineTile>(X, TW, tid, NT);
   cpx<T>* out = reinterpret_cast<cpx<T>*>(a.fft_out);
   // last stage: consecutive threads take consecutive frequencies, so the stores coalesce
   constexpr int r3 = SRad<L>::r3, B = L / r3;
@@ -1007,7 +1007,7 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_xf
     const int k0 = g % B, c = g / B;
     const long long line = (long long)blockIdx.x * C + c;
     cpx<T> v[r3];
-    dif_last<L, C, -1>(X, block_of_freq<L>(k0), c, v);
+    dif_last<L, C, -1, LineTile>(X, block_of_freq<L>(k0), c, v);
     if (line < a.nlines) {
 #pragma unroll
       for (int t = 0; t < r3; ++t) out[line * a.line_len_out + k0 + B * t] = settle(v[t]);
@@ -1049,10 +1049,10 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_xi
 #pragma unroll
     for (int t = 1; t < 8; ++t) v[t] = twL_mul<+1>(v[t], TW, j * t);
 #pragma unroll
-    for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
+    for (int t = 0; t < 8; ++t) st_stage(X + LineTile<L, C>::idx(j + t * S8, c, t), settle(v[t]));
   }
   __syncthreads();
-  dif_middle<L, C, +1>(X, TW, tid, NT);
+  dif_middle<L, C, +1, LineTile>(X, TW, tid, NT);
   double2 acc = make_double2(0.0, 0.0);
   cpx<T> accT = czero<T>();
   constexpr int r3 = SRad<L>::r3, B = L / r3;
@@ -1060,7 +1060,7 @@ __global__ void __launch_bounds__(LSmem<L, C, T>::NT, LSmem<L, C, T>::MINB) k_xi
     const int k0 = g % B, c = g / B;
     const long long line = (long long)blockIdx.x * C + c;
     cpx<T> v[r3];
-    dif_last<L, C, +1>(X, block_of_freq<L>(k0), c, v);
+    dif_last<L, C, +1, LineTile>(X, block_of_freq<L>(k0), c, v);
     if (line < a.nlines) {
 #pragma unroll
       for (int t = 0; t < (r3 + 1) / 2; ++t) {   // x < n <= L/2
@@ -1880,7 +1880,7 @@ __global__ void __launch_bounds__(ZSmem<L, C, T>::NT, ZSmem<L, C, T>::MINB) k_zc
 #pragma unroll
       for (int t = 1; t < 8; ++t) v[t] = twL_mul<-1>(v[t], TW, j * t);
 #pragma unroll
-      for (int t = 0; t < 8; ++t) st_stage(X + sidx<C>(j + t * S8, c), settle(v[t]));
+      for (int t = 0; t < 8; ++t) st_stage(X + ColTile<L, C>::idx(j + t * S8, c, t), settle(v[t]));
     }
     __syncthreads();
     if (next < ntiles) zpipe_prefetch_rows<T, L, C, NT>(a, next, per_rhs, S, tid);
@@ -1900,7 +1900,7 @@ __global__ void __launch_bounds__(ZSmem<L, C, T>::NT, ZSmem<L, C, T>::MINB) k_zc
         v[t] = settle(cmul(v[t], ldgc(gp + (long long)mirror_index(k0 + (L / r3) * t, L) * a.H * a.H)));
       dft<r3, +1, false>(v);
 #pragma unroll
-      for (int t = 0; t < r3; ++t) st_stage(X + sidx<C>(blk * r3 + t, c), settle(v[t]));
+      for (int t = 0; t < r3; ++t) st_stage(X + ColTile<L, C>::idx(blk * r3 + t, c, 0), settle(v[t]));
     }
     __syncthreads();
     dit_middle<L, C>(X, TW, tid, NT);
@@ -1910,7 +1910,7 @@ __global__ void __launch_bounds__(ZSmem<L, C, T>::NT, ZSmem<L, C, T>::MINB) k_zc
       const int c = g % C, j = g / C;
       cpx<T> v[8];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) v[t] = ld_stage(X + sidx<C>(j + t * S8, c));
+      for (int t = 0; t < 8; ++t) v[t] = ld_stage(X + ColTile<L, C>::idx(j + t * S8, c, t));
 #pragma unroll
       for (int t = 1; t < 8; ++t) v[t] = twL_mul<+1>(v[t], TW, j * t);
       dft<8, +1, false>(v);

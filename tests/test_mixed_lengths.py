@@ -140,6 +140,37 @@ def test_digit_order_and_stages(L):
     assert np.array_equal((k % 8 * r2 + (qk - qk // r2 * r2)) * r3 + qk // r2, p)
 
 
+RADICES = {64: (1, 8), 128: (1, 16), 256: (8, 4), 512: (8, 8), 1024: (8, 16), 2048: (16, 16),
+           **{L: v[:2] for L, v in MIX.items()}}
+
+
+@pytest.mark.parametrize("L", RADICES)
+def test_line_tiles_of_the_shared_memory_x_passes(L):
+    """A padded line (one element per L / 8 points): every point has its place, each
+    stage addresses it by its own eighth, and the eight consecutive frequencies a
+    quarter warp takes in the last stage lie on different 16-byte banks (two to a
+    bank at L = 200)."""
+    r2, r3 = RADICES[L]
+    assert 8 * r2 * r3 == L
+    j = np.arange(L)
+    place = j + j // (L // 8)
+    assert len(np.unique(place)) == L and place.max() < L + 8
+    jj, t = grid(L // 8, 8)
+    assert np.array_equal((jj + t * (L // 8)) // (L // 8), t)            # first stage
+    if r2 > 1:
+        M = L // 8
+        s = M // r2
+        bi, t = grid(8 * s, r2)
+        assert np.array_equal((bi // s * M + bi % s + t * s) // (L // 8), bi // s)
+    blk, t = grid(L // r3, r3)
+    assert np.array_equal((blk * r3 + t) // (L // 8), blk // r2)         # last stage
+    for k0 in range(0, L // r3 - 7, 8):
+        k = np.arange(k0, k0 + 8)
+        b = (k & 7) * r2 + (k >> 3)
+        banks = (b * r3 + b // r2) % 8
+        assert len(np.unique(banks)) >= (4 if L == 200 else 8)
+
+
 @pytest.mark.parametrize("R", [3, 5, 6, 10, 12, 20])
 def test_prime_factor_map(R):
     P = R & -R
