@@ -408,7 +408,9 @@ static void host_twiddles(int L, cpx<double>* out) {
 
 static bool capturing(cudaStream_t st) {
   cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(st, &c) == cudaSuccess && c != cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &c) == cudaSuccess) return c != cudaStreamCaptureStatusNone;
+  cudaGetLastError();   // leave no error behind for the launches' checks
+  return false;
 }
 
 // Stream handoff: the plan's private stream waits for the caller's stream,
@@ -1273,6 +1275,7 @@ ori_status ori_matvec(ori_plan_t p, const double* x_dev, double* y_dev, int form
   if (p->lean && (form == ORI_FORM_A || precision == ORI_FP64))
     return fail(ORI_ERR_UNSUPPORTED, "a lean plan applies only the B form in FP32 or paired FP32");
   cudaStream_t user = reinterpret_cast<cudaStream_t>(stream);
+  ORI_TRY(ensure_capacity(p, 1));   // none is left after a batch that did not fit
   cudaStream_t run = nullptr;
   ORI_TRY(enter_direct(p, user, &run));
   XArgs pro{}, epi{};
@@ -1308,6 +1311,7 @@ ori_status ori_matvec32(ori_plan_t p, const float* x_dev, float* y_dev, int form
   if (x_dev == y_dev) return fail(ORI_ERR_INVALID_ARG, "x_dev and y_dev must not overlap");
   if (p->lean && form == ORI_FORM_A) return fail(ORI_ERR_UNSUPPORTED, "a lean plan applies only the B form");
   cudaStream_t user = reinterpret_cast<cudaStream_t>(stream);
+  ORI_TRY(ensure_capacity(p, 1));   // none is left after a batch that did not fit
   cudaStream_t run = nullptr;
   ORI_TRY(enter_direct(p, user, &run));
   XArgs pro{}, epi{};
