@@ -144,17 +144,22 @@ __device__ __forceinline__ void dif_last(const cpx<T>* X, int blk, int c, cpx<T>
 }
 
 // Threads of a tile of C columns, between most / 2 and most: the multiple of 32
-// that wastes the fewest thread-points over the three stages.
+// that wastes the fewest thread-points over the three stages.  With `ctas` > 0,
+// the few CTAs that shared memory lets on an SM, the warps they make count too:
+// W of them hide latency like W / (W + 12) (paired-FP32 Z pass at n = 200, 400
+// points: 1.69 ms with two CTAs of 160 threads and the least waste, 1.54 with
+// two of 224; at n = 400 12.2 ms with 320 threads, 11.8 with 416).
 template <int L>
-constexpr int stage_threads(int C, int most) {
+constexpr int stage_threads(int C, int most, int ctas = 0) {
   int best = most;
-  long long best_cost = 1LL << 60;
+  double best_cost = 1e30;
   for (int nt = (most / 2 + 31) / 32 * 32; nt <= most; nt += 32) {
-    long long cost = 0;
+    double cost = 0;
     for (int r : {8, SRad<L>::r2, SRad<L>::r3}) {
       const int items = C * (L / r);
-      if (r > 1) cost += (long long)((items + nt - 1) / nt) * nt * r;
+      if (r > 1) cost += double((items + nt - 1) / nt) * nt * r;
     }
+    if (ctas > 0) cost *= 1 + 12.0 / (ctas * (nt / 32));
     if (cost <= best_cost) {
       best_cost = cost;
       best = nt;

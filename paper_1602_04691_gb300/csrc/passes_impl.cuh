@@ -1834,7 +1834,8 @@ struct ZSmem {
   // per SM measured 9% slower at L = 2048), else two CTAs of half the threads,
   // whose phases overlap
   static constexpr bool TWO = SMEM_BYTES + 1024 <= 114 * 1024;
-  static constexpr int NT = is_mixed_len(L) ? stage_threads<L>(C, TWO ? 256 : 512) : (TWO ? 256 : 512);
+  static constexpr int fit = int(227 * 1024 / (SMEM_BYTES + 1024));
+  static constexpr int NT = is_mixed_len(L) ? stage_threads<L>(C, TWO ? 256 : 512, fit <= 2 ? fit : 0) : (TWO ? 256 : 512);
   static constexpr int MINB = TWO ? 2 : 1;
 };
 
