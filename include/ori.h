@@ -168,8 +168,8 @@ void ori_default_plan_opts(ori_plan_opts* o);
  *            in (L/2, L]: the same operator with less padding.  L <= 1024 runs the register-tile and persistent
  *            pipelined FFT passes; at L = 2048 the FP32 passes stay pipelined
  *            (the TILES schedules of the Y and Z passes select shared-memory
- *            radix-8 kernels) and the FP64 and paired-FP32 passes run
- *            shared-memory radix-8 kernels.
+ *            kernels) and the FP64 and paired-FP32 passes run shared-memory
+ *            kernels.
  *   k        wave number, finite and > 0 (Eq. 2.1).
  *   dom      cube corner and side (Eq. 3.3.5 uses the unit cube at the origin).
  *   h_dev    n^3 complex128 impedance samples h(x_p) (Eq. 2.13), device.

@@ -1293,8 +1293,8 @@ struct ZPipe {
 // Bulk-copy staging of the FP32 Z pass (ZPipe::TMA).  Thread 0 issues the
 // copies; every thread waits on the barrier.  The n_in input rows of a tile,
 // 128 bytes each, come as ceil(n_in / zbox) boxes of zbox rows through the
-// tensor map a.zrows (rows past n_in are zero-filled; zbox is a power of two
-// dividing L / 2 or equal to it, so the boxes end within the L / 2 + 1 rows of S).
+// tensor map a.zrows (rows past n_in are not used; zbox divides L / 2, so the
+// boxes end within the L / 2 + 1 rows of S).
 template <int L, int C>
 __device__ __forceinline__ void zpipe_tma_rows(const SArgs& a, int tile, int per_rhs, cpx<float>* S,
                                                unsigned long long* bar) {
@@ -1822,8 +1822,11 @@ cudaError_t launch_zconv_mix_L(SArgs a, cudaStream_t s, bool setup, int sm_count
 // ---------------------------------------------------------------------------
 // Z convolution for the paired-FP32 residual: persistent CTAs, a tile of C
 // columns (C * 16 B = 128 B rows) held in shared memory and transformed in
-// place by looped radix-8 stages (dfft.cuh); the next tile's input rows
-// stream into a staging buffer with cp.async meanwhile.
+// place in three stages (dfft.cuh), the last forward one, the spectrum product
+// and the first inverse one in one sweep; the next tile's input rows stream
+// into a staging buffer with cp.async meanwhile.  Bound by the paired
+// arithmetic (FMA pipe 63%, 2.5 to 4 warps a scheduler): n = 512 25.9 -> 20.2 ms
+// with the fused stages.
 // ---------------------------------------------------------------------------
 template <int L, int C, class T>
 struct ZSmem {
