@@ -694,7 +694,7 @@ static int vgrid_sum(const ori_plan_s* p, int nrhs) {
 // mapped address of a pinned mirror).
 static ori_status small_copy(ori_plan_s* p, void* dst, const void* src, size_t bytes, int rows = 1,
                              size_t dpitch = 0, size_t spitch = 0) {
-  k_small_copy<<<1, 256, 0, p->ps>>>(static_cast<const unsigned char*>(src), static_cast<unsigned char*>(dst),
+  launch_dep(k_small_copy, dim3(1), 256, 0, p->ps, static_cast<const unsigned char*>(src), static_cast<unsigned char*>(dst),
                                      (long long)bytes, (long long)(spitch ? spitch : bytes),
                                      (long long)(dpitch ? dpitch : bytes), rows);
   ORI_CUDA(cudaGetLastError());
@@ -1365,7 +1365,7 @@ struct InnerResult {
 // Copy the scalar heads of all right-hand sides and the fault flag to their
 // pinned mirrors (one launch) and wait for them.
 static ori_status read_heads(ori_plan_s* p, int nrhs) {
-  k_read_heads<<<1, 256, 0, p->ps>>>(p->sc, nrhs, static_cast<unsigned long long*>(p->h_sc_d), p->d_fault,
+  launch_dep(k_read_heads, dim3(1), 256, 0, p->ps, p->sc, nrhs, static_cast<unsigned long long*>(p->h_sc_d), p->d_fault,
                                      static_cast<int*>(p->h_fault_d));
   ORI_CUDA(cudaGetLastError());
   launched(p);
@@ -1398,7 +1398,7 @@ static ori_status cocg_inner(ori_plan_s* p, int nrhs, int rhs_per_k, cpx<T>* x, 
   ORI_TRY(small_copy(p, p->d_tols, p->h_small_d, nrhs * sizeof(double)));   // h_tols is h_small
   const int vg = vgrid_sum(p, nrhs);
   ORI_VEC(p, ORI_PASS_VECTOR + (sizeof(T) == 4 ? 0 : ORI_PASS_FP64),
-          (k_cocg_init<T><<<dim3(vg, nrhs), 256, 0, p->ps>>>(r, x, p->n3, p->sc, p->partials, p->d_tols, maxit,
+          (launch_dep(k_cocg_init<T>, dim3(vg, nrhs), 256, 0, p->ps, r, x, p->n3, p->sc, p->partials, p->d_tols, maxit,
                                                                zero_x ? 1 : 0)));
   auto any_running = [&]() {
     for (int i = 0; i < nrhs; ++i)
@@ -1663,7 +1663,7 @@ static ori_status solve_B(ori_plan_s* p, int nrhs, int rhs_per_k, const double* 
     if (budget <= 0) break;
     ORI_TRY(push_doubles(p, p->d_scl, inv.data(), nrhs, SLOT_INV));
     const int vg = vgrid(p, nrhs);
-    ORI_VEC(p, ORI_PASS_VECTOR, (k_normalise_to_f32<<<dim3(vg, nrhs), 256, 0, p->ps>>>(w_set ? p->r64 : p->b64, p->r32, n3,
+    ORI_VEC(p, ORI_PASS_VECTOR, (launch_dep(k_normalise_to_f32, dim3(vg, nrhs), 256, 0, p->ps, w_set ? p->r64 : p->b64, p->r32, n3,
                                                                                        p->d_scl)));
     ORI_TRY(cocg_inner<float>(p, nrhs, rhs_per_k, p->x32, p->r32, p->p32, p->q32, p->S32, tin.data(), budget,
                               o.check_every, graph, ir.data()));
@@ -1682,7 +1682,7 @@ static ori_status solve_B(ori_plan_s* p, int nrhs, int rhs_per_k, const double* 
     }
     if (nonfinite_all) break;
     ORI_TRY(push_doubles(p, p->d_scl, scl.data(), nrhs, SLOT_ACC));
-    ORI_VEC(p, ORI_PASS_VECTOR, (k_accumulate<<<dim3(vg, nrhs), 256, 0, p->ps>>>(p->w, p->x32, n3, p->d_scl, w_set ? 0 : 1)));
+    ORI_VEC(p, ORI_PASS_VECTOR, (launch_dep(k_accumulate, dim3(vg, nrhs), 256, 0, p->ps, p->w, p->x32, n3, p->d_scl, w_set ? 0 : 1)));
     // residual: updated with the FP32 operator when every active RHS allows it
     bool upd = o.resid_update != 0;
     std::vector<double> upd_err(nrhs, 0.0);
@@ -1796,11 +1796,11 @@ static ori_status solve_batch(ori_plan_s* p, int nk, int ndir, const double* rhs
   ORI_TRY(push_doubles(p, p->d_dir, dv.data(), 3 * nrhs, SLOT_DIR));
   const int vg = vgrid(p, nrhs);
   ORI_VEC(p, ORI_PASS_VECTOR,
-          (k_phases<<<dim3(unsigned((3 * p->n + 255) / 256), nrhs), 256, 0, p->ps>>>(
+          (launch_dep(k_phases, dim3(unsigned((3 * p->n + 255) / 256), nrhs), 256, 0, p->ps, 
               p->d_kv, p->d_dir, p->n, p->d, p->origin[0], p->origin[1], p->origin[2], p->d_phase)));
   // u0 is kept only where S = 0 cells need it for the recovery
   ORI_VEC(p, ORI_PASS_VECTOR,
-          (k_rhs<<<dim3(vgrid_sum(p, nrhs), nrhs), 256, rhs_dev ? 0 : 3 * size_t(p->n) * sizeof(cpx<double>), p->ps>>>(
+          (launch_dep(k_rhs, dim3(vgrid_sum(p, nrhs), nrhs), 256, rhs_dev ? 0 : 3 * size_t(p->n) * sizeof(cpx<double>), p->ps, 
               reinterpret_cast<const cpx<double>*>(rhs_dev), p->S64, p->zero_S ? p->u0 : nullptr, p->b64, p->n,
               p->d_phase, p->sc, p->partials)));
   ORI_TRY(read_heads(p, nrhs));
@@ -1813,7 +1813,7 @@ static ori_status solve_batch(ori_plan_s* p, int nk, int ndir, const double* rhs
   // u = w / S; cells with S = 0 take u = u0 - K (S w) (one more FP64 application)
   if (p->zero_S == 0) {
     ORI_VEC(p, ORI_PASS_VECTOR,
-            (k_recover<<<dim3(vg, nrhs), 256, 0, p->ps>>>(p->w, p->Sinv, p->S64, reinterpret_cast<cpx<double>*>(u_dev),
+            (launch_dep(k_recover, dim3(vg, nrhs), 256, 0, p->ps, p->w, p->Sinv, p->S64, reinterpret_cast<cpx<double>*>(u_dev),
                                                            p->n3)));
   } else {
     const long long bsv = p->n3 * (long long)sizeof(cpx<double>);

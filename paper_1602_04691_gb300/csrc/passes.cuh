@@ -218,7 +218,8 @@ constexpr int even_box(int rows) {
 // than the overlap gives (n = 400: FP32 operator 4.14 ms with an early trigger,
 // 3.92 without, 3.93 with plain launches; n = 128: 0.112, 0.103 and 0.118 ms).
 // FP32 operator (five passes) at n = 100: 79.9 -> 66.7 us; FP64 operator at
-// n = 12: 44.0 -> 34.4 us; mixed solve at n = 20: 0.83 -> 0.72 ms.
+// n = 12: 44.0 -> 34.4 us; mixed solve at n = 20: 0.83 -> 0.72 ms, and with the
+// solver's vector and control kernels launched the same way 0.68 -> 0.65 ms.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... P, class... A>

@@ -88,6 +88,7 @@ __global__ void k_medium(const cpx<double>* __restrict__ h, const double* __rest
 // 8-byte words when every address, size and pitch allows.
 __global__ void k_small_copy(const unsigned char* src, unsigned char* dst, long long bytes, long long spitch,
                              long long dpitch, int rows) {
+  dep_wait();
   const bool words = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) |
                        uintptr_t(bytes) | uintptr_t(spitch) | uintptr_t(dpitch)) & 7u) == 0;
   for (int r = 0; r < rows; ++r) {
@@ -107,6 +108,7 @@ __global__ void k_small_copy(const unsigned char* src, unsigned char* dst, long 
 // fault flag, to their mapped mirrors: what the host reads between launches,
 // in one launch.  The mirror of the heads keeps the stride of Scalars.
 __global__ void k_read_heads(const Scalars* sc, int nrhs, unsigned long long* out, const int* fault, int* out_fault) {
+  dep_wait();
   constexpr int W = int(offsetof(Scalars, hist) / 8), STRIDE = int(sizeof(Scalars) / 8);
   static_assert(offsetof(Scalars, hist) % 8 == 0 && sizeof(Scalars) % 8 == 0, "whole words");
   const unsigned long long* in = reinterpret_cast<const unsigned long long*>(sc);
@@ -201,6 +203,7 @@ __device__ __forceinline__ void block_partial2(double2 a, double2 b, double2* re
 // out[rb][axis * n + i] = exp(i k_rb a_rb,axis (o_axis + (i + 1/2) d)).
 __global__ void k_phases(const double* __restrict__ kvals, const double* __restrict__ dirs, int n, double d,
                          double ox, double oy, double oz, cpx<double>* out) {
+  dep_wait();
   const int rb = blockIdx.y;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 3 * n) return;
@@ -214,6 +217,7 @@ __global__ void k_phases(const double* __restrict__ kvals, const double* __restr
 __global__ void k_rhs(const cpx<double>* __restrict__ rhs, const cpx<double>* __restrict__ S,
                       cpx<double>* u0, cpx<double>* b, int n, const cpx<double>* __restrict__ phases,
                       Scalars* sc0, double2* partials0) {
+  dep_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
   cpx<double>* e = reinterpret_cast<cpx<double>*>(smraw);   // [3][n]
   __shared__ double2 red[64];
@@ -274,6 +278,7 @@ __global__ void k_adj_rhs(const cpx<double>* __restrict__ ec, const cpx<double>*
 template <class T>
 __global__ void k_cocg_init(const cpx<T>* __restrict__ r, cpx<T>* x, long long n3, Scalars* sc0,
                             double2* partials0, const double* __restrict__ tols, int maxit, int zero_x) {
+  dep_wait();
   __shared__ double2 red[64];
   __shared__ int s_last;
   const int rb = blockIdx.y;
@@ -438,6 +443,7 @@ __global__ void k_cocg_update<float>(cpx<float>* __restrict__ x, const cpx<float
 // Mixed refinement: r32 = r64 / ||r64||.
 __global__ void k_normalise_to_f32(const cpx<double>* __restrict__ r64, cpx<float>* r32,
                                    long long n3, const double* __restrict__ invs) {
+  dep_wait();
   const int rb = blockIdx.y;
   const double inv = invs[rb];
   r64 += rb * n3;
@@ -453,6 +459,7 @@ __global__ void k_normalise_to_f32(const cpx<double>* __restrict__ r64, cpx<floa
 // step from w = 0).
 __global__ void k_accumulate(cpx<double>* w, const cpx<float>* __restrict__ d32, long long n3,
                              const double* __restrict__ scales, int set) {
+  dep_wait();
   const int rb = blockIdx.y;
   const double scale = scales[rb];
   if (scale == 0.0 && !set) return;
@@ -474,6 +481,7 @@ __global__ void k_accumulate(cpx<double>* w, const cpx<float>* __restrict__ d32,
 // u = w / S = w * (1/S) (every S != 0; 1/S is kept by the plan).
 __global__ void k_recover(const cpx<double>* __restrict__ w, const cpx<double>* __restrict__ Sinv,
                           const cpx<double>* __restrict__ S, cpx<double>* u, long long n3) {
+  dep_wait();
   w += blockIdx.y * n3;
   u += blockIdx.y * n3;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n3;
