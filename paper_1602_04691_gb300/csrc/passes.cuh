@@ -213,7 +213,14 @@ constexpr int even_box(int rows) {
 // waits in dep_wait until the previous kernel has completed and its writes
 // are visible.  Every kernel launched this way calls dep_wait before it
 // touches anything another kernel writes or reads (all but the plan's
-// twiddle tables), in every thread.  The successor's launch is not triggered
+// twiddle tables), in every thread.  Such a kernel is alive while its
+// predecessor still writes, so it reads what a predecessor writes by coherent
+// loads only: no __ldg, and no `const __restrict__` parameter, which lets the
+// compiler take non-coherent loads, for which nothing may write the data while
+// the kernel lives and which dep_wait need not hold back.  __restrict__ stays
+// on the arrays of the medium and the caller's right-hand side, complete
+// before the chain of launches starts, and on a kernel's own outputs.
+// The successor's launch is not triggered
 // early: CTAs waiting on an SM from the start of their predecessor cost more
 // than the overlap gives (n = 400: FP32 operator 4.14 ms with an early trigger,
 // 3.92 without, 3.93 with plain launches; n = 128: 0.112, 0.103 and 0.118 ms).

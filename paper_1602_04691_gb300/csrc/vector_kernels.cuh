@@ -201,8 +201,8 @@ __device__ __forceinline__ void block_partial2(double2 a, double2 b, double2* re
 // every cell costs two complex products.
 // Phase factors of the separable plane wave, once per right-hand side:
 // out[rb][axis * n + i] = exp(i k_rb a_rb,axis (o_axis + (i + 1/2) d)).
-__global__ void k_phases(const double* __restrict__ kvals, const double* __restrict__ dirs, int n, double d,
-                         double ox, double oy, double oz, cpx<double>* out) {
+__global__ void k_phases(const double* kvals, const double* dirs, int n, double d, double ox, double oy, double oz,
+                         cpx<double>* out) {
   dep_wait();
   const int rb = blockIdx.y;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -215,7 +215,7 @@ __global__ void k_phases(const double* __restrict__ kvals, const double* __restr
 }
 
 __global__ void k_rhs(const cpx<double>* __restrict__ rhs, const cpx<double>* __restrict__ S,
-                      cpx<double>* u0, cpx<double>* b, int n, const cpx<double>* __restrict__ phases,
+                      cpx<double>* __restrict__ u0, cpx<double>* __restrict__ b, int n, const cpx<double>* phases,
                       Scalars* sc0, double2* partials0) {
   dep_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -276,8 +276,8 @@ __global__ void k_adj_rhs(const cpx<double>* __restrict__ ec, const cpx<double>*
 // COCG start: x = 0, rho = r^T r, ||r||^2; sets tol/maxit and the flags.
 // Sums in T over 8 elements per thread, then in FP64.
 template <class T>
-__global__ void k_cocg_init(const cpx<T>* __restrict__ r, cpx<T>* x, long long n3, Scalars* sc0,
-                            double2* partials0, const double* __restrict__ tols, int maxit, int zero_x) {
+__global__ void k_cocg_init(const cpx<T>* r, cpx<T>* __restrict__ x, long long n3, Scalars* sc0,
+                            double2* partials0, const double* tols, int maxit, int zero_x) {
   dep_wait();
   __shared__ double2 red[64];
   __shared__ int s_last;
@@ -332,9 +332,8 @@ struct KahanF {
 // COCG update: x += alpha p, r -= alpha q; rho' = r^T r and ||r||^2 of the new
 // residual.  FP64 vectors: sums over 8 elements per thread in FP64.
 template <class T>
-__global__ void k_cocg_update(cpx<T>* __restrict__ x, const cpx<T>* __restrict__ p,
-                              cpx<T>* __restrict__ r, const cpx<T>* __restrict__ q, long long n3,
-                              Scalars* sc0, double2* partials0) {
+__global__ void k_cocg_update(cpx<T>* __restrict__ x, const cpx<T>* p, cpx<T>* __restrict__ r, const cpx<T>* q,
+                              long long n3, Scalars* sc0, double2* partials0) {
   dep_wait();
   __shared__ double2 red[64];
   __shared__ int s_last;
@@ -378,8 +377,8 @@ __global__ void k_cocg_update(cpx<T>* __restrict__ x, const cpx<T>* __restrict__
 // unrolled group issued before any arithmetic, Kahan-compensated FP32 sums
 // widened to FP64 once per thread.
 template <>
-__global__ void k_cocg_update<float>(cpx<float>* __restrict__ x, const cpx<float>* __restrict__ p,
-                                     cpx<float>* __restrict__ r, const cpx<float>* __restrict__ q,
+__global__ void k_cocg_update<float>(cpx<float>* __restrict__ x, const cpx<float>* p,
+                                     cpx<float>* __restrict__ r, const cpx<float>* q,
                                      long long n3, Scalars* sc0, double2* partials0) {
   dep_wait();
   __shared__ double2 red[64];
@@ -441,8 +440,8 @@ __global__ void k_cocg_update<float>(cpx<float>* __restrict__ x, const cpx<float
 }
 
 // Mixed refinement: r32 = r64 / ||r64||.
-__global__ void k_normalise_to_f32(const cpx<double>* __restrict__ r64, cpx<float>* r32,
-                                   long long n3, const double* __restrict__ invs) {
+__global__ void k_normalise_to_f32(const cpx<double>* r64, cpx<float>* __restrict__ r32, long long n3,
+                                   const double* invs) {
   dep_wait();
   const int rb = blockIdx.y;
   const double inv = invs[rb];
@@ -457,8 +456,8 @@ __global__ void k_normalise_to_f32(const cpx<double>* __restrict__ r64, cpx<floa
 
 // Mixed refinement: w += scale * d32, or w = scale * d32 when `set` (the first
 // step from w = 0).
-__global__ void k_accumulate(cpx<double>* w, const cpx<float>* __restrict__ d32, long long n3,
-                             const double* __restrict__ scales, int set) {
+__global__ void k_accumulate(cpx<double>* __restrict__ w, const cpx<float>* d32, long long n3, const double* scales,
+                             int set) {
   dep_wait();
   const int rb = blockIdx.y;
   const double scale = scales[rb];
@@ -479,8 +478,8 @@ __global__ void k_accumulate(cpx<double>* w, const cpx<float>* __restrict__ d32,
 }
 
 // u = w / S = w * (1/S) (every S != 0; 1/S is kept by the plan).
-__global__ void k_recover(const cpx<double>* __restrict__ w, const cpx<double>* __restrict__ Sinv,
-                          const cpx<double>* __restrict__ S, cpx<double>* u, long long n3) {
+__global__ void k_recover(const cpx<double>* w, const cpx<double>* __restrict__ Sinv,
+                          const cpx<double>* __restrict__ S, cpx<double>* __restrict__ u, long long n3) {
   dep_wait();
   w += blockIdx.y * n3;
   u += blockIdx.y * n3;
