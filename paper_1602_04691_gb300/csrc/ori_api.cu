@@ -413,39 +413,52 @@ static bool capturing(cudaStream_t st) {
   return false;
 }
 
-// Stream handoff: the plan's private stream waits for the caller's stream,
-// and for the plan's last work on another caller's stream (evl; not under
-// capture, where only the captured work is ordered).
-static ori_status enter(ori_plan_s* p, cudaStream_t user) {
-  ORI_CUDA(cudaEventRecord(p->evj, user));
-  ORI_CUDA(cudaStreamWaitEvent(p->ps, p->evj, 0));
-  if (!capturing(user)) ORI_CUDA(cudaStreamWaitEvent(p->ps, p->evl, 0));
-  return ORI_OK;
-}
-static ori_status leave(ori_plan_s* p, cudaStream_t user) {
-  const cudaEvent_t e = capturing(user) ? p->evj : p->evl;
-  ORI_CUDA(cudaEventRecord(e, p->ps));
-  ORI_CUDA(cudaStreamWaitEvent(user, e, 0));
-  return ORI_OK;
-}
+// Stream handoff of one call.  enter: the plan's private stream waits for the
+// caller's stream, and for the plan's last work on another caller's stream (evl;
+// not under capture, where only the captured work is ordered).  The operator
+// calls launch on the caller's own stream instead (enter with `direct`): no hop
+// to the private stream and back (two event waits a call; FP64 operator at
+// n = 12: 48.6 -> 44.0 us); under capture they go through the private stream as
+// the other calls do.  `run` is the stream to launch on.  Every way out of an
+// entered call, an error return too, marks the end of its work (leave, or the
+// destructor): what the call had in flight still uses the plan's scratch, and
+// the next call may run on another stream.
+struct Handoff {
+  ori_plan_s* p = nullptr;
+  cudaStream_t user = nullptr, run = nullptr;
 
-// The operator calls launch on the caller's own stream: no hop to the private
-// stream and back (two event waits a call; FP64 operator at n = 12: 48.6 -> 44.0 us).  *run is the stream to launch on.  Under capture they go
-// through the private stream as the other calls do.
-static ori_status enter_direct(ori_plan_s* p, cudaStream_t user, cudaStream_t* run) {
-  if (capturing(user)) {
-    *run = p->ps;
-    return enter(p, user);
+  Handoff() = default;
+  Handoff(const Handoff&) = delete;
+  Handoff& operator=(const Handoff&) = delete;
+  ~Handoff() {
+    if (p != nullptr && close() != cudaSuccess) cudaGetLastError();   // the call's own error is the one reported
   }
-  *run = user;
-  ORI_CUDA(cudaStreamWaitEvent(user, p->evl, 0));
-  return ORI_OK;
-}
-static ori_status leave_direct(ori_plan_s* p, cudaStream_t user, cudaStream_t run) {
-  if (run == p->ps) return leave(p, user);
-  ORI_CUDA(cudaEventRecord(p->evl, user));
-  return ORI_OK;
-}
+  ori_status enter(ori_plan_s* plan, cudaStream_t stream, bool direct = false) {
+    const bool cap = capturing(stream);
+    user = stream;
+    run = direct && !cap ? stream : plan->ps;
+    if (run != user) {
+      ORI_CUDA(cudaEventRecord(plan->evj, user));
+      ORI_CUDA(cudaStreamWaitEvent(run, plan->evj, 0));
+    }
+    p = plan;
+    if (!cap) ORI_CUDA(cudaStreamWaitEvent(run, p->evl, 0));
+    return ORI_OK;
+  }
+  ori_status leave() {
+    ORI_CUDA(close());
+    return ORI_OK;
+  }
+
+ private:
+  cudaError_t close() {
+    const cudaEvent_t done = capturing(user) ? p->evj : p->evl;
+    cudaError_t e = cudaEventRecord(done, run);
+    if (e == cudaSuccess && run != user) e = cudaStreamWaitEvent(user, done, 0);
+    p = nullptr;
+    return e;
+  }
+};
 
 // Wait for all of the plan's work.
 static cudaError_t sync_plan(ori_plan_s* p) {
@@ -1096,7 +1109,8 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
         (st = setup_kernels<dfl>(p->M, &bxdf, p->n, p->sm_count)))
       break;
     p->xinv_blocks = std::max({bx32, bx64, bxdf});
-    if ((st = enter(p, user))) break;
+    Handoff io;
+    if ((st = io.enter(p, user))) break;
     {
       cpx<double>* twd = new cpx<double>[p->M];
       cpx<float>* twf = new cpx<float>[p->M];
@@ -1122,7 +1136,7 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
     if ((st = set_medium(p, h_dev, N_dev))) break;
     if ((st = ensure_capacity(p, 1))) break;   // before the spectrum build, which uses its cubes
     if ((st = spec ? load_spectrum(p, static_cast<const unsigned char*>(spec)) : build_spectrum(p))) break;
-    if ((st = leave(p, user))) break;
+    if ((st = io.leave())) break;
   } while (0);
   if (st != ORI_OK) {
     plan_free(p);
@@ -1160,7 +1174,8 @@ ori_status ori_plan_save_spectrum(ori_plan_t p, void* host_buf, size_t bytes, vo
   g_last_error.clear();
   if (!p || !host_buf) return fail(ORI_ERR_INVALID_ARG, "NULL argument");
   if (bytes < spectrum_bytes(p)) return fail(ORI_ERR_INVALID_ARG, "host_buf is shorter than ori_plan_spectrum_bytes");
-  ORI_TRY(enter(p, reinterpret_cast<cudaStream_t>(stream)));
+  Handoff io;
+  ORI_TRY(io.enter(p, reinterpret_cast<cudaStream_t>(stream)));
   SpecHeader hd{};
   std::memcpy(hd.tag, kSpecTag, sizeof(kSpecTag));
   hd.version = 1;
@@ -1191,7 +1206,7 @@ ori_status ori_plan_save_spectrum(ori_plan_t p, void* host_buf, size_t bytes, vo
       std::memcpy(dst + i, &v, sizeof(v));
     }
   }
-  ORI_TRY(leave(p, reinterpret_cast<cudaStream_t>(stream)));
+  ORI_TRY(io.leave());
   return ORI_OK;
 }
 
@@ -1210,9 +1225,10 @@ ori_status ori_plan_set_medium(ori_plan_t p, const double* h_dev, const double* 
   g_last_error.clear();
   if (!p || !h_dev || !N_dev) return fail(ORI_ERR_INVALID_ARG, "NULL argument");
   cudaStream_t user = reinterpret_cast<cudaStream_t>(stream);
-  ORI_TRY(enter(p, user));
+  Handoff io;
+  ORI_TRY(io.enter(p, user));
   ORI_TRY(set_medium(p, h_dev, N_dev));
-  return leave(p, user);
+  return io.leave();
 }
 
 ori_status ori_plan_set_timing(ori_plan_t p, int on) {
@@ -1275,8 +1291,9 @@ ori_status ori_matvec(ori_plan_t p, const double* x_dev, double* y_dev, int form
     return fail(ORI_ERR_UNSUPPORTED, "a lean plan applies only the B form in FP32 or paired FP32");
   cudaStream_t user = reinterpret_cast<cudaStream_t>(stream);
   ORI_TRY(ensure_capacity(p, 1));   // none is left after a batch that did not fit
-  cudaStream_t run = nullptr;
-  ORI_TRY(enter_direct(p, user, &run));
+  Handoff io;
+  ORI_TRY(io.enter(p, user, true));
+  const cudaStream_t run = io.run;
   XArgs pro{}, epi{};
   pro.x = x_dev;
   epi.xin = x_dev;
@@ -1300,7 +1317,7 @@ ori_status ori_matvec(ori_plan_t p, const double* x_dev, double* y_dev, int form
     epi.scale = p->Sdf;
     ORI_TRY(run_conv<dfl>(p, pro, epi, FIN_NONE, run, Mask{}));
   }
-  return leave_direct(p, user, run);
+  return io.leave();
 }
 
 ori_status ori_matvec32(ori_plan_t p, const float* x_dev, float* y_dev, int form, void* stream) {
@@ -1311,8 +1328,9 @@ ori_status ori_matvec32(ori_plan_t p, const float* x_dev, float* y_dev, int form
   if (p->lean && form == ORI_FORM_A) return fail(ORI_ERR_UNSUPPORTED, "a lean plan applies only the B form");
   cudaStream_t user = reinterpret_cast<cudaStream_t>(stream);
   ORI_TRY(ensure_capacity(p, 1));   // none is left after a batch that did not fit
-  cudaStream_t run = nullptr;
-  ORI_TRY(enter_direct(p, user, &run));
+  Handoff io;
+  ORI_TRY(io.enter(p, user, true));
+  const cudaStream_t run = io.run;
   XArgs pro{}, epi{};
   pro.x = x_dev;
   pro.mode = PRO_SCALE;
@@ -1322,7 +1340,7 @@ ori_status ori_matvec32(ori_plan_t p, const float* x_dev, float* y_dev, int form
   epi.mode = form == ORI_FORM_A ? EPI_PLUS : EPI_PLUS_S;
   epi.scale = p->S32;
   ORI_TRY(run_conv<float>(p, pro, epi, FIN_NONE, run, Mask{}));
-  return leave_direct(p, user, run);
+  return io.leave();
 }
 
 }  // extern "C"
@@ -1781,7 +1799,8 @@ static ori_status solve_batch(ori_plan_s* p, int nk, int ndir, const double* rhs
     return fail(ORI_ERR_UNSUPPORTED, "a lean plan solves in mixed precision with the paired-FP32 residual only");
   ORI_TRY(ensure_capacity(p, nrhs));
   if (o.history) p->history.assign(size_t(nrhs), std::vector<double>());
-  ORI_TRY(enter(p, user));
+  Handoff io;
+  ORI_TRY(io.enter(p, user));
   ORI_CUDA(cudaEventRecord(p->ev0, p->ps));
   std::vector<double> kv(nrhs), dv(3 * nrhs);
   for (int ik = 0; ik < nk; ++ik)
@@ -1839,7 +1858,7 @@ static ori_status solve_batch(ori_plan_s* p, int nk, int ndir, const double* rhs
   cudaEventElapsedTime(&ms, p->ev0, p->ev1);
   if (p->timing) t_harvest(p);
   for (int i = 0; i < nrhs; ++i) infos[i].ms = ms;
-  ORI_TRY(leave(p, user));
+  ORI_TRY(io.leave());
   return ORI_OK;
 }
 
@@ -1901,7 +1920,8 @@ ori_status ori_adjoint_solve(ori_plan_t p, const double* u_dev, const double* ec
   cudaStream_t user = reinterpret_cast<cudaStream_t>(stream);
   ORI_TRY(ensure_capacity(p, 1));
   if (o.history) p->history.assign(1, std::vector<double>());
-  ORI_TRY(enter(p, user));
+  Handoff io;
+  ORI_TRY(io.enter(p, user));
   ORI_CUDA(cudaEventRecord(p->ev0, p->ps));
   ORI_VEC(p, ORI_PASS_VECTOR,
           (k_adj_rhs<<<vgrid_sum(p, 1), 256, 0, p->ps>>>(reinterpret_cast<const cpx<double>*>(econj_dev), p->S64, p->b64,
@@ -1918,7 +1938,7 @@ ori_status ori_adjoint_solve(ori_plan_t p, const double* u_dev, const double* ec
   ORI_CUDA(cudaEventSynchronize(p->ev1));
   cudaEventElapsedTime(&info.ms, p->ev0, p->ev1);
   if (p->timing) t_harvest(p);
-  ORI_TRY(leave(p, user));
+  ORI_TRY(io.leave());
   if (info_out) *info_out = info;
   if (info.status != ORI_OK)
     return fail(ori_status(info.status), std::string("adjoint solve ended with status ") + ori_status_string(info.status));
@@ -2106,7 +2126,8 @@ ori_status ori_plan_autotune(ori_plan_t p, int nrhs, int reps, ori_schedule* bes
   if (nrhs < 1 || nrhs > 4096) return fail(ORI_ERR_INVALID_ARG, "nrhs must be in [1, 4096]");
   if (reps < 1 || reps > 100) return fail(ORI_ERR_INVALID_ARG, "reps must be in [1, 100]");
   cudaStream_t user = reinterpret_cast<cudaStream_t>(stream);
-  ORI_TRY(enter(p, user));
+  Handoff io;
+  ORI_TRY(io.enter(p, user));
   ORI_CUDA(cudaStreamSynchronize(p->ps));
   if (p->timing) t_harvest(p);
   const bool timing = p->timing;
@@ -2116,7 +2137,7 @@ ori_status ori_plan_autotune(ori_plan_t p, int nrhs, int reps, ori_schedule* bes
   p->timing = timing;
   p->stats = saved;
   if (st != ORI_OK) return st;
-  return leave(p, user);
+  return io.leave();
 }
 
 }  // extern "C"
@@ -2142,7 +2163,8 @@ extern "C" ori_status ori_field(ori_plan_t p, const double* u_dev, int64_t npts,
   }
   cudaStream_t user = reinterpret_cast<cudaStream_t>(stream);
   ORI_TRY(ensure_capacity(p, 1));
-  ORI_TRY(enter(p, user));
+  Handoff io;
+  ORI_TRY(io.enter(p, user));
   const double coef = -p->c_S * p->d * p->d * p->d;
   ORI_VEC(p, ORI_PASS_VECTOR,
           (k_charges<<<p->vec_grid, 256, 0, p->ps>>>(reinterpret_cast<const cpx<double>*>(u_dev), p->h, p->N, coef,
@@ -2170,5 +2192,5 @@ extern "C" ori_status ori_field(ori_plan_t p, const double* u_dev, int64_t npts,
                 partials, S, pts, np, p->ks[0], a[0], a[1], a[2], alpha_host ? 1 : 0,
                 reinterpret_cast<cpx<double>*>(out_dev) + c0)));
   }
-  return leave(p, user);
+  return io.leave();
 }
