@@ -375,7 +375,9 @@ __global__ void k_cocg_update(cpx<T>* __restrict__ x, const cpx<T>* p, cpx<T>* _
 
 // FP32 vectors: two complex numbers per 16-byte access, all loads of an
 // unrolled group issued before any arithmetic, Kahan-compensated FP32 sums
-// widened to FP64 once per thread.
+// widened to FP64 once per thread.  With an odd number of cells every second
+// system of a batch starts 8 bytes off a 16-byte boundary: its first element
+// goes on its own then, and the last one in the other systems.
 template <>
 __global__ void k_cocg_update<float>(cpx<float>* __restrict__ x, const cpx<float>* p,
                                      cpx<float>* __restrict__ r, const cpx<float>* q,
@@ -391,11 +393,12 @@ __global__ void k_cocg_update<float>(cpx<float>* __restrict__ x, const cpx<float
   const double2 ad = sc->alpha;
   const float ar = float(ad.x), ai = float(ad.y);
   KahanF kr, ki, kn;
-  const long long nv = n3 / 2;                        // float4 = two complex numbers
-  float4* x4 = reinterpret_cast<float4*>(x);
-  float4* r4 = reinterpret_cast<float4*>(r);
-  const float4* p4 = reinterpret_cast<const float4*>(p);
-  const float4* q4 = reinterpret_cast<const float4*>(q);
+  const int head = int((rb * n3) & 1);                // the arrays themselves start on 256 bytes
+  const long long nv = (n3 - head) / 2;               // float4 = two complex numbers
+  float4* x4 = reinterpret_cast<float4*>(x + head);
+  float4* r4 = reinterpret_cast<float4*>(r + head);
+  const float4* p4 = reinterpret_cast<const float4*>(p + head);
+  const float4* q4 = reinterpret_cast<const float4*>(q + head);
   const long long stride = (long long)gridDim.x * blockDim.x;
   constexpr int U = 4;
   for (long long base = blockIdx.x * (long long)blockDim.x + threadIdx.x; base < nv; base += U * stride) {
@@ -422,8 +425,8 @@ __global__ void k_cocg_update<float>(cpx<float>* __restrict__ x, const cpx<float
       }
     }
   }
-  if ((n3 & 1) && blockIdx.x == 0 && threadIdx.x == 0) {   // odd length: the last element
-    const long long i = n3 - 1;
+  if ((n3 & 1) && blockIdx.x == 0 && threadIdx.x == 0) {   // odd length: the element without a partner
+    const long long i = head ? 0 : n3 - 1;
     cpx<float> X = x[i], R = r[i];
     const cpx<float> P = p[i], Q = q[i];
     X.x += ar * P.x - ai * P.y;  X.y += ar * P.y + ai * P.x;
