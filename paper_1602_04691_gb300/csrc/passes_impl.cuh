@@ -570,15 +570,16 @@ __global__ void __launch_bounds__(XInvPipe<L, C>::NT, L > 1024 ? 1 : 3) k_xinv_p
   const cpx<T>* tw = reinterpret_cast<const cpx<T>*>(a.twL);
   const int tid = threadIdx.x;
   const int ntiles = int((a.nlines + C - 1) / C);
-  const bool staged = xinv_stage_epi(a.mode) && (a.n % 2 == 0);
+  // staged in 16-byte pieces (a caller's complex64 vector may start on 8 bytes)
+  const bool staged = xinv_stage_epi(a.mode) && (a.n % 2 == 0) &&
+                      ((reinterpret_cast<uintptr_t>(a.xin) | reinterpret_cast<uintptr_t>(a.scale)) & 15u) == 0;
   // Bulk copies (TMA, one thread issues them): a tile's C lines of T1 are one
   // contiguous block and its epilogue inputs two more (n even keeps every
   // offset and size a multiple of 16 bytes; the shared-memory regions start
   // on 16-byte boundaries when their element counts are even).
   constexpr bool kBulkFits = XP::BUF % 2 == 0 && (XP::EPI / 2) % 2 == 0;
   const bool bulk = kBulkFits && staged &&
-                    ((reinterpret_cast<uintptr_t>(a.in) | reinterpret_cast<uintptr_t>(a.xin) |
-                      reinterpret_cast<uintptr_t>(a.scale)) & 15u) == 0;
+                    (reinterpret_cast<uintptr_t>(a.in) & 15u) == 0;
   unsigned ph_t = 0, ph_e = 0;      // barrier phases awaited next
   bool pend_t = false, pend_e = false, failed = false;
   if (bulk) {
@@ -1112,10 +1113,13 @@ cudaError_t launch_xfwd_pipe_L(const XArgs& a, cudaStream_t s, bool setup) {
 }
 
 // The pipelined kernel serves the solver's prologues on whole contiguous lines
-// of even length; the plan's kernel cube and the mixed-arithmetic prologue
-// take the one-tile-per-CTA kernel.
+// of even length whose arrays start on 16 bytes (a caller's complex64 vector
+// may start on 8); the plan's kernel cube, the mixed-arithmetic prologue and
+// the rest take the one-tile-per-CTA kernel.
 inline bool xfwd_pipe_ok(const XArgs& a, int L) {
-  return (a.mode == PRO_SCALE || a.mode == PRO_COCG_FIRST || a.mode == PRO_COCG) && a.n % 2 == 0 &&
+  const uintptr_t at = reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.scale) |
+                       (a.mode == PRO_COCG ? reinterpret_cast<uintptr_t>(a.p) : 0);
+  return (a.mode == PRO_SCALE || a.mode == PRO_COCG_FIRST || a.mode == PRO_COCG) && a.n % 2 == 0 && (at & 15u) == 0 &&
          a.n_in == a.n && a.line_len_in == a.n && a.line_len_out == L && 2 * a.n <= L;
 }
 
