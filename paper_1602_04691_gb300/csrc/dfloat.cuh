@@ -14,8 +14,9 @@
 // Products accumulate all four partial products.  Neither renormalises its
 // result: the pair hi + lo stays an exact-enough representation (|lo| grows
 // by about one unit of 2^-24 |hi| per level of additions), so the FFT stages
-// add and multiply unnormalised pairs and renormalise each value once, when
-// they store it (settle), instead of after every operation: an addition
+// add and multiply unnormalised pairs and renormalise each value when they
+// store it, and after three levels of additions at the latest where a stage
+// has more (settle), instead of after every operation: an addition
 // costs 8 FP32 operations instead of 11, a product 16 instead of 19.
 #pragma once
 
@@ -210,21 +211,6 @@ struct TwR<R, dfl> {
   static constexpr dfl c(int j) { return split(turn_cos_sin(8LL * j, 8LL * R).c); }
   static constexpr dfl s(int j) { return split(turn_cos_sin(8LL * j, 8LL * R).s); }
 };
-
-// Odd eighths of a turn, (+-1 +- i) / sqrt 2: two sums and two real products
-// (24 operations) instead of a complex product (32).
-template <int SIGN>
-__device__ __forceinline__ cpx<dfl> tw64_mul(cpx<dfl> z, int idx) {
-  idx &= 63;
-  if ((idx & 15) != 8) return tw64_mul<SIGN, dfl>(z, idx);
-  const dfl c = tw64c<dfl>(8);
-  // w = (re + i im) / sqrt 2 with re, im = +-1
-  const bool re = idx == 8 || idx == 56, im = (idx == 8 || idx == 24) == (SIGN > 0);
-  const dfl u = z.x + z.y, d = re == im ? z.x - z.y : z.y - z.x;
-  // re == im:  z w = re ((x - y) + i (x + y)) c;  else  im == -re:  re ((x + y) + i (y - x)) c
-  const cpx<dfl> p = re == im ? cpx<dfl>{d * c, u * c} : cpx<dfl>{u * c, d * c};
-  return re ? p : cpx<dfl>{-p.x, -p.y};
-}
 
 __device__ __forceinline__ cpx<dfl> ldgc(const cpx<dfl>* p) {
   const float4 v = __ldg(reinterpret_cast<const float4*>(p));

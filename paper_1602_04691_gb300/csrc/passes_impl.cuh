@@ -1893,7 +1893,8 @@ __global__ void __launch_bounds__(ZSmem<L, C, T>::NT, ZSmem<L, C, T>::MINB) k_zc
     __syncthreads();
     if (next < ntiles) zpipe_prefetch_rows<T, L, C, NT>(a, next, per_rhs, S, tid);
     dif_middle<L, C>(X, TW, tid, NT);
-    // last forward stage, spectrum and first inverse stage on the same r3 points
+    // last forward stage, spectrum and first inverse stage on the same r3
+    // points, renormalised before the product (it drops the product of the low parts)
     const int my = mirror_index(ky, L);
     constexpr int r3 = SRad<L>::r3;
     for (int g = tid; g < C * (L / r3); g += NT) {
@@ -1905,7 +1906,7 @@ __global__ void __launch_bounds__(ZSmem<L, C, T>::NT, ZSmem<L, C, T>::MINB) k_zc
       dif_last<L, C, -1>(X, blk, c, v);
 #pragma unroll
       for (int t = 0; t < r3; ++t)
-        v[t] = settle(cmul(v[t], ldgc(gp + (long long)mirror_index(k0 + (L / r3) * t, L) * a.H * a.H)));
+        v[t] = settle(cmul(settle(v[t]), ldgc(gp + (long long)mirror_index(k0 + (L / r3) * t, L) * a.H * a.H)));
       dft<r3, +1, false>(v);
 #pragma unroll
       for (int t = 0; t < r3; ++t) st_stage(X + ColTile<L, C>::idx(blk * r3 + t, c, 0), settle(v[t]));
