@@ -252,13 +252,87 @@ __device__ __forceinline__ void dft_radix2(cpx<T> (&a)[R]) {
 constexpr bool is_pow2(int v) { return (v & (v - 1)) == 0; }
 constexpr int pow2_part(int v) { return (v & 1) ? 1 : 2 * pow2_part(v / 2); }
 
+// cos/sin of 2 pi j / M, M divisible by 8, rounded from a double-double
+// evaluation (error-free sums and products of Knuth and Dekker): the angle
+// 2 pi j / M of a length that is no power of two is itself rounded, and with the
+// angle and the series in plain FP64 the values were up to two units off, the
+// cos of 2 pi / 3 among them.  For compile time only: a fused multiply-add would
+// spoil the error-free sums.
+struct DD {
+  double h, l;
+};
+constexpr DD dd_sum(double a, double b) {
+  const double s = a + b, bb = s - a;
+  return {s, (a - (s - bb)) + (b - bb)};
+}
+constexpr DD dd_prod(double a, double b) {
+  const double p = a * b, ca = 134217729.0 * a, cb = 134217729.0 * b;   // halves of 26 bits
+  const double ah = ca - (ca - a), bh = cb - (cb - b), al = a - ah, bl = b - bh;
+  return {p, ((ah * bh - p) + ah * bl + al * bh) + al * bl};
+}
+constexpr DD operator+(DD a, DD b) {
+  const DD s = dd_sum(a.h, b.h);
+  return dd_sum(s.h, s.l + (a.l + b.l));
+}
+constexpr DD operator*(DD a, DD b) {
+  const DD p = dd_prod(a.h, b.h);
+  return dd_sum(p.h, p.l + (a.h * b.l + a.l * b.h));
+}
+constexpr DD operator/(DD a, double n) {
+  const double q = a.h / n;
+  const DD p = dd_prod(q, n);
+  return dd_sum(q, ((a.h - p.h) - p.l + a.l) / n);
+}
+constexpr CosSin precise_cos_sin(long long j, long long M) {
+  const long long jm = ((j % M) + M) % M, m8 = M / 8, oct = jm / m8, rem = jm % m8;
+  const DD two_pi = {6.283185307179586, 2.4492935982947064e-16};
+  double c[2] = {0, 0}, s[2] = {0, 0};   // of rem and of m8 - rem, both in [0, pi/4]
+  for (int v = 0; v < 2; ++v) {
+    const DD x = two_pi * DD{double(v == 0 ? rem : m8 - rem), 0.0} / double(M), x2 = x * x;
+    DD tc = {1.0, 0.0}, ts = x, sc = tc, ss = x;
+    for (int i = 1; i < 15; ++i) {
+      tc = tc * x2 / double(-(2 * i - 1) * (2 * i));
+      ts = ts * x2 / double(-(2 * i) * (2 * i + 1));
+      sc = sc + tc;
+      ss = ss + ts;
+    }
+    c[v] = sc.h;
+    s[v] = ss.h;
+  }
+  switch (oct) {
+    case 0: return {c[0], s[0]};
+    case 1: return {s[1], c[1]};
+    case 2: return {-s[0], c[0]};
+    case 3: return {-c[1], s[1]};
+    case 4: return {-c[0], -s[0]};
+    case 5: return {-s[1], -c[1]};
+    case 6: return {s[0], -c[0]};
+    default: return {c[1], -s[1]};
+  }
+}
+
 // cos/sin of 2 pi j / R as a compile-time constant of type T (paired FP32
 // specialises it in dfloat.cuh).
 template <int R, class T>
 struct TwR {
-  static constexpr T c(int j) { return T(turn_cos_sin(8LL * j, 8LL * R).c); }
-  static constexpr T s(int j) { return T(turn_cos_sin(8LL * j, 8LL * R).s); }
+  static constexpr T c(int j) { return T(precise_cos_sin(8LL * j, 8LL * R).c); }
+  static constexpr T s(int j) { return T(precise_cos_sin(8LL * j, 8LL * R).s); }
 };
+
+template <int R>
+struct TwTab {
+  double c[R], s[R];
+};
+template <int R>
+constexpr TwTab<R> make_twtab() {
+  TwTab<R> t{};
+  for (int j = 0; j < R; ++j) {
+    const CosSin v = precise_cos_sin(8LL * j, 8LL * R);
+    t.c[j] = v.c;
+    t.s[j] = v.s;
+  }
+  return t;
+}
 
 // a + s t and m + SIGN i n (a quarter turn folded into the sums).
 template <class T>
@@ -315,7 +389,8 @@ __device__ __forceinline__ void dft(cpx<T> (&a)[R]);
 template <int R, int SIGN, class T>
 __device__ __forceinline__ cpx<T> twR_mul(cpx<T> z, int j) {
   if (j == 0) return z;
-  const T c = TwR<R, T>::c(j), s = TwR<R, T>::s(j);
+  constexpr TwTab<R> t = make_twtab<R>();
+  const T c = T(t.c[j]), s = T(t.s[j]);
   return cmul(z, cpx<T>{c, SIGN > 0 ? s : -s});
 }
 

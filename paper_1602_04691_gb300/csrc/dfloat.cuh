@@ -208,8 +208,8 @@ __device__ __forceinline__ dfl tw64s<dfl>(int i) { return {c_tw64df.sh[i], c_tw6
 template <int R>
 struct TwR<R, dfl> {
   static constexpr dfl split(double v) { return dfl{float(v), float(v - double(float(v)))}; }
-  static constexpr dfl c(int j) { return split(turn_cos_sin(8LL * j, 8LL * R).c); }
-  static constexpr dfl s(int j) { return split(turn_cos_sin(8LL * j, 8LL * R).s); }
+  static constexpr dfl c(int j) { return split(precise_cos_sin(8LL * j, 8LL * R).c); }
+  static constexpr dfl s(int j) { return split(precise_cos_sin(8LL * j, 8LL * R).s); }
 };
 
 __device__ __forceinline__ cpx<dfl> ldgc(const cpx<dfl>* p) {
