@@ -78,7 +78,8 @@ def peaks():
 
 # ---------------------------------------------------------------------------
 # Algorithmic bytes per launch of each pass (complex element = 8 B in FP32,
-# 16 B in FP64; N = n^3 cells; H = L/2 + 1).  COCG-mode prologue/epilogue.
+# 16 B in FP64; N = n^3 cells; L = the plan's transform length, H = L/2 + 1).
+# COCG-mode prologue/epilogue.
 # ---------------------------------------------------------------------------
 def alg_bytes(kind: str, n: int, L: int, cb: int) -> float:
     N = n ** 3
@@ -138,13 +139,25 @@ def split_L1(L: int) -> int:
     return 1 << ((lg + 1) // 2)
 
 
+# First-stage radix of the transform lengths between the powers of two (MixRad in the sources).
+MIXED_L1 = {144: 12, 200: 20, 288: 24, 400: 20, 576: 24, 800: 40}
+
+
 def fp32_kernel_name(kind: str, L: int, sched: dict) -> str:
-    """The FP32 kernel that runs a pass of the B-form matvec at padded length L
+    """The FP32 kernel that runs a pass of the B-form matvec at transform length L
     (L >= 64) under a launch schedule (1 = ORI_SCHED_TILES; *_variant: tile
-    width and radix split of the persistent Y and Z kernels at L = 256..1024)."""
+    width and radix split of the persistent Y and Z kernels at L = 256..1024;
+    lengths between the powers of two have one kernel a pass)."""
     tiles = {key: sched.get(key, 0) == 1 for key in ("yfwd", "zconv", "yinv")}
     if kind == "update":
         return "k_cocg_update<float>"
+    if L in MIXED_L1:
+        L1 = MIXED_L1[L]
+        L2 = L // L1
+        x = next(c for c in range(1, 65) if c * L2 % 32 == 0 and c * L2 >= 96)
+        y = 16 if L % 16 == 0 and L <= 400 else 8
+        return {"xfwd": f"k_xfwd_pipe<{L}, {x}>", "xinv": f"k_xinv_pipe<{L}, {x}>", "zconv": f"k_zconv_mix<{L}>",
+                "yfwd": f"k_yfwd_pipe<float, {L}, {y}, {L1}>", "yinv": f"k_yinv_pipe<{L}, {y}, {L1}>"}[kind]
     L1 = split_L1(L)
 
     def pipe(key):
@@ -436,7 +449,7 @@ def ours_arm(args, world, rank, local):
     t0 = time.perf_counter()
     plan = Plan(n, k, h_dev, N_dev, lean=args.lean)
     plan_s = time.perf_counter() - t0
-    L = plan.L
+    L = plan.transform_length
     if args.lean and args.no_e2e and (args.no_cufft or args.matvec_reps <= 0):
         # a lean plan keeps no reference to h and N, and no later leg reads them:
         # give their 24 bytes a cell back to the solver's vectors (n = 1000)
@@ -660,7 +673,7 @@ def ours_arm(args, world, rank, local):
         "clocks": ck,
         "solve": {"iters": last["iters"], "outer_iters": last["outer_iters"], "relres": last["relres"],
                   "fp64_matvecs": last["fp64_matvecs"], "status": last["status"]},
-        "plan_s": plan_s, "fp64_solve": fp64, "mixed_fp64_residual": mixed_native,
+        "transform_length": L, "plan_s": plan_s, "fp64_solve": fp64, "mixed_fp64_residual": mixed_native,
         "residual_arith": "paired FP32 (double-float) FFT passes, complex128 vectors",
         "matvec": matvec, "passes": passes,
         "schedule": tuned["schedule"], "schedule_operator_ms": tuned["ms"],
@@ -724,7 +737,7 @@ def cufft_comparator(plan, h_dev, N_dev, x32, y_ours, n, k, L, dev, reps=5):
     torch.cuda.empty_cache()
     return {"ms": ms, "speedup_of_ours": ms / max(1e-9, float(_last_ms[0])) if _last_ms else None,
             "rel_l2_vs_ours_of_K_part": diff,
-            "how": "torch.fft.fftn/ifftn (cuFFT C2C, complex64) on the zero-padded L^3 cube + elementwise pad, "
+            "how": f"torch.fft.fftn/ifftn (cuFFT C2C, complex64) on the zero-padded {L}^3 cube + elementwise pad, "
                    "spectrum multiply, crop and axpy"}
 
 

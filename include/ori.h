@@ -225,6 +225,10 @@ ori_status ori_plan_destroy(ori_plan_t plan);
 /* Grid size, padded length L (ori_plan), and bytes of device memory the plan holds. */
 ori_status ori_plan_info(ori_plan_t plan, int64_t* n, int64_t* L, size_t* bytes);
 
+/* *M = the length the plan's FFT passes transform at (ori_plan): L, or a
+ * shorter length between the powers of two. */
+ori_status ori_plan_transform_length(ori_plan_t plan, int64_t* M);
+
 /*
  * ori_matvec - y = A x or y = B x (form) for n^3 complex128 vectors.
  *   precision ORI_FP64: every pass in FP64.

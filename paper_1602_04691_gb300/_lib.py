@@ -39,7 +39,7 @@ EXPORTS = [
     "ori_plan_set_timing", "ori_plan_get_stats", "ori_plan_reset_stats", "ori_matvec_noalloc",
     "ori_cocg_solve_batch", "ori_plan_get_schedule", "ori_plan_set_schedule", "ori_plan_autotune",
     "ori_field", "ori_plan_spectrum_bytes", "ori_plan_save_spectrum", "ori_plan_from_spectrum",
-    "ori_plan_residual_history",
+    "ori_plan_residual_history", "ori_plan_transform_length",
 ]
 
 ORI_SCHED_PERSISTENT = 0
@@ -152,6 +152,8 @@ def load():
     lib.ori_plan_destroy.restype = i
     lib.ori_plan_info.argtypes = [vp, C.POINTER(i64), C.POINTER(i64), C.POINTER(C.c_size_t)]
     lib.ori_plan_info.restype = i
+    lib.ori_plan_transform_length.argtypes = [vp, C.POINTER(i64)]
+    lib.ori_plan_transform_length.restype = i
     lib.ori_matvec.argtypes = [vp, vp, vp, i, i, vp]
     lib.ori_matvec.restype = i
     lib.ori_matvec32.argtypes = [vp, vp, vp, i, vp]

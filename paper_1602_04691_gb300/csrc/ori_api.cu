@@ -1301,6 +1301,12 @@ ori_status ori_plan_info(ori_plan_t p, int64_t* n, int64_t* L, size_t* bytes) {
   return ORI_OK;
 }
 
+ori_status ori_plan_transform_length(ori_plan_t p, int64_t* M) {
+  if (!p || !M) return fail(ORI_ERR_INVALID_ARG, "NULL argument");
+  *M = p->M;
+  return ORI_OK;
+}
+
 ori_status ori_matvec(ori_plan_t p, const double* x_dev, double* y_dev, int form, int precision,
                       void* stream) {
   g_last_error.clear();

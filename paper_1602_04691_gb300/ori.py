@@ -147,6 +147,8 @@ class Plan:
         lib.ori_plan_info(self._h, C.byref(nn), C.byref(LL), C.byref(by))
         self.L = int(LL.value)
         self.bytes = int(by.value)
+        lib.ori_plan_transform_length(self._h, C.byref(LL))
+        self.transform_length = int(LL.value)   # of the FFT passes; L or a shorter length between the powers of two
         self.medium_version = 0   # counts set_medium calls (OriSolve checks it in backward)
 
     # -- lifetime ------------------------------------------------------------
