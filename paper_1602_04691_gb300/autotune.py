@@ -2,17 +2,20 @@
 
 The library times the candidate launch schedules of the FP32 passes on a
 plan; this module keeps the winners in a JSON file keyed by GPU name, grid
-size n, batch size and arithmetic, so that later plans for the same key take
+size n, batch size, arithmetic and transform length M (plans of one n differ in
+it with min_L or a saved spectrum), so that later plans for the same key take
 the cached schedule without timing anything.  The file maps
 
-    "<gpu name>|n=<n>|nrhs=<nrhs>|arith=fp32|sched=2"  ->  {"schedule": {...}, "ms": t}
+    "<gpu name>|n=<n>|nrhs=<nrhs>|arith=fp32|sched=2|M=<M>"  ->  {"schedule": {...}, "ms": t}
 
 where "schedule" holds the ori_schedule fields (kernel choice, launch variant
 (tile width and radix split) and CTA cap of the FP32 Y-forward, Z and
 Y-inverse passes, and the vector-kernel grid) and "ms" the FP32 operator time
 of the whole batch measured when the entry was written.  "sched" numbers the
 set of fields the tuner searches: entries written for an older set are tuned
-again.
+again.  So are entries without a length: they were timed on kernels that other
+lengths have replaced, and an old cap of one CTA per SM, free with the kernels
+of one CTA per SM it was found with, would hold back those that count on several.
 
 Cache location: the ``path`` argument, else the ORI_AUTOTUNE_CACHE
 environment variable, else ``~/.cache/ori_autotune.json``.
@@ -37,8 +40,9 @@ def cache_path(path: str | None = None) -> str:
     return os.path.join(os.path.expanduser("~"), ".cache", "ori_autotune.json")
 
 
-def cache_key(gpu_name: str, n: int, nrhs: int, arith: str = ARITH) -> str:
-    return f"{gpu_name}|n={int(n)}|nrhs={int(nrhs)}|arith={arith}|sched={SCHED_FIELDS_VERSION}"
+def cache_key(gpu_name: str, n: int, nrhs: int, arith: str = ARITH, transform_length: int | None = None) -> str:
+    key = f"{gpu_name}|n={int(n)}|nrhs={int(nrhs)}|arith={arith}|sched={SCHED_FIELDS_VERSION}"
+    return key if transform_length is None else f"{key}|M={int(transform_length)}"
 
 
 def load(path: str) -> dict:
@@ -77,11 +81,11 @@ def valid_schedule(s) -> bool:
 
 def tune(plan, nrhs: int, gpu_name: str, path: str | None = None, reps: int = 3,
          force: bool = False) -> dict:
-    """Give `plan` the schedule for (gpu_name, plan.n, nrhs): from the cache when
+    """Give `plan` the schedule for (gpu_name, plan.n, nrhs) and its transform length: from the cache when
     present (and `force` is false), else by timing on the plan and storing the
     result.  Returns {"schedule": ..., "ms": ..., "cached": bool, "key": ...}."""
     p = cache_path(path)
-    key = cache_key(gpu_name, plan.n, nrhs)
+    key = cache_key(gpu_name, plan.n, nrhs, transform_length=getattr(plan, "transform_length", None))
     if not force:
         entry = load(p).get(key)
         if isinstance(entry, dict) and valid_schedule(entry.get("schedule")):
