@@ -385,7 +385,8 @@ typedef struct {
                            have variant 0 only.  A plan whose transform length M
                            is not a power of two runs one persistent kernel per
                            pass whatever these fields say (zconv_variant 1: its
-                           rows by cp.async instead of TMA)                        */
+                           rows by cp.async instead of TMA), at ctas_per_sm CTAs
+                           per SM like the others                                  */
   int zconv_variant;
   int yinv_variant;
 } ori_schedule;
@@ -401,9 +402,10 @@ ori_status ori_plan_set_schedule(ori_plan_t plan, const ori_schedule* s);
  * ori_plan_autotune - time the candidate schedules on this plan for a batch of
  * nrhs systems (1..4096) and keep the fastest.  Starting from the plan's
  * schedule, each field in turn (Y-forward, Z and Y-inverse kernels, their
- * launch variants 1 and 2 where the length has them and the kernel is the
- * persistent one, then the persistent CTA cap 1 or 2) takes the alternative
- * that lowers the time of
+ * launch variants where the length has them and the kernel is the
+ * persistent one, then the persistent CTA cap 0, 1 or 2; at a transform length
+ * that is no power of two zconv_variant 0 or 1 and the cap) takes the value
+ * that gives the lowest time of
  * `reps` (1..100) FP32 operator applications y = B x on the plan's scratch
  * vectors (each timing after one warm-up); then the vector grid (4, 8 or 16
  * CTAs per SM) is timed on the FP32 COCG update.  Grows the plan's batch scratch to nrhs like
@@ -411,8 +413,8 @@ ori_status ori_plan_set_schedule(ori_plan_t plan, const ori_schedule* s);
  * spectra); leaves ori_plan_stats unchanged.  *best (may be NULL) receives the
  * chosen schedule, *best_ms (may be NULL) its operator time for the whole
  * batch in milliseconds.  Synchronising.  A cache of results keyed by GPU,
- * n, nrhs and arithmetic belongs to the caller (the Python binding keeps one
- * as JSON).
+ * n, nrhs, arithmetic and transform length belongs to the caller (the Python
+ * binding keeps one as JSON).
  */
 ori_status ori_plan_autotune(ori_plan_t plan, int nrhs, int reps, ori_schedule* best,
                              float* best_ms, void* stream);

@@ -2056,6 +2056,39 @@ static ori_status time_fp32_update(ori_plan_s* p, int nrhs, int reps, float* ms)
   return ORI_OK;
 }
 
+// The schedule search: one field at a time, every value it can take, keeping
+// the best before the next field.  Fields 0-2: kernel choice of Y forward, Z, Y
+// inverse; 3-5 their launch variants (nv of them; persistent kernels only); 6
+// the cap on persistent CTAs per SM.  The mixed lengths have one kernel a pass:
+// only the staging of the Z rows (zconv_variant) and the cap are left to choose.
+// *best is the start and *best_t its time.
+template <class Time>
+static ori_status search_schedule(ori_schedule* best, float* best_t, bool mixed, int nv, Time time) {
+  int ori_schedule::*const fields[7] = {&ori_schedule::yfwd,         &ori_schedule::zconv,         &ori_schedule::yinv,
+                                        &ori_schedule::yfwd_variant, &ori_schedule::zconv_variant, &ori_schedule::yinv_variant,
+                                        &ori_schedule::ctas_per_sm};
+  for (int i = 0; i < 7; ++i) {
+    const bool variant = i >= 3 && i < 6;
+    if (mixed && i != 4 && i != 6) continue;
+    if (!mixed && variant && best->*fields[i - 3] != ORI_SCHED_PERSISTENT) continue;
+    const int count = variant ? nv : (i < 3 ? 2 : 3);
+    const int first = best->*fields[i];   // timed already
+    for (int v = 0; v < count; ++v) {
+      if (v == first) continue;
+      ori_schedule s = *best;
+      s.*fields[i] = v;
+      float t = 0.f;
+      const ori_status st = time(s, &t);
+      if (st != ORI_OK) return st;
+      if (t < *best_t) {
+        *best_t = t;
+        *best = s;
+      }
+    }
+  }
+  return ORI_OK;
+}
+
 static ori_status autotune(ori_plan_s* p, int nrhs, int reps, ori_schedule* best_out, float* best_ms) {
   NvtxRange nvtx("ori autotune");
   ORI_TRY(ensure_capacity(p, nrhs));
@@ -2064,39 +2097,14 @@ static ori_status autotune(ori_plan_s* p, int nrhs, int reps, ori_schedule* best
     ORI_CUDA(cudaMemsetAsync(v, 0, n3 * sizeof(cpx<float>), p->ps));
   ori_schedule best = current_schedule(p);
   float best_t = 0.f;
-  // FFT pass schedules (only the FP32 passes at L >= 64 have alternatives):
-  // one field at a time, keeping the best value of each before the next
+  // only the FP32 passes at 64 to 1024 points have alternatives
+  const bool mixed = is_mixed_len(p->M);
   ORI_TRY(time_fp32_operator(p, nrhs, reps, &best_t));
-  if (p->M >= 64 && p->M <= 1024 && !is_mixed_len(p->M)) {   // longer and mixed transforms have one schedule
-    const int nv = pipe_variants(p->L);
-    // fields: 0-2 kernel choice of Y fwd, Z, Y inv; 3-5 their launch variants
-    // (persistent kernels only); 6 the persistent CTA cap
-    for (int field = 0; field < 7; ++field) {
-      const bool var_field = field >= 3 && field < 6;
-      if (var_field) {
-        const int sched = field == 3 ? best.yfwd : field == 4 ? best.zconv : best.yinv;
-        if (sched != SCHED_PERSISTENT || nv < 2) continue;
-      }
-      const int nval = field < 3 ? 1 : (var_field ? nv - 1 : 2);
-      for (int vi = 0; vi < nval; ++vi) {
-        ori_schedule s = best;
-        int* f = field == 0 ? &s.yfwd : field == 1 ? &s.zconv : field == 2 ? &s.yinv
-               : field == 3 ? &s.yfwd_variant : field == 4 ? &s.zconv_variant : field == 5 ? &s.yinv_variant
-               : &s.ctas_per_sm;
-        const int value = field < 3 ? SCHED_TILES : (var_field ? (vi + 1 == *f ? 0 : vi + 1) : vi + 1);
-        if (value == *f) continue;
-        *f = value;
-        apply_schedule(p, s);
-        float t = 0.f;
-        ORI_TRY(time_fp32_operator(p, nrhs, reps, &t));
-        if (t < best_t) {
-          best_t = t;
-          best = s;
-        }
-        apply_schedule(p, best);
-      }
-    }
-  }
+  if (p->M >= 64 && p->M <= 1024)
+    ORI_TRY(search_schedule(&best, &best_t, mixed, mixed ? 2 : pipe_variants(p->M), [&](const ori_schedule& sc, float* t) {
+      apply_schedule(p, sc);
+      return time_fp32_operator(p, nrhs, reps, t);
+    }));
   apply_schedule(p, best);
   // vector-kernel grid
   float best_v = 0.f;
