@@ -201,8 +201,9 @@ ori_status ori_plan(int64_t n, double k, const ori_domain* dom,
  *   Synchronises `stream`.
  * ori_plan_from_spectrum - as ori_plan, but the spectra come from a saved form
  *   instead of being computed: n, c_S (opts->c_S) and side (dom->side) must
- *   equal the saved ones, the saved length must be this plan's M or its L
- *   (with opts->min_L; the plan then transforms at the saved length), and the
+ *   equal the saved ones, the saved length must be this plan's L (with
+ *   opts->min_L) or, unless min_L is above the power of two, the M of a plan
+ *   of this n (the plan then transforms at the saved length), and the
  *   wave numbers are the saved ones (k, opts->n_k and opts->ks are ignored).  A mismatch, or a
  *   buffer that is too short or not a saved spectrum, returns
  *   ORI_ERR_INVALID_ARG.  Synchronises `stream`.

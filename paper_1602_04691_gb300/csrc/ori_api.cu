@@ -1027,9 +1027,10 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
       return fail(ORI_ERR_INVALID_ARG, "saved spectrum: not a saved spectrum of this format");
     int Lw = 4;
     while (Lw < 2 * n) Lw *= 2;
-    // saved at this plan's transform length, or at the power of two: the
-    // plan then runs at that length
-    const int Mw = o.min_L ? std::max(Lw, o.min_L) : transform_length(int(n), Lw);
+    // saved at the transform length of this n, or at the power of two: the
+    // plan then runs at that length; a min_L above the power of two asks for
+    // that length alone
+    const int Mw = o.min_L > Lw ? o.min_L : transform_length(int(n), Lw);
     Lw = std::max(Lw, o.min_L);
     if (hd.n != n || (hd.L != Lw && hd.L != Mw))
       return fail(ORI_ERR_INVALID_ARG, "saved spectrum: n or padded length L differs from this plan's");
