@@ -528,10 +528,15 @@ static bool z_bulk_staged(const ori_plan_s* p) {
   return !(has_pipe_variants(L) && p->var_z == 1);
 }
 
-// The tensor map of the FP32 Z pass's input T2f, [rhs][ky / B][z][ky % B][kx]
-// with dims (kx: L, ky % B: B, (ky / B) n + z: n L / B, rhs: R), 8-byte elements, boxes of
-// 16 x 1 x zbox x 1 (128-byte rows; zbox = min(L / 2, 256), so that the boxes
-// covering z < n end within the tile's L / 2 + 1 staged rows).  Encoded when
+// The tensor map of the FP32 Z pass's input T2f, [rhs][ky / B][z][ky % B][kx]:
+// dims (kx: L, ky % B: B, z: n, ky / B: L / B, rhs: R), 8-byte elements, boxes of
+// w x 1 x zbox rows (w = 16, 128-byte rows, zbox = min(L / 2, 256); or a group's
+// columns and even_box(L / 2)), so that the boxes covering z < n end within the
+// tile's L / 2 + 1 staged rows.  z is a dimension of its own, so the rows of a
+// box past n are zero-filled; with (ky / B) n + z in one they were the next
+// block's rows, read and not used (n = 300, 800 points: a third more than the
+// tile's own).  Where T2 is in plain order (B = L) the ky / B dimension goes.
+// Encoded when
 // T2f or the batch size changes; without an encoder, an aligned base or a
 // length the kernel stages by bulk copies, the kernel keeps cp.async.
 static void z_tensor_map(ori_plan_s* p, SArgs& z, int nrhs) {
@@ -543,23 +548,28 @@ static void z_tensor_map(ori_plan_s* p, SArgs& z, int nrhs) {
     p->zmap_ptr = p->T2f;
     p->zmap_R = R;
     p->zmap_w = w;
-    const int L = p->M;
+    const int L = p->M, n = p->n;
     const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (enc != nullptr && L >= 64 && L <= 1024 && (reinterpret_cast<uintptr_t>(p->T2f) & 15u) == 0) {
       const cuuint64_t es = sizeof(cpx<float>);
-      const cuuint64_t B = cuuint64_t(yblk(L));
-      const cuuint64_t dims[4] = {cuuint64_t(L), B, cuuint64_t(p->n) * (L / B), cuuint64_t(R)};
-      const cuuint64_t strides[3] = {cuuint64_t(L) * es, B * L * es, cuuint64_t(t2_elems(p)) * es};
+      const int B = yblk(L);
+      const cuuint64_t row = cuuint64_t(B) * L * es, rhs = cuuint64_t(t2_elems(p)) * es;
+      const cuuint64_t dims_b[5] = {cuuint64_t(L), cuuint64_t(B), cuuint64_t(n), cuuint64_t(L / B), cuuint64_t(R)};
+      const cuuint64_t str_b[4] = {cuuint64_t(L) * es, row, cuuint64_t(n) * row, rhs};
+      const cuuint64_t dims_p[4] = {cuuint64_t(L), cuuint64_t(L), cuuint64_t(n), cuuint64_t(R)};
+      const cuuint64_t str_p[3] = {cuuint64_t(L) * es, row, rhs};
       const int zbox = std::min(L / 2, 256);
+      const int rows = w == kZGroup ? zbox : even_box(L / 2);
       const cuuint32_t box[4] = {cuuint32_t(kZGroup), 1, cuuint32_t(zbox), 1};
-      const cuuint32_t gbox[4] = {cuuint32_t(w), 1, cuuint32_t(even_box(L / 2)), 1};
-      const cuuint32_t estr[4] = {1, 1, 1, 1};
-      if (enc(&p->zmap, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, p->T2f, dims, strides,
-              w == kZGroup ? box : gbox, estr,
+      const cuuint32_t box_b[5] = {cuuint32_t(w), 1, cuuint32_t(rows), 1, 1};
+      const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+      const bool plain = B == L;
+      if (enc(&p->zmap, CU_TENSOR_MAP_DATA_TYPE_UINT64, plain ? 4 : 5, p->T2f, plain ? dims_p : dims_b,
+              plain ? str_p : str_b, plain && w == kZGroup ? box : box_b, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS) {
         p->zmap_ok = 1;
-        p->zbox = w == kZGroup ? zbox : even_box(L / 2);
+        p->zbox = rows;
       }
     }
   }

@@ -137,8 +137,8 @@ struct SArgs {
   int variant;                     // pipelined FP32 kernels: launch variant (has_pipe_variants)
   // FP32 Z and Y passes with 16-column tiles: the input rows of a tile
   // arrive by TMA (cp.async.bulk.tensor) through this map of the input cube:
-  // Z pass, dims (kx, ky % B, (ky / B) n + z, right-hand side) of T2 and box
-  // (16, 1, zbox, 1); Y forward, dims (kx, y, z, right-hand side) of T1 and box
+  // Z pass, dims (kx, ky % B, z, ky / B, right-hand side) of T2 and box
+  // (16, 1, zbox, 1, 1); Y forward, dims (kx, y, z, right-hand side) of T1 and box
   // (16, zbox, 1, 1); Y inverse, dims (kx, ky % B, ky / B, z, right-hand side)
   // of T2 and box (16, B, zbox / B, 1, 1); zrows_ok = 0 keeps cp.async
   CUtensorMap zrows;

@@ -1297,7 +1297,7 @@ struct ZPipe {
 // Bulk-copy staging of the FP32 Z pass (ZPipe::TMA).  Thread 0 issues the
 // copies; every thread waits on the barrier.  The n_in input rows of a tile,
 // 128 bytes each, come as ceil(n_in / zbox) boxes of zbox rows through the
-// tensor map a.zrows (rows past n_in are not used; zbox divides L / 2, so the
+// tensor map a.zrows (rows past n_in are zero-filled; zbox divides L / 2, so the
 // boxes end within the L / 2 + 1 rows of S).
 template <int L, int C>
 __device__ __forceinline__ void zpipe_tma_rows(const SArgs& a, int tile, int per_rhs, cpx<float>* S,
@@ -1312,10 +1312,10 @@ __device__ __forceinline__ void zpipe_tma_rows(const SArgs& a, int tile, int per
   mbar_expect_tx(bar, unsigned(nbox * a.zbox * C * int(sizeof(cpx<float>))));
   if constexpr (yblk(L) == L) {
     for (int q = 0; q < nbox; ++q) tma_load_4d(S + q * a.zbox * C, &a.zrows, cb * C, ky, q * a.zbox, rhs, bar);
-  } else {   // rows past n_in belong to the next block of ky (or are zero-filled): staged, not used
-    const int kb = ky / yblk(L), z0 = kb * a.n_in;
+  } else {
+    const int kb = ky / yblk(L);
     for (int q = 0; q < nbox; ++q)
-      tma_load_4d(S + q * a.zbox * C, &a.zrows, cb * C, ky - kb * yblk(L), z0 + q * a.zbox, rhs, bar);
+      tma_load_5d(S + q * a.zbox * C, &a.zrows, cb * C, ky - kb * yblk(L), q * a.zbox, kb, rhs, bar);
   }
 }
 // The spectrum slice of a tile: the L / 2 + 1 rows of its columns are C / W
