@@ -816,6 +816,9 @@ static ori_status set_medium(ori_plan_s* p, const double* h_dev, const double* N
 // and keeps kz < H in the same way, in place.  FP64 throughout; the octant is stored in FP64, FP32 and
 // paired FP32 with c_S |Delta| / L^3 folded in, plus the Z-tile-ordered FP32
 // copy.
+static bool spectrum_fits_scratch(const ori_plan_s* p) {
+  return t2_elems(p) >= size_t(p->H) * p->H * p->H + size_t(p->M) * p->H;   // the octant and one plane
+}
 static ori_status build_spectrum(ori_plan_s* p) {
   NvtxRange nvtx("ori plan spectrum");
   const int L = p->M, n = p->n, H = p->H;
@@ -825,7 +828,8 @@ static ori_status build_spectrum(ori_plan_s* p) {
   const long long plane = (long long)L * H;   // a plane's lines y = 0..H-1
   int nz = int(std::max<long long>(1, std::min<long long>(H, (1LL << 26) / plane)));   // <= 1 GiB per batch
   // The octant and the planes live in the pass scratch (T2, idle until the
-  // first operator), in transient memory where min_L makes them larger.
+  // first operator), in transient memory where min_L makes them larger
+  // (spectrum_fits_scratch; there is no scratch yet then).
   cpx<double>* oct = p->T2d;
   cpx<double>* own = nullptr;
   const long long room = (long long)t2_elems(p) * p->cap;
@@ -1167,8 +1171,11 @@ static ori_status plan_create(int64_t n, double k, const ori_domain* dom, const 
       if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) { st = fail(ORI_ERR_CUDA, "twiddle upload failed"); break; }
     }
     if ((st = set_medium(p, h_dev, N_dev))) break;
-    if ((st = ensure_capacity(p, 1))) break;   // before the spectrum build, which uses its cubes
+    // the pass scratch comes before the spectrum where the build can work in it,
+    // else after it, so that the build's own memory is free again by then
+    if (spectrum_fits_scratch(p) && (st = ensure_capacity(p, 1))) break;
     if ((st = spec ? load_spectrum(p, static_cast<const unsigned char*>(spec)) : build_spectrum(p))) break;
+    if ((st = ensure_capacity(p, 1))) break;
     if ((st = io.leave())) break;
   } while (0);
   if (st != ORI_OK) {
