@@ -1413,7 +1413,7 @@ __device__ __forceinline__ void zpipe_prefetch_ghat(const SArgs& a, int rhs, int
 // 50% busy, the sum of their times); groups out of phase overlap them (67% and
 // 68%).  Tile by tile it is k_zconv_pipe's two stages; the column pitch of the
 // exchange spreads the columns and rows of a half warp over 16 different 8-byte
-// banks (2 modulo 4 for 8 columns, 4 modulo 8 for 4), and the twiddle table is
+// banks (2 modulo 4), and the twiddle table is
 // padded to L2 + 1 entries a row for the same reason (a square split reads it
 // by its symmetry instead).  The spectrum is grouped by C columns (zgroup), so
 // a tile's slice is one contiguous run.
@@ -1428,8 +1428,7 @@ struct ZGroups {
   static constexpr int L1 = Split<L>::L1, L2 = Split<L>::L2;
   static constexpr int NT = C * L2, NI = L1 / L2;                     // threads of a group
   static constexpr int PK = L2 + 1, PKI = L1 + 1;
-  static constexpr int MOD = C == 8 ? 4 : 8, REM = MOD / 2;
-  static constexpr int pitch(int v) { return v + ((REM - v % MOD) + MOD) % MOD; }
+  static constexpr int pitch(int v) { return v + (6 - v % 4) % 4; }   // 2 modulo 4
   static constexpr int PC = pitch(L1 * PK), PCI = pitch(L2 * PKI);
   static constexpr int PT = L1 == L2 ? L2 : L2 + 1;
   static constexpr int r16(int v) { return (v + 15) / 16 * 16; }      // regions start on 128 bytes
@@ -1470,7 +1469,8 @@ __device__ __forceinline__ void zconv_groups(const SArgs& a) {
   constexpr int L1 = Z::L1, L2 = Z::L2, NT = Z::NT, NI = Z::NI;
   constexpr int PK = Z::PK, PC = Z::PC, PKI = Z::PKI, PCI = Z::PCI, PT = Z::PT;
   constexpr int kSlice = (L / 2 + 1) * C;
-  static_assert(C == zgroup(L) && (G == 1 || NT % 32 == 0), "one run of the spectrum per tile; whole warps");
+  static_assert(C == zgroup(L) && C == 8 && (G == 1 || NT % 32 == 0),
+                "one run of the spectrum per tile; the pitches are for 8 columns; whole warps");
   extern __shared__ __align__(128) unsigned char smraw[];
   unsigned char* base = smraw + ((128u - (smem_addr(smraw) & 127u)) & 127u);
   const int g = G == 1 ? 0 : int(threadIdx.x) / NT;
