@@ -148,7 +148,8 @@ __device__ __forceinline__ void dif_last(const cpx<T>* X, int blk, int c, cpx<T>
 // the few CTAs that shared memory lets on an SM, the warps they make count too:
 // W of them hide latency like W / (W + 12) (paired-FP32 Z pass at n = 200, 400
 // points: 1.69 ms with two CTAs of 160 threads and the least waste, 1.54 with
-// two of 224; at n = 400 12.2 ms with 320 threads, 11.8 with 416).
+// two of 224; at n = 400 12.2 ms with 320 threads, 11.8 with 416; both before
+// the renormalisations inside the stages, with which they are 1.61 and 12.7).
 template <int L>
 constexpr int stage_threads(int C, int most, int ctas = 0) {
   int best = most;

@@ -116,7 +116,7 @@ struct SArgs {
   int nouter;
   const void* twL;
   const void* ghat;                // spectrum, H^3 entries (SMODE_ZCONV)
-  const void* ghatZ;               // FP32 spectrum in Z-tile order [my][kx/kZGroup][mz][kZGroup]
+  const void* ghatZ;               // FP32 spectrum in Z-tile order [my][kx/W][mz][W], W = zgroup(L)
   int H;                           // L/2 + 1
   const int* done;
   int sm_count;                    // persistent kernels: CTAs to launch
@@ -149,7 +149,7 @@ struct SArgs {
 
 enum { SCHED_PERSISTENT = 0, SCHED_TILES = 1 };
 
-// Columns per group of the Z-tile-ordered FP32 spectrum [my][kx / kZGroup][mz][kZGroup].
+// Columns per group of the Z-tile-ordered FP32 spectrum [my][kx / W][mz][W]: W = kZGroup,
 constexpr int kZGroup = 16;
 // ... at transform length L, where the Z pass works in groups of fewer columns
 // (zconv_groups): their number.
@@ -226,7 +226,8 @@ constexpr int even_box(int rows) {
 // 3.92 without, 3.93 with plain launches; n = 128: 0.112, 0.103 and 0.118 ms).
 // FP32 operator (five passes) at n = 100: 79.9 -> 66.7 us; FP64 operator at
 // n = 12: 44.0 -> 34.4 us; mixed solve at n = 20: 0.83 -> 0.72 ms, and with the
-// solver's vector and control kernels launched the same way 0.68 -> 0.65 ms.
+// solver's vector and control kernels launched the same way 0.73 -> 0.68 ms
+// (n = 40: 1.01 -> 0.94; three runs of each side in turn, within 0.002).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... P, class... A>

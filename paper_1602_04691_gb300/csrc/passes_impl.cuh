@@ -1408,16 +1408,22 @@ __device__ __forceinline__ void zpipe_prefetch_ghat(const SArgs& a, int rhs, int
 // ---------------------------------------------------------------------------
 // FP32 Z convolution in groups of C columns that do not wait for one another:
 // the G groups of a CTA share the twiddle table and nothing else, each with its
-// own exchange buffer, staging buffer, barriers and tiles.  With the whole CTA
-// in step the FMA pipe and the shared-memory pipe of an SM took turns (59% and
-// 50% busy, the sum of their times); groups out of phase overlap them (67% and
-// 68%).  Tile by tile it is k_zconv_pipe's two stages; the column pitch of the
+// own exchange buffer, staging buffer, barriers and tiles.  Narrow tiles are
+// worth it with T2 in blocks of ky (passes.cuh): in a stand-alone build of the
+// pass at n = 512, 16 columns in step took 3.25 ms on plain T2 and 3.17 on the
+// blocked one, two groups of 8 3.41 and 2.84.  What the groups do not do is
+// keep the pipes busier: FMA 58.5% of the active cycles and shared memory 48.0%
+// of all against 57.7 and 47.6 in step, fewer waits for the pipes (math
+// throttle 1.61 against 1.91 warps an issue, memory-instruction throttle 0.67
+// against 1.03), and on a grid of few rows, where the addresses cost little,
+// no gain (n = 130 at 1024 points 3.12 ms, in step on plain T2 3.01).
+// Tile by tile it is k_zconv_pipe's two stages; the column pitch of the
 // exchange spreads the columns and rows of a half warp over 16 different 8-byte
 // banks (2 modulo 4), and the twiddle table is
 // padded to L2 + 1 entries a row for the same reason (a square split reads it
 // by its symmetry instead).  The spectrum is grouped by C columns (zgroup), so
 // a tile's slice is one contiguous run.
-//   L = 1024, 2 groups of 8: n = 512 3.18 -> 2.94 ms
+//   L = 1024, 2 groups of 8: n = 512 3.18 -> 2.94 ms, n = 400 3.15 -> 2.89
 //   mixed lengths, 1 group of 8 and several CTAs per SM: n = 260 (576 points) 0.55 ms,
 //   where the 1024-point pass on the same grid takes 3.06 ms
 // At L = 512 two 16-column CTAs in step each are faster (n = 256: 0.362 ms,
@@ -1829,7 +1835,7 @@ cudaError_t launch_zconv_mix_L(SArgs a, cudaStream_t s, bool setup, int sm_count
 // place in three stages (dfft.cuh), the last forward one, the spectrum product
 // and the first inverse one in one sweep; the next tile's input rows stream
 // into a staging buffer with cp.async meanwhile.  Bound by the paired
-// arithmetic (FMA pipe 63%, 2.5 to 4 warps a scheduler): n = 512 25.9 -> 20.2 ms
+// arithmetic (FMA pipe 63%, 2.5 to 4 warps a scheduler): n = 512 26.1 -> 20.7 ms
 // with the fused stages.
 // ---------------------------------------------------------------------------
 template <int L, int C, class T>
@@ -2388,7 +2394,7 @@ cudaError_t launch_yinv_pipe_L(SArgs a, cudaStream_t s, bool setup, int sm_count
   return dispatch_pipe_variant<float, L, C, YinvPipeLaunch>(a, s, setup, sm_count);
 }
 
-// Z-pass kernel choice for L >= 64: the shared-memory radix-8 kernel for
+// Z-pass kernel choice for L >= 64: the shared-memory kernel for
 // paired FP32; for FP32 the pipelined persistent kernel or, by schedule, the
 // one-CTA-per-tile strided kernel; the pipelined kernel for FP64; the plain
 // strided kernel for small L.
@@ -2412,7 +2418,7 @@ cudaError_t launch_zconv_reg_L(SArgs a, cudaStream_t s, bool setup) {
 }
 
 // Lengths beyond kMaxRegL: the FP64 and paired-FP32 passes use the
-// shared-memory radix-8 kernels (a register tile of L1 = 64 of their points
+// shared-memory kernels (a register tile of L1 = 64 of their points
 // per thread does not fit).  The FP32 passes stay pipelined: each 64-point
 // stage either has a zero-padded half on input or keeps half its outputs.
 constexpr int kMaxRegL = 1024;
@@ -2540,7 +2546,7 @@ cudaError_t launch_strided_L(SArgs a, cudaStream_t s, bool setup) {
     } else {
       // FP32 Y passes: the pipelined kernels fit for the reason the Z kernel does
       // (a 64-point stage with a zero half on input, or with half its outputs
-      // kept); the TILES schedule keeps the radix-8 kernels below
+      // kept); the TILES schedule keeps the shared-memory kernels below
       if constexpr (std::is_same<T, float>::value && SMODE == SMODE_FWD && HALF) {
         if (setup) {
           cudaError_t e = launch_yfwd_pipe_L<T, L>(a, s, true, a.sm_count);
@@ -2572,7 +2578,7 @@ cudaError_t launch_strided_L(SArgs a, cudaStream_t s, bool setup) {
 // The Z pass beyond kMaxRegL: for FP32 the pipelined kernel still fits, since
 // its first stage holds 32 nonzero inputs of the 64-point DFT (dft<64> with
 // the zero-padded half) and its last keeps 32 of 64 outputs; it reads the
-// Z-tile-ordered spectrum.  The radix-8 shared-memory kernel is the TILES
+// Z-tile-ordered spectrum.  The shared-memory kernel is the TILES
 // schedule and the kernel of the other arithmetics.
 template <class T, int L>
 cudaError_t launch_zconv_L(SArgs a, cudaStream_t s, bool setup) {
