@@ -155,6 +155,7 @@ struct ori_plan_s {
   cudaStream_t ps = nullptr;       // private stream (capturable)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, evj = nullptr;
   cudaEvent_t evl = nullptr;       // end of the plan's last asynchronous work, on whatever stream it ran
+  bool last_direct = false;        // it ran on a caller's stream
   // captured COCG blocks (FP32 and FP64 inner solvers)
   cudaGraphExec_t graph_f = nullptr, graph_d = nullptr;
   int graph_f_len = 0, graph_d_len = 0, graph_f_nrhs = 0, graph_d_nrhs = 0;
@@ -448,6 +449,7 @@ static bool capturing(cudaStream_t st) {
 struct Handoff {
   ori_plan_s* p = nullptr;
   cudaStream_t user = nullptr, run = nullptr;
+  bool cap = false;   // the caller's stream is being captured
 
   Handoff() = default;
   Handoff(const Handoff&) = delete;
@@ -456,7 +458,7 @@ struct Handoff {
     if (p != nullptr && close() != cudaSuccess) cudaGetLastError();   // the call's own error is the one reported
   }
   ori_status enter(ori_plan_s* plan, cudaStream_t stream, bool direct = false) {
-    const bool cap = capturing(stream);
+    cap = capturing(stream);
     user = stream;
     run = direct && !cap ? stream : plan->ps;
     if (run != user) {
@@ -464,7 +466,11 @@ struct Handoff {
       ORI_CUDA(cudaStreamWaitEvent(run, plan->evj, 0));
     }
     p = plan;
-    if (!cap) ORI_CUDA(cudaStreamWaitEvent(run, p->evl, 0));
+    if (cap) return ORI_OK;
+    // after a call on the private stream the next one there follows by itself
+    const bool wait = run != p->ps || p->last_direct;
+    p->last_direct = run != p->ps;
+    if (wait) ORI_CUDA(cudaStreamWaitEvent(run, p->evl, 0));
     return ORI_OK;
   }
   ori_status leave() {
@@ -474,7 +480,7 @@ struct Handoff {
 
  private:
   cudaError_t close() {
-    const cudaEvent_t done = capturing(user) ? p->evj : p->evl;
+    const cudaEvent_t done = cap ? p->evj : p->evl;
     cudaError_t e = cudaEventRecord(done, run);
     if (e == cudaSuccess && run != user) e = cudaStreamWaitEvent(user, done, 0);
     p = nullptr;
