@@ -347,10 +347,11 @@ __device__ __forceinline__ cpx<T> add_i(cpx<T> m, cpx<T> n) {
 // P-point transforms in dft_pfa and those of the first radix-4 stage of a
 // 16-point transform: a pair then goes through no more additions between two
 // renormalisations than in a radix-8 stage.  Error against 64 bits of a
-// convolution alone, root mean square of four media, without and with them:
-// 10.2 and 8.8e-15 at n = 260, 11.0 and 9.9 at n = 280; powers of two 8.3 to
-// 10.5.  Cost: operator at n = 144 0.89 -> 0.95 ms, n = 200 2.80 -> 2.94,
-// n = 400 22.3 both.
+// convolution alone, root mean square of 24 media, without and with them: 10.0
+// and 9.1e-15 at n = 72, 10.2 and 9.4 at n = 144, 10.2 and 9.6 at n = 200, 10.4
+// and 9.4 at n = 280.  (It falls with the padding: at 256 points 6.5 at n = 68,
+// 7.8 at n = 100, 9.5 at n = 128.)  Cost: operator at n = 144 0.89 -> 0.95 ms,
+// n = 200 2.80 -> 2.94, n = 400 22.3 both.
 template <int SIGN, class T>
 __device__ __forceinline__ void dft3(cpx<T>& a, cpx<T>& b, cpx<T>& c) {
   constexpr T half = TwR<3, T>::c(1), sn = TwR<3, T>::s(1);   // cos = -1/2
